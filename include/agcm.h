@@ -23,12 +23,13 @@
  *  - Streams: `stream` is a cudaStream_t passed as void* (NULL = default
  *    stream).  Calls that take a stream are asynchronous on it unless stated.
  *    A state also owns five internal streams, created with stream
- *    priorities (the launches with the longest blocks highest): each stage
- *    of agcm_step, agcm_step_split, agcm_tendency and agcm_step_adjoint forks
- *    some of its launches onto them after the work already queued on
- *    `stream` and joins them back before `stream` continues, so ordering on
- *    `stream` (and capture of `stream` into a CUDA graph) is as for one
- *    launch.
+ *    priorities: a stage of a small grid, and the products of
+ *    agcm_step_adjoint, fork some of their launches onto them after the work
+ *    already queued on `stream` and join them back before `stream` continues,
+ *    so ordering on `stream` (and capture of `stream` into a CUDA graph) is as
+ *    for one launch.  A stage that is one launch is a programmatic dependent
+ *    of the launch before it: its blocks may start while that one ends, but
+ *    touch nothing it reads or writes until it has completed.
  *  - Errors: every call returns AGCM_OK (0) or a negative-free positive code
  *    below; agcm_last_error() returns a message for the calling thread.  The
  *    library never aborts the process and never traps on the device.
@@ -249,10 +250,10 @@ int agcm_diagnostics(const agcm_state_t* state, agcm_diag_t* out, void* stream);
  * agcm_profile_read synchronises the recorded events and returns, per kernel
  * id 0..agcm_kernel_count()-1, the summed milliseconds and the launch count.
  * The events bracket a whole stage of the stage kernel, which is one launch
- * or several concurrent ones (the row-segment kernel once per stride class,
- * the column kernel for the rows next to the poles; or the column kernel's
- * stride-1 row band and the other rows): its milliseconds are per stage, its
- * count is of launches.
+ * or, on grids of fewer than 4096 columns, several concurrent ones (the
+ * row-segment kernel once per stride class; or the column kernel's stride-1
+ * row band and the other rows): its milliseconds are per stage, its count is
+ * of launches.
  * ms_total and launches hold at least agcm_kernel_count() entries.
  */
 int agcm_profile_enable(agcm_state_t* state, int enable);
@@ -261,13 +262,12 @@ int agcm_profile_enable(agcm_state_t* state, int enable);
  * kernel runs the steps, tendencies and adjoint recomputes of every state
  * (process-wide; results agree to rounding, both match the oracle).
  *   0 (default): the row-segment kernel (whole latitude-row segments staged in
- *     shared memory) when the grid's rows are 16-byte aligned (nlon % 4 == 0)
- *     and its row segments make at least two waves of CTAs on the GPU, else
- *     the column kernel (one thread per column, stencil read through L1);
+ *     shared memory) on grids of at least 4096 columns, else the column kernel
+ *     (one thread per column, stencil read through L1);
  *   1: always the column kernel;
- *   2: the row-segment kernel wherever the rows allow it, on any grid size.
- * Rows whose leap stride exceeds 63 (next to the poles on fine grids) always
- * run the column kernel.  Other values return AGCM_EINVAL.  Host only.
+ *   2: the row-segment kernel on any grid size.
+ * Rows whose leap stride exceeds 31 (next to the poles on fine grids) always
+ * run the column kernel's code.  Other values return AGCM_EINVAL.  Host only.
  */
 int agcm_set_stage_kernel(int choice);
 /*
@@ -300,9 +300,9 @@ const char* agcm_kernel_name(int id);
  * CUDA graph once a first call has uploaded the dt values (nsteps = 0 only
  * prepares: it uploads dt and the members' vertical means without stepping).
  * agcm_ensemble_configure sets the launch shape: warps per block 1 (one-warp
- * blocks running the column body on items of 32 columns) or 8 (256-thread
- * blocks running the row-segment body on (member, row segment) items, the
- * rows it leaves on the column body), and blocks per SM (0 = as many as
+ * blocks running the column body on items of 32 columns) or 8 (blocks of the
+ * row-segment kernel's shape running its body on (member, row segment) items,
+ * the rows it leaves on the column body), and blocks per SM (0 = as many as
  * fit); agcm_ensemble_tile sets the row tile of a one-warp work item (1, 2 or
  * 4 consecutive rows of 32 columns, taken by one warp in order); an
  * autotuner picks among them (ensemble.py).  Set both before capturing

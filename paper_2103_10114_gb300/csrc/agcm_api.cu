@@ -57,24 +57,14 @@ std::atomic<uint64_t> g_grid_uid{0};
 // 2 = row-segment kernel wherever the rows allow it.
 std::atomic<int> g_stage_choice{0};
 
-// Whether `items` row-segment CTAs make at least two waves on the current
-// device (three resident CTAs per SM); smaller grids run the column kernel,
-// whose one-warp blocks give more parallelism (measured on GB300: 720x360
-// rows, 2.3 waves, 0.165 against 0.185 ms per FP32 stage; 256x128, half a
-// wave, 0.072 against 0.043 ms).
-inline int rows_fill_device(long long items) {
-  int dev = 0, nsm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return items >= 2LL * 3 * nsm ? 1 : 0;
-}
-
 // Guards every grid's lazily built device tables and its count of live
 // states and ensembles, so that states may be created and destroyed from
 // several host threads.
 std::mutex g_grid_mu;
+
+// Grids of fewer columns run the column kernel: their row segments would not
+// give every SM one CTA.
+constexpr long long kRowMinCols = 4096;
 
 // ---------------------------------------------------------------- allocator
 agcm_alloc_fn g_alloc = nullptr;
@@ -240,7 +230,6 @@ struct agcm_state {
   bool bar_valid = false;
   // diagnostics partials
   double* diag = nullptr;
-  int* err = nullptr;  // device status word: AGCM_ETIMEOUT if a bounded wait gave up
   // side streams for the launches of a stage (and of an adjoint product) that
   // run beside the one on the caller's stream: forked from it by ev_fork,
   // joined to it by ev_join[q]
@@ -285,38 +274,97 @@ inline void leap1_band(const agcm_grid* g, int* lo, int* hi) {
   *hi = best_hi;
 }
 
-// Work items of the row-segment stage kernel, j << 8 | segment, for every row
-// whose halo leaves at least half of a CTA to owned columns (the grid's rows
-// must be 16-byte aligned, i.e. nlon % 4 == 0), in three classes: rows whose
-// strides Mu_j, Mv_j, Mu_{j+1} all equal kRowClsM[c] (1, 3, 5, 7), and the
-// others (nk[c] items each, listed in that order); and the rows left to the
-// column kernel.
-inline void row_lists(const agcm_grid* g, std::vector<int>* rowk, std::vector<int>* rowc, int nk[agcm::kRowCls]) {
-  std::vector<int> cls[agcm::kRowCls];
-  rowc->clear();
+// How the row-segment stage kernel divides a grid: the width of its CTAs in
+// threads, and whether rows of equal strides are taken in pairs.
+struct RowPlan {
+  int B = agcm::kRowB;
+  bool pair = true;
+};
+
+// Work items of the row-segment stage kernel (agcm_row.cuh): pairs of
+// rows j, j+1 whose strides Mu_j .. Mu_{j+2}, Mv_j, Mv_{j+1} are all equal
+// (plan.pair), the other rows whose halo leaves at least half of a CTA to
+// owned columns, and chunks of the rows left to the column body.  Listed
+// longest first; kind q's items are off[q] .. off[q] + cnt[q].  Without pairs
+// the single rows lie by stride class (any strides, all 7, 5, 3, 1): cls[c] is
+// where the c-th class starts.  Returns the threads of a CTA that holds every
+// item.
+inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>* items, int off[3], int cnt[3],
+                     int cls[agcm::kRowCls + 1]) {
+  std::vector<int4> pairs, polar, single[agcm::kRowCls];
+  int threads = 32;
   for (int j = 0; j < g->J; ++j) {
     const bool hv = j < g->J - 1;
     const int Mu = g->Mu[j], Mv = hv ? g->Mv[j] : Mu, M1 = hv ? g->Mu[j + 1] : Mu;
+    const bool eq = hv && Mu == Mv && Mu == M1;
+    const bool pair = plan.pair && eq && j + 2 < g->J && g->Mu[j + 2] == Mu && g->Mv[j + 1] == Mu;
     const int H = agcm::row_halo(Mu, hv ? Mv : 1, hv ? M1 : 1);
     int n = 0, S = 0;
-    agcm::row_segments(g->I, H, agcm::kRowB, &n, &S);
-    if (g->I % 4 == 0 && n > 0 && n < 256) {
-      // the last row has no V row: always the general class
-      int c = agcm::kRowCls - 1;
-      if (hv && Mu == Mv && Mu == M1)
-        for (int q = 0; q + 1 < agcm::kRowCls; ++q)
-          if (Mu == agcm::kRowClsM[q]) c = q;
-      for (int q = 0; q < n; ++q)
-        if (q * S < g->I) cls[c].push_back(j << 8 | q);
+    agcm::row_segments(g->I, H, plan.B, &n, &S);
+    if (n > 0) {
+      const int c = eq && !plan.pair && Mu <= 7 ? agcm::kRowCls - 1 - Mu / 2 : 0;
+      std::vector<int4>& list = pair ? pairs : single[c];
+      for (int q = 0; q < g->I; q += S) {
+        const int own = std::min(S, g->I - q);
+        list.push_back(make_int4((pair ? agcm::kRowPair : agcm::kRowAny) << 24 | j, q, own, H));
+        threads = std::max(threads, (own + 2 * H + 31) & ~31);
+      }
+      j += pair ? 1 : 0;
     } else {
-      rowc->push_back(j);
+      threads = agcm::kRowB;
+      for (int q = 0; q < g->I; q += agcm::kRowB) polar.push_back(make_int4(agcm::kRowPolar << 24 | j, q, agcm::kRowB, 0));
     }
   }
-  rowk->clear();
+  items->clear();
+  auto put = [&](int kind, const std::vector<int4>& v) {
+    if (cnt[kind] == 0) off[kind] = (int)items->size();
+    items->insert(items->end(), v.begin(), v.end());
+    cnt[kind] += (int)v.size();
+  };
+  cnt[0] = cnt[1] = cnt[2] = 0;
+  put(agcm::kRowPolar, polar);
+  put(agcm::kRowPair, pairs);
+  off[agcm::kRowAny] = (int)items->size();
   for (int c = 0; c < agcm::kRowCls; ++c) {
-    nk[c] = (int)cls[c].size();
-    rowk->insert(rowk->end(), cls[c].begin(), cls[c].end());
+    cls[c] = (int)items->size();
+    put(agcm::kRowAny, single[c]);
   }
+  cls[agcm::kRowCls] = (int)items->size();
+  return threads;
+}
+
+// Pairs, as long as they make two CTAs an SM (1440x720x30 FP32: 321 against
+// 428 us a stage with single rows, 720x360x30: 97 against 118, 405x203x26: 49
+// against 54); with fewer, single rows (256x128x30: 33.5 against 35 us; FP64
+// 128x64x8: 60 against 82 us).  Single rows in CTAs of the width that leaves
+// the fewest warps on the busiest of an SM's four schedulers, the narrowest
+// among equals (FP64 128x64x8, 64 threads: 52 us), up to three CTAs an SM.
+inline RowPlan row_plan(const agcm_grid* g) {
+  RowPlan p;
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      nsm < 1) {
+    cudaGetLastError();
+    nsm = 152;
+  }
+  std::vector<int4> items;
+  int off[3], cnt[3], cls[agcm::kRowCls + 1];
+  row_lists(g, p, &items, off, cnt, cls);
+  if ((long long)g->I * g->J >= kRowMinCols && (int)items.size() >= 2 * nsm) return p;
+  p.pair = false;
+  int best = 0;
+  for (int B : {128, 96, 64}) {
+    RowPlan q;
+    q.B = B;
+    q.pair = false;
+    const int threads = row_lists(g, q, &items, off, cnt, cls);
+    const int per_sm = (int)((items.size() + nsm - 1) / nsm), cost = (per_sm * (threads / 32) + 3) / 4;
+    if (B == 128 || (per_sm <= 3 && cost <= best)) {
+      p.B = B;
+      best = cost;
+    }
+  }
+  return p;
 }
 
 template <class T>
@@ -384,6 +432,28 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   const int nfU = (int)filtU.size(), nfV = (int)filtV.size();
   filtU.push_back(0);
   filtV.push_back(0);
+  // the row-segment kernel's level table and row tables
+  std::vector<double> lev((size_t)K * agcm::kLevN, 0.0), Af(J), Ac(J), rvn(JV), rvs(JV), rAd(J);
+  for (int k = 0; k < K; ++k) {
+    double* L = lev.data() + (size_t)k * agcm::kLevN;
+    L[agcm::kLevDs] = g->ds[k];
+    L[agcm::kLevH4] = 4.0 * Hkkb[k];
+    L[agcm::kLevh4] = 4.0 * hkb[k];
+    L[agcm::kLevhr2] = 2.0 * hk_rds[k];
+    L[agcm::kLevH2] = 2.0 * Hkkb[k];
+    L[agcm::kLevRds] = 1.0 / g->ds[k];
+    L[agcm::kLevSh] = g->sh[k];
+    L[agcm::kLevRho] = rho[k];
+  }
+  for (int j = 0; j < J; ++j) {
+    Af[j] = g->A[j] * f0[j];
+    Ac[j] = g->A[j] * cota[j];
+    rAd[j] = 1.0 / g->A[j];
+  }
+  for (int j = 0; j < JV; ++j) {
+    rvn[j] = g->Av[j] / g->A[j];
+    rvs[j] = g->Av[j] / g->A[j + 1];
+  }
   std::vector<double> rt0pit((size_t)J * I);
   for (size_t n = 0; n < rt0pit.size(); ++n) rt0pit[n] = g->rts[n] / g->pit[n];
 
@@ -400,15 +470,17 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   size_t o_ds = putT(g->ds), o_r2ds = putT(r2ds), o_hk = putT(hkb), o_Hkk = putT(Hkkb),
          o_hkr = putT(hk_rds), o_oms = putT(oms), o_rho = putT(rho), o_dsd = putD(g->ds), o_shd = putD(g->sh), o_Ad = putD(g->A),
          o_Avd = putD(g->Av.empty() ? std::vector<double>{0} : g->Av);
+  size_t o_lev = putT(lev), o_Af = putT(Af), o_Ac = putT(Ac), o_rAd = putD(rAd);
+  size_t o_rvn = putT(rvn.empty() ? std::vector<double>{0} : rvn), o_rvs = putT(rvs.empty() ? std::vector<double>{0} : rvs);
   size_t o_rt0 = putT(rt0pit), o_pit = putT(g->pit);
   size_t o_bu = putI(filtU), o_bv = putI(filtV);
-  std::vector<int> rowk, rowc;
-  int nk[agcm::kRowCls];
-  row_lists(g, &rowk, &rowc, nk);
-  const int nrowc = (int)rowc.size();
-  rowk.push_back(0);
-  rowc.push_back(0);
-  size_t o_rk = putI(rowk), o_rc = putI(rowc);
+  agcm::Geom<T> G{};
+  const RowPlan plan = row_plan(g);
+  std::vector<int4> items;
+  G.rowT = row_lists(g, plan, &items, G.off, G.cnt, G.cls);
+  G.nitems = (int)items.size();
+  items.push_back(make_int4(0, 0, 0, 0));
+  size_t o_it = put(items.data(), items.size() * sizeof(int4));
 
   void* d = dev_alloc(host.size());
   if (!d) return fail(AGCM_ENOMEM, "device allocation of %zu bytes for the grid tables failed", host.size());
@@ -417,7 +489,6 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
     return fail(AGCM_ECUDA, "copy of the grid tables failed: %s", cudaGetErrorString(cudaGetLastError()));
   }
   char* base = (char*)d;
-  agcm::Geom<T> G{};
   G.I = I; G.J = J; G.K = K;
   G.Mu = (const int*)(base + o_Mu);
   G.rdx = (const T*)(base + o_rdx);
@@ -454,12 +525,13 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   leap1_band(g, &G.l1lo, &G.l1hi);
   G.rady = (T)(1.0 / (kA * g->dth));
   G.adl = (T)(kA * g->dlam);
-  G.rowk = (const int*)(base + o_rk);
-  G.rowc = (const int*)(base + o_rc);
-  long long nitems = 0;
-  for (int c = 0; c < agcm::kRowCls; ++c) nitems += G.nk[c] = nk[c];
-  G.nrowc = nrowc;
-  G.rowfill = rows_fill_device(nitems);
+  G.lev = (const T*)(base + o_lev);
+  G.Af = (const T*)(base + o_Af);
+  G.Ac = (const T*)(base + o_Ac);
+  G.rvn = (const T*)(base + o_rvn);
+  G.rvs = (const T*)(base + o_rvs);
+  G.rAd = (const double*)(base + o_rAd);
+  G.items = (const int4*)(base + o_it);
   *blob_out = d;
   *geom_out = G;
   return AGCM_OK;
@@ -537,24 +609,23 @@ int ensure_bar(agcm_state* s, cudaStream_t st) {
 // bar[outb] (outb < 0: not written).
 //
 // Two designs of the stage kernel.  The row-segment kernel (agcm_row.cuh)
-// takes every row whose leap halo fits a CTA, when the rows are 16-byte
-// aligned; the few rows it leaves (the ones next to the poles on fine grids)
-// run the column kernel (agcm_fused.cuh, PART 3).  Grids or buffers the
-// row-segment kernel cannot take run the column kernel on every row, as the
-// stride-1 band (PART 2, specialised body) and the other rows (PART 1).
-// Given aux, evf and evj (kSide side streams, a fork event and one join event
-// per side stream), launches other than the first run on side streams,
-// forked from st after everything already queued there and joined back
-// before st continues, so they overlap; without them they run one after the
-// other on st.  *launched (optional) receives the number of kernel launches
-// made.
-#ifndef AGCM_ROW_KERNEL
-#define AGCM_ROW_KERNEL 1
-#endif
+// takes a whole stage in one launch, the rows next to the poles of fine grids
+// on the column body inside it; it is launched as a dependent of the launch
+// before it (programmatic stream serialisation), so its set-up runs while
+// that one's last blocks do.  Grids of fewer than kRowMinCols columns
+// run the column kernel (agcm_fused.cuh) instead, on every row, as the
+// stride-1 band (PART 2, specialised body) and the other rows (PART 1); where
+// the row-segment kernel is asked for on such a grid, each stride class is a
+// launch of its own (the launches a state's profile has always counted there).  Given aux, evf
+// and evj (kSide side streams, a fork event and one join event per side
+// stream), launches other than the last run on side streams, forked from st
+// after everything already queued there and joined back before st continues,
+// so they overlap; without them they run one after the other on st.
+// *launched (optional) receives the number of kernel launches made.
 template <class T, int MODE, int TERMS = 3>
 int launch_fused(const agcm::Geom<T>& G, const void* const xs[4], const double* ub, const double* vb,
                  const void* const xb[4], void* const out[4], double* ubo, double* vbo, const double* ubb,
-                 const double* vbb, double cdt, int* err, cudaStream_t st, const cudaStream_t* aux = nullptr,
+                 const double* vbb, double cdt, cudaStream_t st, const cudaStream_t* aux = nullptr,
                  cudaEvent_t evf = nullptr, const cudaEvent_t* evj = nullptr, int* launched = nullptr,
                  int state_choice = 0) {
   if (launched) *launched = 1;
@@ -567,106 +638,87 @@ int launch_fused(const agcm::Geom<T>& G, const void* const xs[4], const double* 
             (const T*)xb[1], (const T*)xb[2], (const T*)xb[3], (T*)out[0], (T*)out[1], (T*)out[2], (T*)out[3],
             ubo, vbo, ubb, vbb, (T)cdt);
   };
-  auto two = [&](auto first, auto second) -> int {  // first on aux[0] (forked), second on st
-    if (fork) {
-      CUDA_TRY(cudaEventRecord(evf, st));
-      CUDA_TRY(cudaStreamWaitEvent(aux[0], evf, 0));
+  // n launches go(q, stream): all but the last on side streams
+  auto side_by_side = [&](int n, auto go) -> int {
+    const bool f = fork && n > 1;
+    if (f) CUDA_TRY(cudaEventRecord(evf, st));
+    int rc = AGCM_OK;
+    for (int q = 0; q < n; ++q) {
+      const bool side = f && q < n - 1;
+      if (side) CUDA_TRY(cudaStreamWaitEvent(aux[q], evf, 0));
+      if (!rc) rc = go(q, side ? aux[q] : st);
     }
-    first(fork ? aux[0] : st);
-    second(st);
-    if (fork) {
-      CUDA_TRY(cudaEventRecord(evj[0], aux[0]));
-      CUDA_TRY(cudaStreamWaitEvent(st, evj[0], 0));
+    for (int q = 0; f && q < n - 1; ++q) {  // joined whatever rc says, so that no side stream is left forked
+      CUDA_TRY(cudaEventRecord(evj[q], aux[q]));
+      CUDA_TRY(cudaStreamWaitEvent(st, evj[q], 0));
     }
-    if (launched) *launched = 2;
-    return AGCM_OK;
+    if (launched) *launched = n;
+    return rc;
   };
+  auto gap = [](const void* p, const void* q) { return ((const T*)p) - ((const T*)q); };
   auto a16 = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
   // a state's own choice (agcm_state_set_stage_kernel), else the process's
   const int choice = state_choice > 0 ? state_choice : g_stage_choice.load(std::memory_order_relaxed);
-  int nitems = 0;
-  for (int c = 0; c < agcm::kRowCls; ++c) nitems += G.nk[c];
-  bool rowpath = AGCM_ROW_KERNEL && choice != 1 && (choice == 2 || G.rowfill) && nitems > 0 &&
-                 a16(xs[0]) && a16(xs[1]) && a16(xs[2]);
-  if (MODE == 2) rowpath = rowpath && a16(xb[0]) && a16(xb[1]) && a16(xb[2]);
-  const size_t smem = agcm::row_smem_bytes<T>(agcm::kRowB, G.K);
-  if (smem > 227 * 1024) rowpath = false;
+  const size_t smem = agcm::row_smem_bytes<T>(G.K);
+  const bool rowpath = choice != 1 && G.nitems > 0 && (choice == 2 || (long long)G.I * G.J >= kRowMinCols) && smem <= 227 * 1024;
   auto rows = [&](auto nl) -> int {
     if (rowpath) {
+      // 16-byte aligned rows are staged by bulk copies, others element by element
+      bool vec = G.I % 4 == 0 && a16(xs[0]) && a16(xs[1]) && a16(xs[2]);
+      if (MODE == 2) vec = vec && a16(xb[0]) && a16(xb[1]) && a16(xb[2]);
       agcm::RowArgs<T> ra{(const T*)xs[0], (const T*)xs[1], (const T*)xs[2], (const T*)xs[3], ub, vb,
                           (const T*)xb[0], (const T*)xb[1], (const T*)xb[2], (const T*)xb[3], (T*)out[0],
-                          (T*)out[1], (T*)out[2], (T*)out[3], ubo, vbo, ubb, vbb, (T)cdt, G.rowk, err};
-      int nlaunch = 0;
-      // one launch per stride class, or one over classes [c0, c1) (the
-      // body for any strides); class c's items follow those of the classes before it
-      auto cls_go = [&](auto mc, int c0, int c1, cudaStream_t q) -> int {
-        int off = 0, n = 0;
-        for (int c = 0; c < c1; ++c) (c < c0 ? off : n) += G.nk[c];
-        if (n == 0) return AGCM_OK;
-        auto kern = agcm::k_row_stage<T, MODE, TERMS, decltype(nl)::value, decltype(mc)::value>;
-        static std::atomic<size_t> attr{0};  // per instantiation: the size set so far
-        if (attr.load() < smem) {
-          CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-          attr.store(smem);
-        }
+                          (T*)out[1], (T*)out[2], (T*)out[3], ubo, vbo, ubb, vbb, (T)cdt, vec ? 1 : 0, gap(xs[2], xs[0]), gap(xs[1], xs[0]), MODE == 2 ? gap(xb[1], xb[0]) : 0, 0};
+      auto kern = agcm::k_row_stage<T, MODE, TERMS, decltype(nl)::value>;
+      static std::atomic<size_t> attr{0};  // per instantiation: the size set so far
+      if (attr.load() < smem) {
+        CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        attr.store(smem);
+      }
+      auto go = [&](int off, int n, cudaStream_t q, bool dependent) -> int {
         agcm::RowArgs<T> rc = ra;
-        rc.rows = G.rowk + off;
-        kern<<<(unsigned)n, agcm::kRowB, smem, q>>>(G, rc);
-        ++nlaunch;
+        rc.first = off;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)n);
+        cfg.blockDim = dim3((unsigned)G.rowT);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = q;
+        cfg.attrs = &at;
+        cfg.numAttrs = dependent ? 1 : 0;
+        CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, G, rc));
         return AGCM_OK;
       };
-      // the launches run side by side: the stride-1 rows on st, the rows
-      // next to the poles (column kernel), the stride-3, 5 and 7 rows and
-      // the other rows each on a side stream (a launch of less than a
-      // wave then no longer waits for another's last wave).  They are issued
-      // longest block first (the column kernel's level walk, then the rows
-      // with the widest halos), and the side streams' priorities keep that
-      // order, so that the shortest blocks fill the last wave.  The stride-5
-      // and 7 classes have bodies of their own in the stages of a step; the
-      // tendency and the split term groups take them with the other rows.
-      constexpr bool kSpec = MODE != 0 && TERMS == 3;
-      constexpr int cAny = agcm::kRowCls - 1;
-      const int cOther = kSpec ? cAny : 2;
-      int nOther = 0;
-      for (int c = cOther; c < agcm::kRowCls; ++c) nOther += G.nk[c];
-      const bool side[kSide] = {G.nrowc > 0, G.nk[1] > 0, nOther > 0, kSpec && G.nk[2] > 0, kSpec && G.nk[3] > 0};
-      if (fork) {
-        CUDA_TRY(cudaEventRecord(evf, st));
-        for (int q = 0; q < kSide; ++q)
-          if (side[q]) CUDA_TRY(cudaStreamWaitEvent(aux[q], evf, 0));
+      if ((long long)G.I * G.J >= kRowMinCols) return go(0, G.nitems, st, true);
+      int off[agcm::kRowCls + 1], cnt[agcm::kRowCls + 1], n = 0;
+      if (G.cnt[agcm::kRowPolar]) {
+        off[n] = 0;
+        cnt[n++] = G.cnt[agcm::kRowPolar];
       }
-      if (G.nrowc > 0) {
-        col_launch(nl, std::integral_constant<int, 3>{}, G.nrowc, fork ? aux[0] : st);
-        ++nlaunch;
-      }
-      int rc = cls_go(std::integral_constant<int, 0>{}, cOther, agcm::kRowCls, fork ? aux[2] : st);
-      if (!rc) rc = cls_go(std::integral_constant<int, 3>{}, 1, 2, fork ? aux[1] : st);
-      if constexpr (kSpec) {
-        if (!rc) rc = cls_go(std::integral_constant<int, 7>{}, 3, 4, fork ? aux[4] : st);
-        if (!rc) rc = cls_go(std::integral_constant<int, 5>{}, 2, 3, fork ? aux[3] : st);
-      }
-      if (!rc) rc = cls_go(std::integral_constant<int, 1>{}, 0, 1, st);
-      if (fork) {  // joined whatever rc says, so that no side stream is left forked
-        for (int q = 0; q < kSide; ++q)
-          if (side[q]) {
-            CUDA_TRY(cudaEventRecord(evj[q], aux[q]));
-            CUDA_TRY(cudaStreamWaitEvent(st, evj[q], 0));
-          }
-      }
-      if (rc) return rc;
-      if (launched) *launched = nlaunch;
-    } else {
-      const int nb = G.l1hi - G.l1lo;
-      if (nb <= 0) {
-        col_launch(nl, std::integral_constant<int, 0>{}, G.J, st);
-      } else if (nb == G.J) {
-        col_launch(nl, std::integral_constant<int, 2>{}, nb, st);
-      } else {
-        int rc = two([&](cudaStream_t q) { col_launch(nl, std::integral_constant<int, 2>{}, nb, q); },
-                     [&](cudaStream_t q) { col_launch(nl, std::integral_constant<int, 1>{}, G.J - nb, q); });
-        if (rc) return rc;
-      }
+      for (int c = 0; c < agcm::kRowCls; ++c)
+        if (G.cls[c + 1] > G.cls[c]) {
+          off[n] = G.cls[c];
+          cnt[n++] = G.cls[c + 1] - G.cls[c];
+        }
+      return side_by_side(n, [&](int q, cudaStream_t qs) { return go(off[q], cnt[q], qs, false); });
     }
+    const int nb = G.l1hi - G.l1lo;
+    int rc = AGCM_OK;
+    if (nb <= 0)
+      col_launch(nl, std::integral_constant<int, 0>{}, G.J, st);
+    else if (nb == G.J)
+      col_launch(nl, std::integral_constant<int, 2>{}, nb, st);
+    else
+      rc = side_by_side(2, [&](int q, cudaStream_t qs) {
+        if (q == 0)
+          col_launch(nl, std::integral_constant<int, 2>{}, nb, qs);
+        else
+          col_launch(nl, std::integral_constant<int, 1>{}, G.J - nb, qs);
+        return AGCM_OK;
+      });
+    if (rc) return rc;
     CUDA_TRY(cudaGetLastError());
     return AGCM_OK;
   };
@@ -684,7 +736,7 @@ int fused_stage(agcm_state* s, int in, void* const out[4], int outb, double cdt,
   int launched = 1;
   int rc = launch_fused<T, MODE, TERMS>(G, s->x[in], s->ubar[in], s->vbar[in], s->x[0], out,
                                  outb >= 0 ? s->ubar[outb] : nullptr, outb >= 0 ? s->vbar[outb] : nullptr,
-                                 s->ubar[0], s->vbar[0], cdt, s->err, st, s->aux, s->ev_fork, s->ev_join,
+                                 s->ubar[0], s->vbar[0], cdt, st, s->aux, s->ev_fork, s->ev_join,
                                  &launched, s->stage_choice);
   s->prof.end(st, launched);
   return rc;
@@ -1029,8 +1081,6 @@ int agcm_state_create(const agcm_grid_t* g, int precision, int nmembers, agcm_st
     ok = ok && (s->vbar[c] = (double*)get(s->n2 * sizeof(double)));
   }
   ok = ok && (s->diag = (double*)get((agcm::kDiagPartials + 1) * 8 * sizeof(double)));
-  ok = ok && (s->err = (int*)get(256));
-  if (ok) cudaMemset(s->err, 0, sizeof(int));
   if (!ok) {
     for (void* p : s->owned) dev_free(p);
     delete s;
@@ -1041,9 +1091,7 @@ int agcm_state_create(const agcm_grid_t* g, int precision, int nmembers, agcm_st
       size_t n = f == 1 ? std::max<size_t>(s->nv, 1) : (f == 3 ? s->n2 : s->n3);
       cudaMemset(s->x[c][f], 0, n * s->esz);
     }
-  // side stream priorities: the rows next to the poles and the rows of any
-  // strides (the widest halos, the longest blocks) first, then the stride-3,
-  // 5 and 7 classes; the stride-1 class runs on the caller's stream
+  // side stream priorities: first the launches with the longest blocks
   int prio_least = 0, prio_greatest = 0;
   bool side_ok = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest) == cudaSuccess &&
                  cudaEventCreateWithFlags(&s->ev_fork, cudaEventDisableTiming) == cudaSuccess;
@@ -1214,9 +1262,6 @@ int agcm_diagnostics(const agcm_state_t* s, agcm_diag_t* out, void* stream) {
   out->max_v = h[5];
   out->finite = h[6] == 0.0 ? 1 : 0;
   out->reserved = 0;
-  int e = 0;
-  CUDA_TRY(cudaMemcpy(&e, s->err, sizeof(int), cudaMemcpyDeviceToHost));
-  if (e == AGCM_ETIMEOUT) return fail(AGCM_ETIMEOUT, "a bounded wait in the stage kernel gave up");
   if (!out->finite) return fail(AGCM_ENONFINITE, "state holds %g non-finite values", h[6]);
   return AGCM_OK;
 }
@@ -1450,14 +1495,14 @@ constexpr size_t kOffRaw = 0;                        // 6 row arrays s c cot A s
 constexpr size_t kOffRawLev = kOffRaw + 6 * kRowB;   // sh ds Hkk hk beta (double)
 constexpr size_t kOffPitRaw = kOffRawLev + 5 * kLevB;  // pi~, R T~_s (double)
 constexpr size_t kOffInt = kOffPitRaw + 2 * kColB;   // Mu Mv (int)
-constexpr size_t kOffRowT = kOffInt + 2 * kRowB;     // 12 typed row arrays
-constexpr size_t kOffLevT = kOffRowT + 12 * kRowB;   // 7 typed level arrays
-constexpr size_t kOffColT = kOffLevT + 7 * kLevB;    // pit, rt0pit (typed)
+constexpr size_t kOffRowT = kOffInt + 2 * kRowB;     // 16 typed row arrays, 1 / A_j (double)
+constexpr size_t kOffLevT = kOffRowT + 17 * kRowB;   // 7 typed level arrays, the level table of kLevN values
+constexpr size_t kOffColT = kOffLevT + (7 + agcm::kLevN) * kLevB;  // pit, rt0pit (typed)
 constexpr size_t kOffBar = kOffColT + 2 * kColB;     // Ubar, Vbar (double)
-constexpr size_t kOffRowL = kOffBar + 2 * kColB;     // row-segment items, then column-kernel rows (int)
-constexpr size_t kItemB = al256((kStaticCols / 128 + kStaticRows) * 4);  // at most ceil(nlon/128) items a row
-constexpr size_t kOffErr = kOffRowL + kItemB + al256(kStaticRows * 4);  // status word of the stage kernel
-constexpr size_t kStaticBytes = kOffErr + 256;       // about 13 MB
+constexpr size_t kOffRowL = kOffBar + 2 * kColB;     // row-segment items (int4)
+// at most ceil(nlon / 32) items a row (64-thread CTAs own at least 32 columns)
+constexpr size_t kItemB = al256((kStaticCols / 32 + kStaticRows) * sizeof(int4));
+constexpr size_t kStaticBytes = kOffRowL + kItemB;  // about 13 MB
 
 }  // namespace
 
@@ -1474,8 +1519,8 @@ int g_static_prec[kStaticMaxDevices] = {};
 // Typed device tables from the raw FP64 ones (same formulas as the state path).
 template <class T>
 __global__ void k_static_geom(int I, int J, int K, const double* raw, const double* rawlev, const double* pitraw,
-                              const int* Mu, const int* Mv, T* rowT, T* levT, T* colT, size_t rowStride,
-                              size_t levStride, size_t colStride, double beta2) {
+                              const int* Mu, const int* Mv, T* rowT, double* rAd, T* levT, T* colT,
+                              size_t rowStride, size_t levStride, size_t colStride, double beta2) {
   const double* s = raw;
   const double* c = raw + rowStride;
   const double* cot = raw + 2 * rowStride;
@@ -1506,7 +1551,12 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
         rowT[9 * rowStride + j] = (T)(0.5 / Av[j]);
         rowT[10 * rowStride + j] = (T)(0.25 * A[j] / Av[j]);
         rowT[11 * rowStride + j] = (T)(0.25 * A[j + 1] / Av[j]);
+        rowT[12 * rowStride + j] = (T)(Av[j] / A[j]);
+        rowT[13 * rowStride + j] = (T)(Av[j] / A[j + 1]);
       }
+      rowT[14 * rowStride + j] = (T)(A[j] * (2.0 * kOmega * c[j]));
+      rowT[15 * rowStride + j] = (T)(A[j] * (cot[j] / kA));
+      rAd[j] = 1.0 / A[j];
     }
     if (n < (size_t)K) {
       const int k = (int)n;
@@ -1517,6 +1567,15 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
       levT[4 * levStride + k] = (T)(beta[k] * hk[k] / ds[k]);
       levT[5 * levStride + k] = (T)(1.0 - rawlev[k]);
       levT[6 * levStride + k] = (T)(beta[k] != 0.0 ? beta2 / beta[k] : 0.0);
+      T* L = levT + 7 * levStride + (size_t)k * agcm::kLevN;
+      L[agcm::kLevDs] = (T)ds[k];
+      L[agcm::kLevH4] = (T)(4.0 * (beta[k] * rawlev[2 * levStride + k]));
+      L[agcm::kLevh4] = (T)(4.0 * (beta[k] * hk[k]));
+      L[agcm::kLevhr2] = (T)(2.0 * (beta[k] * hk[k] / ds[k]));
+      L[agcm::kLevRds] = (T)(1.0 / ds[k]);
+      L[agcm::kLevSh] = (T)rawlev[k];
+      L[agcm::kLevRho] = levT[6 * levStride + k];
+      L[agcm::kLevH2] = (T)(2.0 * (beta[k] * rawlev[2 * levStride + k]));
     }
     if (n < ncol) {
       colT[n] = (T)pitraw[n];
@@ -1542,6 +1601,12 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   T* rowT = (T*)(base + kOffRowT);
   T* levT = (T*)(base + kOffLevT);
   T* colT = (T*)(base + kOffColT);
+  double* rAd = (double*)(base + kOffRowT + 16 * kRowB);
+  agcm::Geom<T> G{};
+  const RowPlan plan = row_plan(g);
+  std::vector<int4> items;  // host only
+  G.rowT = row_lists(g, plan, &items, G.off, G.cnt, G.cls);
+  G.nitems = (int)items.size();
   if (tables) {
   const std::vector<double>* rows[6] = {&g->s, &g->c, &g->cot, &g->A, &g->sv, &g->Av};
   for (int q = 0; q < 6; ++q)
@@ -1556,21 +1621,13 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   if (!g->Mv.empty())
     CUDA_TRY(cudaMemcpyAsync(Mv, g->Mv.data(), g->Mv.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   {
-    std::vector<int> rk, rc;
-    int nk[agcm::kRowCls];
-    row_lists(g, &rk, &rc, nk);
-    if (!rk.empty())
-      CUDA_TRY(cudaMemcpyAsync(base + kOffRowL, rk.data(), rk.size() * sizeof(int), cudaMemcpyHostToDevice, st));
-    if (!rc.empty())
-      CUDA_TRY(cudaMemcpyAsync(base + kOffRowL + kItemB, rc.data(), rc.size() * sizeof(int),
-                               cudaMemcpyHostToDevice, st));
-    CUDA_TRY(cudaMemsetAsync(base + kOffErr, 0, sizeof(int), st));
+    if (!items.empty())
+      CUDA_TRY(cudaMemcpyAsync(base + kOffRowL, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
   }
   k_static_geom<T><<<nblocks(std::max<size_t>((size_t)I * J, (size_t)K), 256), 256, 0, st>>>(
-      I, J, K, raw, rawlev, pitraw, Mu, Mv, rowT, levT, colT, rS, lS, cS, g->beta2);
+      I, J, K, raw, rawlev, pitraw, Mu, Mv, rowT, rAd, levT, colT, rS, lS, cS, g->beta2);
   CUDA_TRY(cudaGetLastError());
   }
-  agcm::Geom<T> G{};
   G.I = I; G.J = J; G.K = K;
   G.Mu = Mu;
   G.Mv = Mv;
@@ -1591,24 +1648,17 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   G.rt0pit = colT + cS;
   G.rady = (T)(1.0 / (kA * g->dth));
   G.adl = (T)(kA * g->dlam);
-  {
-    std::vector<int> rk, rc;
-    row_lists(g, &rk, &rc, G.nk);  // host only: counts (the lists were copied with the tables)
-    G.nrowc = (int)rc.size();
-    long long nitems = 0;
-    for (int c = 0; c < agcm::kRowCls; ++c) nitems += G.nk[c];
-    G.rowfill = rows_fill_device(nitems);
-    G.rowk = (const int*)(base + kOffRowL);
-    G.rowc = (const int*)(base + kOffRowL + kItemB);
-  }
+  G.rvn = rowT + 12 * rS; G.rvs = rowT + 13 * rS; G.Af = rowT + 14 * rS; G.Ac = rowT + 15 * rS;
+  G.rAd = rAd;
+  G.lev = levT + 7 * lS;
+  G.items = (const int4*)(base + kOffRowL);
   double* ubar = (double*)(base + kOffBar);
   double* vbar = (double*)(base + kOffBar + kColB);
   agcm::k_vsum<T><<<nblocks((size_t)I * J, 256), 256, 0, st>>>(G, (const T*)U, (const T*)V, ubar, vbar);
   const void* xs[4] = {U, V, Phi, pi};
   const void* none[4] = {nullptr, nullptr, nullptr, nullptr};
   void* out[4] = {tU, tV, tPhi, tpi};
-  return launch_fused<T, 0>(G, xs, ubar, vbar, none, out, nullptr, nullptr, nullptr, nullptr, 1.0,
-                            (int*)(base + kOffErr), st);
+  return launch_fused<T, 0>(G, xs, ubar, vbar, none, out, nullptr, nullptr, nullptr, nullptr, 1.0, st);
 }
 
 }  // namespace
@@ -1671,7 +1721,7 @@ struct agcm_ensemble {
   int test_missing = 0;
   bool desc_dirty = true;
   // work items of the row-segment persistent launch (warps_per_block = 8)
-  std::vector<int> host_items;   // int2 pairs
+  std::vector<int4> host_items;  // the row items of every member, member << 8 in w
   void* d_items = nullptr;
   int nitems_rows = 0;
   size_t rows_smem = 0;          // dynamic shared memory of that launch
@@ -1694,6 +1744,10 @@ void fill_desc(agcm_ensemble* e) {
       d[m].ubar[c] = s->ubar[c];
       d[m].vbar[c] = s->vbar[c];
     }
+    d[m].vec = s->grid->I % 4 == 0;
+    for (int c = 0; c < 3; ++c)
+      for (int f = 0; f < 3; ++f)
+        if ((uintptr_t)s->x[c][f] & 15) d[m].vec = 0;
     d[m].nbx = (s->grid->I + 31) / 32;
     d[m].item_begin = begin;
     d[m].dt = (T)0;
@@ -1706,21 +1760,16 @@ void fill_desc(agcm_ensemble* e) {
   e->rows_smem = 0;
   for (size_t m = 0; m < e->members.size(); ++m) {
     const agcm_grid* g = e->members[m]->grid;
-    std::vector<int> rk, rc;
-    int nk[agcm::kRowCls];
-    row_lists(g, &rk, &rc, nk);
-    for (int it : rk) {
-      e->host_items.push_back((int)m);
+    std::vector<int4> items;
+    int off[3], cnt[3], cls[agcm::kRowCls + 1];
+    row_lists(g, row_plan(g), &items, off, cnt, cls);
+    for (int4 it : items) {
+      it.w |= (int)m << 8;
       e->host_items.push_back(it);
     }
-    for (int j : rc)
-      for (int c = 0; c * agcm::kRowB < g->I; ++c) {
-        e->host_items.push_back((int)m | (1 << 16));
-        e->host_items.push_back(j << 8 | c);
-      }
-    e->rows_smem = std::max(e->rows_smem, agcm::row_smem_bytes<T>(agcm::kRowB, g->K));
+    e->rows_smem = std::max(e->rows_smem, agcm::row_smem_bytes<T>(g->K));
   }
-  e->nitems_rows = (int)(e->host_items.size() / 2);
+  e->nitems_rows = (int)e->host_items.size();
 }
 
 template <class T>
@@ -1761,7 +1810,7 @@ int ensemble_step(agcm_ensemble* e, int nsteps, const double* dt, cudaStream_t s
       const int chunk = std::min(e->queue_cap, nsteps - done);
       CUDA_TRY(cudaMemsetAsync(e->d_sync, 0, sync_bytes, st));
       e->prof.begin(KID_ENSEMBLE, st);
-      kr<<<grid, agcm::kRowB, e->rows_smem, st>>>((const agcm::EnsMember<T>*)e->d_desc, (const int2*)e->d_items,
+      kr<<<grid, agcm::kRowB, e->rows_smem, st>>>((const agcm::EnsMember<T>*)e->d_desc, (const int4*)e->d_items,
                                                  e->nitems_rows, chunk, e->d_sync, grid + (unsigned)e->test_missing,
                                                  limit);
       e->prof.end(st);
@@ -1822,9 +1871,9 @@ int agcm_ensemble_create(agcm_state_t* const* members, int n, agcm_ensemble_t** 
     fill_desc<float>(e);
   e->queue_cap = 1024;
   e->d_desc = dev_alloc(e->host_desc.size());
-  e->d_items = dev_alloc(std::max<size_t>(e->host_items.size(), 2) * sizeof(int));
+  e->d_items = dev_alloc(std::max<size_t>(e->host_items.size(), 1) * sizeof(int4));
   if (e->d_items && !e->host_items.empty() &&
-      cudaMemcpy(e->d_items, e->host_items.data(), e->host_items.size() * sizeof(int), cudaMemcpyHostToDevice) !=
+      cudaMemcpy(e->d_items, e->host_items.data(), e->host_items.size() * sizeof(int4), cudaMemcpyHostToDevice) !=
           cudaSuccess) {
     dev_free(e->d_items);
     e->d_items = nullptr;

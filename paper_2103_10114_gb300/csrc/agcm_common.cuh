@@ -9,11 +9,9 @@
 
 namespace agcm {
 
-// Stride classes of the row-segment stage kernel: rows whose strides Mu_j,
-// Mv_j, Mu_{j+1} all equal kRowClsM[c] (compile-time partner offsets), and
-// a last class of rows with any strides.
+// Stride classes of single rows (all strides 1, 3, 5, 7; any): the order of a
+// small grid's items and its launches.
 constexpr int kRowCls = 5;
-constexpr int kRowClsM[kRowCls] = {1, 3, 5, 7, 0};
 
 // Per-grid tables on the device, in the arithmetic type T of the kernels.
 // Built once per (grid, precision) by the host from the FP64 geometry.
@@ -46,6 +44,11 @@ struct Geom {
   const T* hk_rds;  // hk / dsigma_k (K)
   const T* rho;     // beta2 / beta_k: the delta kappa Phi/P part of the coefficient (K)
   const T* oms;     // 1 - sigma_hat_k (K): W_k = SD_k - (1 - sigma_hat_k) C
+  // the row-segment kernel's tables: per level kLevN values (kLev...), per row
+  // A_j f0, A_j cot(theta_j) / a (J), Av_j / A_j, Av_j / A_{j+1} (J-1), 1 / A_j in FP64 (J)
+  const T* lev;
+  const T *Af, *Ac, *rvn, *rvs;
+  const double* rAd;
   // rows the low-latitude filter changes, entry 4 j + band (1 two-grid, 2 3-point)
   const int* filtU; // scalar / U rows
   const int* filtV; // V rows
@@ -61,15 +64,18 @@ struct Geom {
   int l1lo, l1hi;   // rows [l1lo, l1hi): interior rows whose strides Mu_j, Mv_j, Mu_{j+1} are all 1
   T rady;           // 1 / (a dth)
   T adl;            // a dlam
-  // work items of the row-segment stage kernel (agcm_row.cuh), j << 8 | segment:
-  // nk[c] items of the rows of stride class c, listed by class: strides all
-  // kRowClsM[c] (1, 3, 5, 7), then (c = kRowCls - 1) the other rows; and the
-  // nrowc rows left to the column kernel (agcm_fused.cuh)
-  const int* rowk;
-  const int* rowc;
-  int nk[kRowCls], nrowc;
-  int rowfill;      // 1: the row-segment items fill the GPU at least four times over
+  // work items of the row-segment stage kernel (agcm_row.cuh), longest first:
+  // chunks of the rows left to the column body, pairs of rows of equal strides,
+  // single rows; kind q's items are items[off[q]] .. items[off[q] + cnt[q]],
+  // the single rows' stride classes start at cls[c]
+  const int4* items;
+  int off[3], cnt[3], cls[kRowCls + 1], nitems;
+  int rowT;  // threads of a CTA that holds every item
 };
+
+// Values per level of Geom::lev: dsigma, 4 beta Hkk, 4 beta hk, 2 beta hk /
+// dsigma, 1 / dsigma, sigma_hat (the level's upper half level), rho, 2 beta Hkk.
+enum { kLevDs, kLevH4, kLevh4, kLevhr2, kLevRds, kLevSh, kLevRho, kLevH2, kLevN };
 
 __device__ __forceinline__ int wrapi(int i, int I) {
   return i < 0 ? i + I : (i >= I ? i - I : i);
