@@ -367,6 +367,12 @@ inline RowPlan row_plan(const agcm_grid* g) {
   return p;
 }
 
+// x as the sum of three FP32 numbers (72 bits)
+inline float4 split3(double x) {
+  const float a = (float)x, b = (float)(x - (double)a);
+  return make_float4(a, b, (float)((x - (double)a) - (double)b), 0.f);
+}
+
 template <class T>
 int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   const int I = g->I, J = g->J, K = g->K;
@@ -470,6 +476,9 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   size_t o_ds = putT(g->ds), o_r2ds = putT(r2ds), o_hk = putT(hkb), o_Hkk = putT(Hkkb),
          o_hkr = putT(hk_rds), o_oms = putT(oms), o_rho = putT(rho), o_dsd = putD(g->ds), o_shd = putD(g->sh), o_Ad = putD(g->A),
          o_Avd = putD(g->Av.empty() ? std::vector<double>{0} : g->Av);
+  std::vector<float4> ds3(K);
+  for (int k = 0; k < K; ++k) ds3[k] = split3(g->ds[k]);
+  size_t o_ds3 = put(ds3.data(), K * sizeof(float4));
   size_t o_lev = putT(lev), o_Af = putT(Af), o_Ac = putT(Ac), o_rAd = putD(rAd);
   size_t o_rvn = putT(rvn.empty() ? std::vector<double>{0} : rvn), o_rvs = putT(rvs.empty() ? std::vector<double>{0} : rvs);
   size_t o_rt0 = putT(rt0pit), o_pit = putT(g->pit);
@@ -525,6 +534,7 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   leap1_band(g, &G.l1lo, &G.l1hi);
   G.rady = (T)(1.0 / (kA * g->dth));
   G.adl = (T)(kA * g->dlam);
+  G.ds3 = (const float4*)(base + o_ds3);
   G.lev = (const T*)(base + o_lev);
   G.Af = (const T*)(base + o_Af);
   G.Ac = (const T*)(base + o_Ac);
@@ -596,7 +606,7 @@ int ensure_bar(agcm_state* s, cudaStream_t st) {
   if (s->bar_valid) return AGCM_OK;
   const agcm::Geom<T>& G = geom_of<T>(s);
   s->prof.begin(KID_VSUM, st);
-  agcm::k_vsum<T><<<nblocks(s->n2, 256), 256, 0, st>>>(G, (const T*)s->x[0][0], (const T*)s->x[0][1], s->ubar[0],
+  agcm::k_vsum<T><<<dim3(nblocks(s->n2, 256), 2), 256, 0, st>>>(G, (const T*)s->x[0][0], (const T*)s->x[0][1], s->ubar[0],
                                                        s->vbar[0]);
   s->prof.end(st);
   CUDA_TRY(cudaGetLastError());
@@ -1497,7 +1507,8 @@ constexpr size_t kOffPitRaw = kOffRawLev + 5 * kLevB;  // pi~, R T~_s (double)
 constexpr size_t kOffInt = kOffPitRaw + 2 * kColB;   // Mu Mv (int)
 constexpr size_t kOffRowT = kOffInt + 2 * kRowB;     // 16 typed row arrays, 1 / A_j (double)
 constexpr size_t kOffLevT = kOffRowT + 17 * kRowB;   // 7 typed level arrays, the level table of kLevN values
-constexpr size_t kOffColT = kOffLevT + (7 + agcm::kLevN) * kLevB;  // pit, rt0pit (typed)
+constexpr size_t kOffDs3 = kOffLevT + (7 + agcm::kLevN) * kLevB;   // dsigma in three FP32 parts
+constexpr size_t kOffColT = kOffDs3 + 2 * kLevB;                    // pit, rt0pit (typed)
 constexpr size_t kOffBar = kOffColT + 2 * kColB;     // Ubar, Vbar (double)
 constexpr size_t kOffRowL = kOffBar + 2 * kColB;     // row-segment items (int4)
 // at most ceil(nlon / 32) items a row (64-thread CTAs own at least 32 columns)
@@ -1519,7 +1530,7 @@ int g_static_prec[kStaticMaxDevices] = {};
 // Typed device tables from the raw FP64 ones (same formulas as the state path).
 template <class T>
 __global__ void k_static_geom(int I, int J, int K, const double* raw, const double* rawlev, const double* pitraw,
-                              const int* Mu, const int* Mv, T* rowT, double* rAd, T* levT, T* colT,
+                              const int* Mu, const int* Mv, T* rowT, double* rAd, T* levT, float4* ds3, T* colT,
                               size_t rowStride, size_t levStride, size_t colStride, double beta2) {
   const double* s = raw;
   const double* c = raw + rowStride;
@@ -1567,6 +1578,10 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
       levT[4 * levStride + k] = (T)(beta[k] * hk[k] / ds[k]);
       levT[5 * levStride + k] = (T)(1.0 - rawlev[k]);
       levT[6 * levStride + k] = (T)(beta[k] != 0.0 ? beta2 / beta[k] : 0.0);
+      {
+        const float x = (float)ds[k], y = (float)(ds[k] - (double)x);
+        ds3[k] = make_float4(x, y, (float)((ds[k] - (double)x) - (double)y), 0.f);
+      }
       T* L = levT + 7 * levStride + (size_t)k * agcm::kLevN;
       L[agcm::kLevDs] = (T)ds[k];
       L[agcm::kLevH4] = (T)(4.0 * (beta[k] * rawlev[2 * levStride + k]));
@@ -1625,7 +1640,7 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
       CUDA_TRY(cudaMemcpyAsync(base + kOffRowL, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
   }
   k_static_geom<T><<<nblocks(std::max<size_t>((size_t)I * J, (size_t)K), 256), 256, 0, st>>>(
-      I, J, K, raw, rawlev, pitraw, Mu, Mv, rowT, rAd, levT, colT, rS, lS, cS, g->beta2);
+      I, J, K, raw, rawlev, pitraw, Mu, Mv, rowT, rAd, levT, (float4*)(base + kOffDs3), colT, rS, lS, cS, g->beta2);
   CUDA_TRY(cudaGetLastError());
   }
   G.I = I; G.J = J; G.K = K;
@@ -1650,11 +1665,12 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   G.adl = (T)(kA * g->dlam);
   G.rvn = rowT + 12 * rS; G.rvs = rowT + 13 * rS; G.Af = rowT + 14 * rS; G.Ac = rowT + 15 * rS;
   G.rAd = rAd;
+  G.ds3 = (const float4*)(base + kOffDs3);
   G.lev = levT + 7 * lS;
   G.items = (const int4*)(base + kOffRowL);
   double* ubar = (double*)(base + kOffBar);
   double* vbar = (double*)(base + kOffBar + kColB);
-  agcm::k_vsum<T><<<nblocks((size_t)I * J, 256), 256, 0, st>>>(G, (const T*)U, (const T*)V, ubar, vbar);
+  agcm::k_vsum<T><<<dim3(nblocks((size_t)I * J, 256), 2), 256, 0, st>>>(G, (const T*)U, (const T*)V, ubar, vbar);
   const void* xs[4] = {U, V, Phi, pi};
   const void* none[4] = {nullptr, nullptr, nullptr, nullptr};
   void* out[4] = {tU, tV, tPhi, tpi};

@@ -54,6 +54,7 @@ struct Geom {
   const int* filtV; // V rows
   int nfU, nfV;
   const double* dsd;  // dsigma_k in FP64 (column integral of the divergence)
+  const float4* ds3;  // dsigma_k as the sum of three FP32 parts x + y + z (K)
   const double* shd;  // half levels sigma_hat_h in FP64 (K+1)
   const double* Ad;   // A_j in FP64 (J)     (diagnostics)
   const double* Avd;  // Av_j in FP64 (J-1)  (diagnostics)
@@ -89,5 +90,29 @@ __device__ __forceinline__ T ldg(const T* p) {
 // sqrt in the kernel's type
 __device__ __forceinline__ double sqrt_t(double x) { return sqrt(x); }
 __device__ __forceinline__ float sqrt_t(float x) { return sqrtf(x); }
+
+// a + b = s + e exactly (TwoSum, Knuth), and a sum of FP32 numbers in three
+// FP32 terms.  Products that go in are formed by __fmul_rn: a multiply-add
+// made of one of these additions would not be exact.
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = a + b;
+  const float bb = s - a;
+  e = (a - (s - bb)) + (b - bb);
+}
+struct Sum3 {
+  float s = 0.f, c = 0.f, d = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    float e, f;
+    two_sum(s, x, s, e);
+    two_sum(c, e, c, f);
+    d += f;
+  }
+  __device__ __forceinline__ void add_low(float x) {  // x below 2^-20 of the sum
+    float f;
+    two_sum(c, x, c, f);
+    d += f;
+  }
+  __device__ __forceinline__ double total() const { return (double)s + ((double)c + (double)d); }
+};
 
 }  // namespace agcm

@@ -399,22 +399,56 @@ __global__ void __launch_bounds__(kTileX, sizeof(T) == 4 ? (PART == 2 ? AGCM_FUS
                                                 pio, Ubar_o, Vbar_o, Ubar_b, Vbar_b, cdt);
 }
 
-// Vertical means Ubar = sum_k dsigma_k U_k, Vbar likewise (FP64), of a state.
+// Vertical means Ubar = sum_k dsigma_k U_k, Vbar likewise (FP64), of a state:
+// one thread per column and field.  FP32 states: GB300 issues FP64, and the
+// conversion to it, at 1/64 of the FP32 rate (one conversion and one
+// multiply-add per value took 231 us at 1440x720x30, where reading the values
+// takes 37), so the products and the sum run in FP32 without loss: dsigma as
+// three FP32 parts, products split exactly by a multiply-add, and a sum of
+// three terms (TwoSum, Knuth; SumK with K = 3, Ogita, Rump and Oishi 2005)
+// that drops nothing above 2^-60 of the largest term, and one FP64 addition
+// per column rounds it: closer to the exact mean than 30 FP64 additions.
+// 109 us at 1440x720x30 (34 operations a value: FP32 issue), 35 at 720x360x30 (63).
+// Columns with a value or partial product out of the range in which that
+// holds (above 2^100, or all below 2^-60, or not finite) are summed in FP64.
+constexpr int kVsumLev = 6;  // levels loaded together
 template <class T>
 __global__ void __launch_bounds__(256) k_vsum(Geom<T> g, const T* __restrict__ U, const T* __restrict__ V,
                                               double* __restrict__ Ubar, double* __restrict__ Vbar) {
   const int I = g.I, J = g.J, K = g.K;
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= I * J) return;
-  const size_t plane = (size_t)J * I, vplane = (size_t)(J - 1) * I;
-  double su = 0.0, sv = 0.0;
-  const bool hasV = n < (J - 1) * I;
-  for (int k = 0; k < K; ++k) {
-    su += g.dsd[k] * (double)U[(size_t)k * plane + n];
-    if (hasV) sv += g.dsd[k] * (double)V[(size_t)k * vplane + n];
+  const bool vf = blockIdx.y != 0;  // field V
+  const size_t plane = (size_t)(vf ? J - 1 : J) * I;
+  if ((size_t)n >= plane) return;
+  const T* __restrict__ F = (vf ? V : U) + n;
+  double* const out = (vf ? Vbar : Ubar) + n;
+  if constexpr (sizeof(T) == 4) {
+    Sum3 a;
+    float big = 0.f;
+    for (int k0 = 0; k0 < K; k0 += kVsumLev) {
+      float x[kVsumLev];
+#pragma unroll
+      for (int q = 0; q < kVsumLev; ++q) x[q] = k0 + q < K ? ldg(F + (size_t)(k0 + q) * plane) : 0.f;
+#pragma unroll
+      for (int q = 0; q < kVsumLev; ++q) {
+        const float4 w = g.ds3[min(k0 + q, K - 1)];
+        const float p = __fmul_rn(w.x, x[q]), r = __fmul_rn(w.y, x[q]);
+        a.add(p);
+        a.add_low(fmaf(w.x, x[q], -p));
+        a.add_low(r);
+        a.d += fmaf(w.y, x[q], -r) + w.z * x[q];
+        big = fmaxf(big, fabsf(x[q]));
+      }
+    }
+    const double t = a.total();
+    if (big < 1.2e30f && (big > 8.7e-19f || big == 0.f) && t - t == 0.0) {
+      *out = t;
+      return;
+    }
   }
-  Ubar[n] = su;
-  if (hasV) Vbar[n] = sv;
+  double s = 0.0;
+  for (int k = 0; k < K; ++k) s += g.dsd[k] * (double)F[(size_t)k * plane];
+  *out = s;
 }
 
 }  // namespace agcm
