@@ -15,14 +15,14 @@
 //                 gathered from the tendencies that read them, the
 //                 transposed prefix / suffix scans and the adjoint Dbar_k of
 //                 D_k.
-//   k_adj_rows    one row segment per block, levels in a loop: the adjoints of
-//                 the mass fluxes F = P^u U, P^v V, of G = U / P^u, V / P^v,
-//                 Phi / P and of U, V through the Coriolis pair, each gathered
-//                 from the tendency points that read it (from factors staged
-//                 in shared memory), then the chain F = P U, G = F / P back to
-//                 U, V, Phi and the level sums of the adjoints of the 2-D
-//                 factors.  k_adj_gather does the same through L1 for the rows
-//                 whose strides reach past a row segment's halo.
+//   k_adj_rows    one row segment per block, levels in a loop over rows staged
+//                 in shared memory: the adjoints of the mass fluxes F = P^u U,
+//                 P^v V, of G = U / P^u, V / P^v, Phi / P and of U, V through
+//                 the Coriolis pair, each gathered from the tendency points
+//                 that read it, then the chain F = P U, G = F / P back to U, V,
+//                 Phi and the level sums of the adjoints of the 2-D factors.
+//                 k_adj_gather does the same through L1 for the rows whose
+//                 strides reach past a row segment's halo.
 //   k_adj_colstate  m^u, m^v are stride-1 means of m: the adjoint of pi.
 //
 // The transposed stencil.  Every advection term is a face flux Z times the
@@ -43,6 +43,7 @@
 #pragma once
 #include "agcm_common.cuh"
 #include "agcm_phases.cuh"
+#include "agcm_row.cuh"
 
 namespace agcm {
 
@@ -491,7 +492,7 @@ __device__ __forceinline__ P* opaque(P* p) {
 // rows whose strides are small, and this kernel the nrows rows in `rows`.
 // The level sums of the 2-D factors' adjoints are written per chunk to
 // part[3][nchunks][nrows][I] and added in chunk order by k_adj_fold.
-constexpr int kAdjLevChunk = 4;
+constexpr int kAdjLevChunk = 1;  // few rows: the more chunks the shorter the launch (256x128x30: 282 against 297 us a reverse step with 4)
 // Offsets in row j (stride M = Mu_j):  a0 = i - (M-1)/2, b0 = i + (M+1)/2 =
 // a0 + M (the pair whose face flux is F^u(i) for a Phi point, one of the two
 // for a U point), a1 = i - (M+1)/2, b1 = i + (M-1)/2 = a1 + M (the other U
@@ -740,334 +741,417 @@ __global__ void __launch_bounds__(256) k_adj_fold(Geom<T> g, const int* __restri
 }
 
 // ---------------------------------------------------------------------------
-// Row-segment form of k_adj_gather.  A CTA of kAdjRowB threads takes one row
-// j and a segment of `own` columns with a halo of H columns on each side
-// (H = the widest offset at which the row's transposed stencil reads:
-// max(M_j, Mv_j, (Mv_{j-1} + 1) / 2)).  Per level, every thread stages the
-// pointwise factors of its column (y / P, x / P and P x of the U, Phi and V
-// points of rows j-1, j, j+1, and three combinations for the Coriolis pair)
-// into shared memory, then the owning threads gather the transposed stencil
-// from there: each factor is formed once per CTA instead of once per reader,
-// and every neighbour read is a shared-memory load at a fixed offset (the
-// seam of the periodic row is resolved when staging).  The vertical
-// neighbours are the thread's own column at levels k-1 and k+1: the previous
-// level's raw values are kept in registers and the next level's are loaded
-// one iteration ahead (they are also what the thread stages next).  Two
-// shared buffers alternate between levels with one barrier per level: the
-// buffer a level writes was last read two levels before, and every thread has
-// passed the barrier between.
-constexpr int kAdjRowB = 256;
-constexpr int kAdjRowMaxH = 48;
+// Row-segment form of k_adj_gather.  A CTA of at most kRowB threads takes one
+// row j and a segment of own columns with a halo of H columns on each side (H
+// no less than the widest offset at which the row's transposed stencil reads:
+// max(M_j, Mv_j, (Mv_{j-1} + 1) / 2)), and streams the levels from the top.
+// Per level, 28 rows arrive in a ring of shared-memory slots by asynchronous
+// copies issued a ring's length ahead, seven a thread: x and ybar (U, Phi, V
+// at j-1, j, j+1), psi, Dbar and W at j, j+1, the adjoint of Phi from the
+// column pass, and the stage sum (of the level above, which this level
+// completes).  Every thread forms the pointwise factors of its column, h =
+// -ybar / (2 A P), G = x / P and the face fluxes, and publishes the sixteen
+// that its neighbours read; after one barrier the columns gather the
+// transposed stencil from there.  The vertical pairs of a level need h and G
+// of the level below: its own column's terms are added one iteration later,
+// when the level is written.
+//
+// As in the forward kernel the areas are multiplied out: the face fluxes carry
+// their face lengths, h the area (and for the U and V points the half of
+// their face means), so a face sum is a plain chain of multiply-adds, about
+// 150 operations a point and level where the terms formed one by one took
+// 240.  M1: all strides of the row are 1, which makes half of the partner
+// reads the own or an already read value.
+//
+// Bound by shared-memory reads (their pipe is busy 62 % of the cycles) and the
+// latency left at 12 warps an SM: 187 us a launch at 720x360x30 FP32 (ncu,
+// cold caches), 377 thread instructions a point, against 250 us and 810 for
+// 256-thread CTAs that loaded their rows into registers a level ahead; 200 at
+// two ring slots, 215 with four CTAs an SM at 128 registers.  FP64: 3.0 ms.
 enum AdjRowArr {
-  kqP0, kGs0, kqU0, kGu0, kFl0, kqV0, kGv0, kFt0,  // row j, V row j
-  kqP1, kGs1, kqU1, kGu1, kFl1, kqV1, kGv1, kFt1,  // row j+1, V row j+1
-  kqPm, kGsm, kqUm, kGum, kqVm, kGvm, kFtm,        // row j-1, V row j-1
-  kVs, kyC, kcUs,                                  // Coriolis combinations
-  kAdjRowNA
+  kpHP, kpGs, kpHU, kpGu, kpFL, kpHV, kpGv, kpFT,  // row j, V row j
+  kpFLs, kpHVm, kpGvm, kpFTm,                       // F^u of row j+1, V row j-1
+  kpYC, kpVs, kpCU, kpEU,                           // Coriolis combinations; U pairs of rows j, j+1
+  kAdjPub
+};
+constexpr int kAdjRaw = 28;
+template <class T>
+struct AdjRing {
+  static constexpr int R = sizeof(T) == 4 ? 4 : 2;
 };
 
 // Halo of row j's adjoint stencil (Mv = 0 without a V row j, Mvm = 0 without
-// a V row j-1) and its segments: nseg segments of at most S owned columns.
+// a V row j-1), a multiple of four columns.
 __host__ __device__ inline int adj_row_halo(int M, int Mv, int Mvm) {
   int h = M > Mv ? M : Mv;
   const int hm = (Mvm + 1) / 2;
   if (hm > h) h = hm;
-  return h < 1 ? 1 : h;
-}
-__host__ __device__ inline void adj_row_segments(int I, int H, int* nseg, int* S) {
-  const int w = kAdjRowB - 2 * H;
-  *nseg = (I + w - 1) / w;
-  *S = (I + *nseg - 1) / *nseg;
+  return (h + 3) & ~3;
 }
 template <class T>
-constexpr size_t adj_row_smem() {
-  return (size_t)2 * kAdjRowNA * kAdjRowB * sizeof(T);
+constexpr size_t adj_row_smem(int K) {
+  return sizeof(T) * ((size_t)kRowB * (AdjRing<T>::R * kAdjRaw + 2 * kAdjPub) + K + 64);
 }
 
 template <class T>
-#ifndef AGCM_ADJROWB
-#define AGCM_ADJROWB 2
-#endif
-__global__ void __launch_bounds__(kAdjRowB, sizeof(T) == 4 ? AGCM_ADJROWB : 1) k_adj_rows(
-    Geom<T> g, const int* __restrict__ items, const T* __restrict__ U, const T* __restrict__ V,
-    const T* __restrict__ Phi, ColState<T> cs, const T* __restrict__ W, const T* __restrict__ psi,
-    const T* __restrict__ Db, const T* __restrict__ aPhi, const T* __restrict__ arPcol, const T* __restrict__ yU,
-    const T* __restrict__ yV, const T* __restrict__ yPhi, AdjM<T> m, AdjOut<T> o) {
-  extern __shared__ __align__(16) unsigned char adj_smem[];
-  T* const sm = reinterpret_cast<T*>(adj_smem);
+struct AdjRowArgs {
+  const T *U, *V, *Phi;      // x
+  const T *yU, *yV, *yPhi;   // ybar
+  const T *W, *psi, *Db, *aPhi, *arPcol;
+  const T *rU, *rV, *rPhi;   // the array added to: stage sum or the output itself; null: none
+  const int4* items;         // kind << 24 | row j, first own column, own columns, halo; kind 1: all strides 1
+  int vec;                   // 1: every row is 16-byte aligned
+};
+
+template <class T, bool M1>
+__device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs, const AdjRowArgs<T>& a,
+                                        const AdjM<T>& m, const AdjOut<T>& o, const int4 item, unsigned char* smem) {
+  constexpr int R = AdjRing<T>::R, NTP = kRowB;
   const int I = g.I, J = g.J, K = g.K;
-  const int item = ldg(items + blockIdx.x);
-  const int j = item >> 8, seg = item & 255;
-  const bool hasS = j < J - 1, hasN = j > 0, hasSS = j + 1 < J - 1;
-  const int M = ldg(g.Mu + j), Mv = hasS ? ldg(g.Mv + j) : 0, Mvm = hasN ? ldg(g.Mv + j - 1) : 0;
-  const int H = adj_row_halo(M, Mv, Mvm);
-  int nseg, S;
-  adj_row_segments(I, H, &nseg, &S);
-  const int s0 = seg * S, own = min(S, I - s0);
+  const int j = item.x & 0xffffff, c0 = item.y, own = item.z, H = item.w;
+  const bool hasS = M1 || j < J - 1, hasN = M1 || j > 0, hasSS = j + 1 < J - 1;
+  const int M = M1 ? 1 : g.Mu[j], Mv = M1 ? 1 : (hasS ? g.Mv[j] : 1), Mvm = M1 ? 1 : (hasN ? g.Mv[j - 1] : 1);
+  const int NT = own + 2 * H, NTW = (NT + 31) & ~31;
   const int t = threadIdx.x;
-  const bool active = t < own + 2 * H, owner = t >= H && t < H + own;
-  int c = (s0 - H + t) % I;
-  if (c < 0) c += I;
+  if (t >= NTW) leave();  // whole warps past the segment
+  const bool owner = t >= H && t < H + own;
+  int cstart = c0 - H;
+  while (cstart < 0) cstart += I;
+  int c = cstart + t;
+  while (c >= I) c -= I;
+  T* const ring = reinterpret_cast<T*>(smem);
+  T* const pub = ring + (size_t)R * kAdjRaw * NTP;
+  T* const s_rds = pub + (size_t)2 * kAdjPub * NTP;  // 1 / dsigma_k
+  for (int k = t; k < K; k += NTW) s_rds[k] = T(2) * g.r2ds[k];
   // element offsets fit 32 bits: nlon * nlat * nlev <= 4e9
   const unsigned plane = (unsigned)J * (unsigned)I, vplane = (unsigned)(J - 1) * (unsigned)I;
   const unsigned r2 = (unsigned)j * (unsigned)I;
-  // row tables
-  const T zf = ldg(g.zf + j), r2A = ldg(g.r2A + j), rdx = ldg(g.rdx + j), f0 = ldg(g.f0 + j),
-          cota = ldg(g.cota + j);
-  const T r2AN = hasN ? ldg(g.r2A + j - 1) : T(0), r2AS = hasS ? ldg(g.r2A + j + 1) : T(0);
-  const T yvS = hasS ? ldg(g.yv + j) : T(0), yvN = hasN ? ldg(g.yv + j - 1) : T(0),
-          yvSS = hasSS ? ldg(g.yv + j + 1) : T(0);
-  const T cnS = hasS ? ldg(g.cn + j) : T(0), csN = hasN ? ldg(g.cs + j - 1) : T(0);
-  const T zfvS = hasS ? ldg(g.zfv + j) : T(0), r2AvS = hasS ? ldg(g.r2Av + j) : T(0);
-  const T r2AvSS = hasSS ? ldg(g.r2Av + j + 1) : T(0);
-  const T zfvN = hasN ? ldg(g.zfv + j - 1) : T(0), r2AvN = hasN ? ldg(g.r2Av + j - 1) : T(0);
-  const T svS = hasS ? ldg(g.sv + j) : T(0), rdyS = hasS ? ldg(g.rdy + j) : T(0),
-          rdyS1 = hasS ? ldg(g.rdy + j + 1) : T(0);
-  const T f0S = hasS ? ldg(g.f0 + j + 1) : T(0), cotaS = hasS ? ldg(g.cota + j + 1) : T(0);
-  const T rady = g.rady;
-  // offsets of the stencil from an owned column
+
+  // Staged rows of a level: 3 f + r, field f = U, Phi, V, yU, yPhi, yV, row r =
+  // j-1, j, j+1; then 18, 19 psi, 20, 21 Dbar, 22, 23 W at j, j+1, 24 the
+  // adjoint of Phi, 25..27 the stage sum's U, Phi, V of the level above.  A
+  // quarter of the threads each: a thread one chunk of four columns of seven
+  // rows.  Rows outside the grid are zeros.
+  const int tr = NTW >> 2, cr = t / tr, cc = 4 * (t - cr * tr);
+  int c4 = cstart + cc;
+  while (c4 >= I) c4 -= I;
+  const int sw = min(I - c4, 4);  // the first element past the periodic seam
+  const int jr = cr < 3 ? j + cr - 1 : j;
+  const bool in = cc < NT, ok3 = in && jr >= 0 && jr < J, okv = in && jr >= 0 && jr < J - 1;
+  const bool oks = in && hasS, okr = in && cc >= H && cc < H + own;
+  const unsigned so = (unsigned)(ok3 ? jr : j) * (unsigned)I + (unsigned)c4, ro = r2 + (unsigned)c4;
+  const unsigned ring_s = smem_addr(ring);
+  auto chunk = [&](auto vec, int row, int s, const T* src, bool ok) __attribute__((always_inline)) {
+    const unsigned d = ring_s + (unsigned)(((s * kAdjRaw + row) * NTP + cc) * (int)sizeof(T));
+    if constexpr (decltype(vec)::value) {
+#pragma unroll
+      for (int e = 0; e < 4; e += 16 / (int)sizeof(T)) copy16_g2s(d + e * sizeof(T), src + e, true, ok);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        copy_elem_g2s<sizeof(T)>(d + e * sizeof(T), src + (e < sw ? e : e - I), true, ok);
+    }
+  };
+  auto issue_form = [&](auto vec, int k, int s) __attribute__((always_inline)) {
+    const unsigned p3 = (unsigned)k * plane, pv = (unsigned)k * vplane;
+    if (cr < 3) {
+      const unsigned ov = pv + (okv ? so : 0u);
+      chunk(vec, cr, s, a.U + (p3 + so), ok3);
+      chunk(vec, 3 + cr, s, a.Phi + (p3 + so), ok3);
+      chunk(vec, 6 + cr, s, a.V + ov, okv);
+      chunk(vec, 9 + cr, s, a.yU + (p3 + so), ok3);
+      chunk(vec, 12 + cr, s, a.yPhi + (p3 + so), ok3);
+      chunk(vec, 15 + cr, s, a.yV + ov, okv);
+      if (a.rU && k > 0) {  // quarter cr: field U, Phi, V
+        const T* const r = cr == 0 ? a.rU : (cr == 1 ? a.rPhi : a.rV);
+        const unsigned q = cr == 2 ? (hasS ? pv - vplane + ro : 0u) : p3 - plane + ro;
+        chunk(vec, 25 + cr, s, r + q, okr && (cr < 2 || hasS));
+      }
+    } else {
+      const unsigned q = p3 + ro, qs = oks ? q + I : q;
+      chunk(vec, 18, s, a.psi + q, in);
+      chunk(vec, 19, s, a.psi + qs, oks);
+      chunk(vec, 20, s, a.Db + q, in);
+      chunk(vec, 21, s, a.Db + qs, oks);
+      chunk(vec, 22, s, a.W + q, in && k > 0);  // W_0 = 0 is not stored
+      chunk(vec, 23, s, a.W + qs, oks && k > 0);
+      chunk(vec, 24, s, a.aPhi + q, in);
+    }
+  };
+  auto issue_level = [&](int k, int s) __attribute__((always_inline)) {
+    if (a.vec)
+      issue_form(std::true_type{}, k, s);
+    else
+      issue_form(std::false_type{}, k, s);
+  };
+  for (int s = 0; s < R; ++s) {
+    if (s < K) issue_level(s, s);
+    copy_commit();
+  }
+
+  // ---- the factors of the own column, rows j-1, j, j+1 (index r)
+  T rP[3], rPu[3], rPv[3], kP[3], kU[3], kV[3], b[3], aF[2];
+  T Pu0 = 0, Pv0 = 0;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const int jj = j - 1 + r;
+    const bool ok = jj >= 0 && jj < J, kv = jj >= 0 && jj < J - 1;
+    const unsigned n = ok ? (unsigned)jj * (unsigned)I + (unsigned)c : r2 + (unsigned)c;
+    rP[r] = ok ? ldg(cs.rP + n) : T(0);
+    rPu[r] = ok ? ldg(cs.rPu + n) : T(0);
+    kP[r] = ok ? -ldg(g.r2A + jj) * rP[r] : T(0);
+    kU[r] = ok ? T(-0.5) * ldg(g.r2A + jj) * rPu[r] : T(0);
+    const T Pu = ok && r > 0 ? ldg(cs.Pu + n) : T(0);
+    if (r == 1) Pu0 = Pu;
+    // row j+1's flux carries V row j's face length
+    if (r > 0) aF[r - 1] = r == 1 ? ldg(g.zf + j) * Pu : (hasS ? ldg(g.zfv + j) * Pu : T(0));
+    rPv[r] = kv ? ldg(cs.rPv + n) : T(0);
+    kV[r] = kv ? T(-0.5) * ldg(g.r2Av + jj) * rPv[r] : T(0);
+    const T Pv = kv ? ldg(cs.Pv + n) : T(0);
+    if (r == 1) Pv0 = Pv;
+    b[r] = kv ? ldg(g.yv + jj) * Pv : T(0);
+  }
+  // ---- row scalars
+  const T zf = g.zf[j], rdx = g.rdx[j], f0 = g.f0[j], cota = g.cota[j], rady = g.rady;
+  const T zS = hasS ? g.zfv[j] : T(0), zN = hasN ? g.zfv[j - 1] : T(0), rm = M1 ? T(1) : zS / zf;
+  const T f1 = hasS ? g.f0[j + 1] : T(0), cota1 = hasS ? g.cota[j + 1] : T(0);
+  const T cn = hasS ? g.cn[j] : T(0), csn = hasN ? g.cs[j - 1] : T(0), yvS = hasS ? g.yv[j] : T(0);
+  const T nr2A = -g.r2A[j], nr2Av = hasS ? -g.r2Av[j] : T(0);
+  const T s0 = hasS ? g.sv[j] * g.rdy[j] : T(0), s1 = hasS ? g.sv[j] * g.rdy[j + 1] : T(0);
+  const T A = T(0.5) / g.r2A[j], Av = hasS ? T(0.5) / g.r2Av[j] : T(0);
+  // ---- offsets of the stencil from the own column.  A halo thread's partner
+  // may lie outside the segment: such reads land in the neighbouring arrays
+  // and feed only results that nobody writes.
   const int oa0 = -(M - 1) / 2, ob0 = (M + 1) / 2, oa1 = -(M + 1) / 2, ob1 = (M - 1) / 2;
-  const int ocS = -(Mv - 1) / 2, odS = (Mv + 1) / 2, ofEv = (Mv - 1) / 2, ofWv = -(Mv + 1) / 2;
+  const int ocS = -(Mv - 1) / 2, odS = (Mv + 1) / 2, ofE = (Mv - 1) / 2, ofW = -(Mv + 1) / 2;
   const int ocN = -(Mvm - 1) / 2, odN = (Mvm + 1) / 2;
-  const int a0g = wrapi(c + oa0, I), b0g = wrapi(c + ob0, I), cp = wrapi(c + 1, I);
-  // the 2-D factors of the staged column c, rows j-1, j, j+1 (V rows alike)
-  const T rP0 = ldg(cs.rP + r2 + c), rPu0 = ldg(cs.rPu + r2 + c), Pu0 = ldg(cs.Pu + r2 + c);
-  const T rP1 = hasS ? ldg(cs.rP + r2 + I + c) : T(0), rPu1 = hasS ? ldg(cs.rPu + r2 + I + c) : T(0),
-          Pu1 = hasS ? ldg(cs.Pu + r2 + I + c) : T(0);
-  const T rPm = hasN ? ldg(cs.rP + r2 - I + c) : T(0), rPum = hasN ? ldg(cs.rPu + r2 - I + c) : T(0);
-  const T rPv0 = hasS ? ldg(cs.rPv + r2 + c) : T(0), Pv0 = hasS ? ldg(cs.Pv + r2 + c) : T(0);
-  const T rPv1 = hasSS ? ldg(cs.rPv + r2 + I + c) : T(0), Pv1 = hasSS ? ldg(cs.Pv + r2 + I + c) : T(0);
-  const T rPvm = hasN ? ldg(cs.rPv + r2 - I + c) : T(0), Pvm = hasN ? ldg(cs.Pv + r2 - I + c) : T(0);
-  // raw values of column c at one level: row j, j+1, j-1 (Phi, U), V rows j, j+1, j-1
-  struct Raw {
-    T yP0, P0, yU0, U0, yV0, V0, yP1, P1, yU1, U1, yV1, V1, yPm, Pm, yUm, Um, yVm, Vm;
-  };
-  auto load_raw = [&](int k, Raw& r) {
-    const unsigned r3 = (unsigned)k * plane + r2 + c, rv = (unsigned)k * vplane + r2 + c;
-    r.yP0 = ldg(yPhi + r3);
-    r.P0 = ldg(Phi + r3);
-    r.yU0 = ldg(yU + r3);
-    r.U0 = ldg(U + r3);
-    r.yV0 = hasS ? ldg(yV + rv) : T(0);
-    r.V0 = hasS ? ldg(V + rv) : T(0);
-    r.yP1 = hasS ? ldg(yPhi + r3 + I) : T(0);
-    r.P1 = hasS ? ldg(Phi + r3 + I) : T(0);
-    r.yU1 = hasS ? ldg(yU + r3 + I) : T(0);
-    r.U1 = hasS ? ldg(U + r3 + I) : T(0);
-    r.yV1 = hasSS ? ldg(yV + rv + I) : T(0);
-    r.V1 = hasSS ? ldg(V + rv + I) : T(0);
-    r.yPm = hasN ? ldg(yPhi + r3 - I) : T(0);
-    r.Pm = hasN ? ldg(Phi + r3 - I) : T(0);
-    r.yUm = hasN ? ldg(yU + r3 - I) : T(0);
-    r.Um = hasN ? ldg(U + r3 - I) : T(0);
-    r.yVm = hasN ? ldg(yV + rv - I) : T(0);
-    r.Vm = hasN ? ldg(V + rv - I) : T(0);
-  };
-  // the owner's other inputs at one level: psi and Dbar at the columns a0,
-  // b0, i of row j and i of row j+1, and the adjoint of Phi from the column pass
-  struct Own {
-    T psa, psb, psc, pss, Dba, Dbb, Dbc, Dbs, aPh;
-  };
-  auto load_own = [&](int k, Own& w) {
-    const unsigned r3 = (unsigned)k * plane + r2;
-    w.psa = ldg(psi + r3 + a0g);
-    w.psb = ldg(psi + r3 + b0g);
-    w.psc = ldg(psi + r3 + c);
-    w.pss = hasS ? ldg(psi + r3 + I + c) : T(0);
-    w.Dba = ldg(Db + r3 + a0g);
-    w.Dbb = ldg(Db + r3 + b0g);
-    w.Dbc = ldg(Db + r3 + c);
-    w.Dbs = hasS ? ldg(Db + r3 + I + c) : T(0);
-    w.aPh = ldg(aPhi + r3 + c);
-  };
-  Raw cur{}, nxt{};
-  Own ocur{}, onxt{};
-  if (active) load_raw(0, cur);
-  if (owner) load_own(0, ocur);
-  // the array the owner reads back and adds to: the stage sum, or the
-  // output itself when accumulating
-  const T* const rmwU = o.sU ? o.rU : (o.accumulate ? o.oU : nullptr);
-  const T* const rmwP = o.sU ? o.rPhi : (o.accumulate ? o.oPhi : nullptr);
-  const T* const rmwV = o.sU ? o.rV : (o.accumulate ? o.oV : nullptr);
-  // own column at level k-1 (row j, V row j)
-  T yPp = 0, Pp = 0, yUp = 0, Up = 0, yVp = 0, Vp = 0;
-  // W at level k (rows j, j+1; columns i, i+1), loaded one level ahead
-  T Wt = 0, Wtp = 0, Wts = 0;
-  T aPu = 0, arPu = 0, aPv = 0, arPv = 0, arP = owner ? ldg(arPcol + r2 + c) : T(0);
-  const T rPc = rP0, rPuc = rPu0, Puc = Pu0, rPvc = rPv0, Pvc = Pv0;
-  for (int k = 0; k < K; ++k) {
-    T* const b = sm + (size_t)(k & 1) * kAdjRowNA * kAdjRowB;
-    // this level's values to add to, loaded before the staging so that the
-    // load is in flight across it
-    T accU = 0, accP = 0, accV = 0;
-    if (owner && rmwU) {
-      const unsigned q = (unsigned)k * plane + r2 + c;
-      accU = rmwU[q];
-      accP = rmwP[q];
-      if (hasS) accV = rmwV[(unsigned)k * vplane + r2 + c];
-    }
-    if (active) {
-      T* const q = b + t;
-      const Raw& r = cur;
-      const T Gu0 = r.U0 * rPu0, Gu1 = r.U1 * rPu1;
-      q[kqP0 * kAdjRowB] = r.yP0 * rP0;
-      q[kGs0 * kAdjRowB] = r.P0 * rP0;
-      q[kqU0 * kAdjRowB] = r.yU0 * rPu0;
-      q[kGu0 * kAdjRowB] = Gu0;
-      q[kFl0 * kAdjRowB] = Pu0 * r.U0;
-      q[kqV0 * kAdjRowB] = r.yV0 * rPv0;
-      q[kGv0 * kAdjRowB] = r.V0 * rPv0;
-      q[kFt0 * kAdjRowB] = Pv0 * r.V0;
-      q[kqP1 * kAdjRowB] = r.yP1 * rP1;
-      q[kGs1 * kAdjRowB] = r.P1 * rP1;
-      q[kqU1 * kAdjRowB] = r.yU1 * rPu1;
-      q[kGu1 * kAdjRowB] = Gu1;
-      q[kFl1 * kAdjRowB] = Pu1 * r.U1;
-      q[kqV1 * kAdjRowB] = r.yV1 * rPv1;
-      q[kGv1 * kAdjRowB] = r.V1 * rPv1;
-      q[kFt1 * kAdjRowB] = Pv1 * r.V1;
-      q[kqPm * kAdjRowB] = r.yPm * rPm;
-      q[kGsm * kAdjRowB] = r.Pm * rPm;
-      q[kqUm * kAdjRowB] = r.yUm * rPum;
-      q[kGum * kAdjRowB] = r.Um * rPum;
-      q[kqVm * kAdjRowB] = r.yVm * rPvm;
-      q[kGvm * kAdjRowB] = r.Vm * rPvm;
-      q[kFtm * kAdjRowB] = Pvm * r.Vm;
-      // V(j-1) + V(j); cn yV(j) + cs yV(j-1); the Coriolis factor yU fs of rows j, j+1
-      q[kVs * kAdjRowB] = r.V0 + r.Vm;
-      q[kyC * kAdjRowB] = cnS * r.yV0 + csN * r.yVm;
-      q[kcUs * kAdjRowB] = r.yU0 * (f0 + Gu0 * cota) + (hasS ? r.yU1 * (f0S + Gu1 * cotaS) : T(0));
-      if (k + 1 < K) load_raw(k + 1, nxt);
-    }
-    if (owner && k + 1 < K) load_own(k + 1, onxt);
-    T Wb = 0, Wbp = 0, Wbs = 0;
-    if (owner && k + 1 < K) {
-      const unsigned wq = (unsigned)(k + 1) * plane + r2;
-      Wb = ldg(W + wq + c);
-      Wbp = ldg(W + wq + cp);
-      Wbs = hasS ? ldg(W + wq + I + c) : T(0);
-    }
-    __syncthreads();
+
+  // ---- carries: sums over the levels, and of the level above: h / dsigma and
+  // G, the adjoints so far, x and -ybar / (2 A) / dsigma (late terms)
+  T aPu = 0, arPu = 0, aPv = 0, arPv = 0, arP = owner ? ldg(a.arPcol + r2 + c) : T(0);
+  T hvU = 0, hvP = 0, hvV = 0, GuP = 0, GsP = 0, GvP = 0;
+  T bU = 0, bP = 0, bV = 0, xU = 0, xP = 0, xV = 0, yrU = 0, yrP = 0, yrV = 0;
+  const bool rmw = a.rU != nullptr;
+  unsigned q3 = r2 + (unsigned)c, qv = q3;  // the own column at the level being written
+  auto write = [&](T accU, T accP, T accV) __attribute__((always_inline)) {
+    const T vU = o.scale * bU, vP = o.scale * bP, vV = o.scale * bV;
     if (owner) {
-      const T* const L = b + t;
-      auto A = [&](int arr, int off) { return L[arr * kAdjRowB + off]; };
-      const unsigned r3 = (unsigned)k * plane + r2, rv = (unsigned)k * vplane + r2;
-      const T r2ds = ldg(g.r2ds + k);
-      const T r2dsU = k > 0 ? ldg(g.r2ds + k - 1) : T(0), r2dsD = k + 1 < K ? ldg(g.r2ds + k + 1) : T(0);
-      const bool up = k > 0, dn = k + 1 < K;
-      // own column at levels k and k+1
-      const T yPc = cur.yP0, Pc = cur.P0, yUc = cur.yU0, Uc = cur.U0, yVc = cur.yV0, Vc = cur.V0;
-      const T yPn = dn ? nxt.yP0 : T(0), Pn = dn ? nxt.P0 : T(0), yUn = dn ? nxt.yU0 : T(0),
-              Un = dn ? nxt.U0 : T(0), yVn = dn ? nxt.yV0 : T(0), Vn = dn ? nxt.V0 : T(0);
-      // ---------------- U point and F^u
-      const T Fla0 = A(kFl0, oa0), Flb0 = A(kFl0, ob0), Fla1 = A(kFl0, oa1), Flb1 = A(kFl0, ob1);
-      T aFl = -zf * r2A * (A(kqP0, oa0) * A(kGs0, ob0) - A(kqP0, ob0) * A(kGs0, oa0));
-      aFl -= T(0.5) * zf * r2A *
-             ((A(kqU0, oa0) * A(kGu0, ob0) - A(kqU0, ob0) * A(kGu0, oa0)) +
-              (A(kqU0, oa1) * A(kGu0, ob1) - A(kqU0, ob1) * A(kGu0, oa1)));
-      if (hasS) aFl -= T(0.5) * zfvS * r2AvS * (A(kqV0, ocS) * A(kGv0, odS) - A(kqV0, odS) * A(kGv0, ocS));
-      if (hasN) aFl -= T(0.5) * zfvN * r2AvN * (A(kqVm, ocN) * A(kGvm, odN) - A(kqVm, odN) * A(kGvm, ocN));
-      aFl += rdx * (ocur.Dba - ocur.Dbb);
-      const T FtS = A(kFt0, 0), FtSp = A(kFt0, 1), FtN = A(kFtm, 0), FtNp = A(kFtm, 1);
-      const T ZEu = T(0.5) * zf * (Flb1 + Flb0), ZWu = T(0.5) * zf * (Fla1 + Fla0);
-      const T YSu = T(0.5) * yvS * (FtS + FtSp), YNu = T(0.5) * yvN * (FtN + FtNp);
-      const T WTu = up ? T(0.5) * (Wt + Wtp) : T(0), WBu = dn ? T(0.5) * (Wb + Wbp) : T(0);
-      const T Cu = A(kyC, 0) + A(kyC, 1);
-      T aGu = -r2A * (A(kqU0, -M) * ZWu - A(kqU0, M) * ZEu);
-      if (hasN) aGu -= r2AN * A(kqUm, 0) * YNu;
-      if (hasS) aGu += r2AS * A(kqU1, 0) * YSu;
-      if (up) aGu -= r2dsU * yUp * rPuc * WTu;
-      if (dn) aGu += r2dsD * yUn * rPuc * WBu;
-      aGu += (T(-0.25) * yUc * (A(kVs, 0) + A(kVs, 1)) + Cu * Uc) * cota;
-      const T aU = Cu * (f0 + Uc * rPuc * cota);
-      T horU = ZEu * A(kGu0, M) - ZWu * A(kGu0, -M) + YSu * A(kGu1, 0) - YNu * A(kGum, 0);
-      const T verU = (dn ? WBu * Un * rPuc : T(0)) - (up ? WTu * Up * rPuc : T(0));
-      const T tRPu = -yUc * (horU * r2A + verU * r2ds);
-      const T tPu = -yUc * (ocur.psb - ocur.psa) * rdx;
-      const T bu = aU + aFl * Puc + aGu * rPuc;
-      aPu += aFl * Uc + tPu;
-      arPu += aGu * Uc + tRPu;
-      {
-        const unsigned q = r3 + c;
-        const T v = o.scale * bu;
-        if (o.sU) {
-          o.oU[q] = v;
-          o.sU[q] = accU + v;
-        } else {
-          o.oU[q] = accU + v;  // accU = 0 unless accumulating
+      if (o.sU) {
+        o.oU[q3] = vU;
+        o.oPhi[q3] = vP;
+        o.sU[q3] = accU + vU;
+        o.sPhi[q3] = accP + vP;
+        if (hasS) {
+          o.oV[qv] = vV;
+          o.sV[qv] = accV + vV;
         }
+      } else {
+        o.oU[q3] = accU + vU;  // accU = 0 unless accumulating
+        o.oPhi[q3] = accP + vP;
+        if (hasS) o.oV[qv] = accV + vV;
       }
-      // ---------------- Phi point
-      T aGs = -r2A * zf * (A(kqP0, -M) * Fla1 - A(kqP0, M) * Flb1);
-      if (hasN) aGs -= r2AN * A(kqPm, 0) * yvN * FtN;
-      if (hasS) aGs += r2AS * A(kqP1, 0) * yvS * FtS;
-      if (up) aGs -= r2dsU * yPp * rPc * Wt;
-      if (dn) aGs += r2dsD * yPn * rPc * Wb;
-      const T horP = zf * (Flb1 * A(kGs0, M) - Fla1 * A(kGs0, -M)) + yvS * FtS * A(kGs1, 0) - yvN * FtN * A(kGsm, 0);
-      const T verP = (dn ? Wb * Pn * rPc : T(0)) - (up ? Wt * Pp * rPc : T(0));
-      const T tRP = -yPc * (horP * r2A + verP * r2ds);
-      const T bp = ocur.aPh + aGs * rPc;
-      arP += aGs * Pc + tRP;
-      {
-        const unsigned q = r3 + c;
-        const T v = o.scale * bp;
-        if (o.sU) {
-          o.oPhi[q] = v;
-          o.sPhi[q] = accP + v;
-        } else {
-          o.oPhi[q] = accP + v;
-        }
-      }
-      // ---------------- V point
-      if (hasS) {
-        const T aYP = -r2A * A(kqP0, 0) * A(kGs1, 0) + r2AS * A(kqP1, 0) * A(kGs0, 0);
-        const T aYU = (-r2A * A(kqU0, 0) * A(kGu1, 0) + r2AS * A(kqU1, 0) * A(kGu0, 0)) +
-                      (-r2A * A(kqU0, -1) * A(kGu1, -1) + r2AS * A(kqU1, -1) * A(kGu0, -1));
-        T aYV = 0;
-        if (hasSS) aYV += -r2AvS * A(kqV0, 0) * A(kGv1, 0) + r2AvSS * A(kqV1, 0) * A(kGv0, 0);
-        if (hasN) aYV += -r2AvN * A(kqVm, 0) * A(kGv0, 0) + r2AvS * A(kqV0, 0) * A(kGvm, 0);
-        T aFt = yvS * aYP + T(0.5) * yvS * (aYU + aYV);
-        aFt += svS * (rdyS * ocur.Dbc - rdyS1 * ocur.Dbs);
-        const T ZEv = T(0.5) * zfvS * (A(kFl0, ofEv) + A(kFl1, ofEv));
-        const T ZWv = T(0.5) * zfvS * (A(kFl0, ofWv) + A(kFl1, ofWv));
-        const T FtSS = A(kFt1, 0);
-        const T YSv = hasSS ? T(0.5) * (yvS * FtS + yvSS * FtSS) : T(0);
-        const T YNv = hasN ? T(0.5) * (yvN * FtN + yvS * FtS) : T(0);
-        const T WTv = up ? T(0.5) * (Wt + Wts) : T(0), WBv = dn ? T(0.5) * (Wb + Wbs) : T(0);
-        T aGv = -r2AvS * (A(kqV0, -Mv) * ZWv - A(kqV0, Mv) * ZEv);
-        if (hasN) aGv -= r2AvN * A(kqVm, 0) * YNv;
-        if (hasSS) aGv += r2AvSS * A(kqV1, 0) * YSv;
-        if (up) aGv -= r2dsU * yVp * rPvc * WTv;
-        if (dn) aGv += r2dsD * yVn * rPvc * WBv;
-        const T aV = T(-0.25) * (A(kcUs, -1) + A(kcUs, 0));
-        const T horV = ZEv * A(kGv0, Mv) - ZWv * A(kGv0, -Mv) + YSv * A(kGv1, 0) - YNv * A(kGvm, 0);
-        const T verV = (dn ? WBv * Vn * rPvc : T(0)) - (up ? WTv * Vp * rPvc : T(0));
-        const T tRPv = -yVc * (horV * r2AvS + verV * r2ds);
-        const T tPv = -yVc * (ocur.pss - ocur.psc) * rady;
-        const T bv = aV + aFt * Pvc + aGv * rPvc;
-        aPv += aFt * Vc + tPv;
-        arPv += aGv * Vc + tRPv;
-        const unsigned q = rv + c;
-        const T v = o.scale * bv;
-        if (o.sU) {
-          o.oV[q] = v;
-          o.sV[q] = accV + v;
-        } else {
-          o.oV[q] = accV + v;
-        }
-      }
-      yPp = yPc; Pp = Pc; yUp = yUc; Up = Uc; yVp = yVc; Vp = Vc;
-      Wt = Wb; Wtp = Wbp; Wts = Wbs;
     }
-    cur = nxt;
-    ocur = onxt;
+    q3 += plane;
+    qv += vplane;
+  };
+
+  copy_wait<R - 1>();
+  row_sync(NTW);  // the level table and the first level are staged
+  int sl0 = 0;
+  auto level = [&](const int k, auto SL) __attribute__((always_inline)) {
+    constexpr int sl = decltype(SL)::value;
+    const int slot = sl0 + sl;
+    const T* const raw = ring + (size_t)slot * (kAdjRaw * NTP) + t;
+    T* const P = pub + (size_t)sl * kAdjPub * NTP + t;
+    auto X = [&](int row) { return raw[row * NTP]; };
+    const T rds = s_rds[k], rA = rds * A, rAv = rds * Av;
+    T U[3], Ph[3], V[3], yU[3], yP[3], yV[3], hP[3], hU[3], hV[3], Gs[3], Gu[3], Gv[3], FT[3], FL[2];
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      U[r] = X(r);
+      Ph[r] = X(3 + r);
+      V[r] = X(6 + r);
+      yU[r] = X(9 + r);
+      yP[r] = X(12 + r);
+      yV[r] = X(15 + r);
+      hP[r] = yP[r] * kP[r];
+      Gs[r] = Ph[r] * rP[r];
+      hU[r] = yU[r] * kU[r];
+      Gu[r] = U[r] * rPu[r];
+      hV[r] = yV[r] * kV[r];
+      Gv[r] = V[r] * rPv[r];
+      FT[r] = b[r] * V[r];
+      if (r > 0) FL[r - 1] = aF[r - 1] * U[r];
+    }
+    const T fs = f0 + cota * Gu[1];
+    const T cU = yU[1] * fs + yU[2] * (f1 + cota1 * Gu[2]);
+    const T yC = cn * yV[1] + csn * yV[0], vs = V[0] + V[1];
+    const T eU = hU[1] * Gu[2] - hU[2] * Gu[1];
+    P[kpHP * NTP] = hP[1];
+    P[kpGs * NTP] = Gs[1];
+    P[kpHU * NTP] = hU[1];
+    P[kpGu * NTP] = Gu[1];
+    P[kpFL * NTP] = FL[0];
+    P[kpHV * NTP] = hV[1];
+    P[kpGv * NTP] = Gv[1];
+    P[kpFT * NTP] = FT[1];
+    P[kpFLs * NTP] = FL[1];
+    P[kpHVm * NTP] = hV[0];
+    P[kpGvm * NTP] = Gv[0];
+    P[kpFTm * NTP] = FT[0];
+    P[kpYC * NTP] = yC;
+    P[kpVs * NTP] = vs;
+    P[kpCU * NTP] = cU;
+    P[kpEU * NTP] = eU;
+    // the staged rows read as they are
+    const T dpsi = raw[18 * NTP + ob0] - raw[18 * NTP + oa0], dpsv = X(19) - X(18);
+    const T dDb = raw[20 * NTP + oa0] - raw[20 * NTP + ob0], dDv = s0 * X(20) - s1 * X(21);
+    const T W0 = X(22), WU = W0 + raw[22 * NTP + 1], WV = W0 + X(23), aPh = X(24);
+    // ---- the level above: its bottom face is this level's top face
+    const T hU0 = hU[1] * rA, hP0 = hP[1] * rA, hV0 = hV[1] * rAv;
+    if (k > 0) {
+      const T dU = -hU0 * WU, dP = -hP0 * W0, dV = -hV0 * WV;
+      bU += dU * rPu[1];
+      bP += dP * rP[1];
+      bV += dV * rPv[1];
+      arPu += dU * xU + yrU * (WU * Gu[1]);
+      arP += dP * xP + yrP * (W0 * Gs[1]);
+      arPv += dV * xV + yrV * (WV * Gv[1]);
+      write(rmw ? X(25) : T(0), rmw ? X(26) : T(0), rmw ? X(27) : T(0));
+    }
+    // ---- what needs no neighbour column
+    const T hyU = T(0.5) * nr2A * yU[1], hyP = nr2A * yP[1], hyV = T(0.5) * nr2Av * yV[1];
+    T agU = hvU * WU, agP = hvP * W0, agV = hvV * WV;
+    agP += hP[0] * FT[0];
+    agP -= hP[2] * FT[1];
+    yrU = hyU * rA;
+    yrP = hyP * rA;
+    yrV = hyV * rAv;
+    arPu -= yrU * (WU * GuP);
+    arP -= yrP * (W0 * GsP);
+    arPv -= yrV * (WV * GvP);
+    T horP = FT[1] * Gs[2] - FT[0] * Gs[0];
+    T eV = eU + hP[1] * Gs[2];
+    eV -= hP[2] * Gs[1];
+    eV += hV[1] * (Gv[2] - Gv[0]);
+    eV += (hV[0] - hV[2]) * Gv[1];
+    const T YSv = FT[1] + FT[2], YNv = FT[0] + FT[1];
+    agV += hV[0] * YNv;
+    agV -= hV[2] * YSv;
+    T horV = YSv * Gv[2] - YNv * Gv[0];
+    hvU = hU0;
+    hvP = hP0;
+    hvV = hV0;
+    GuP = Gu[1];
+    GsP = Gs[1];
+    GvP = Gv[1];
+    copy_wait<R - 2>();
+    row_sync(NTW);
+    // every thread is past its reads of this ring slot: fetch level k + R into it
+    if (k + R < K) issue_level(k + R, slot);
+    copy_commit();
+    auto N = [&](int arr, int off) { return P[arr * NTP + off]; };
+    // ---- partners at +-M, +-Mv
+    const T hPE = N(kpHP, M), hPW = N(kpHP, -M), GsE = N(kpGs, M), GsW = N(kpGs, -M);
+    const T hUE = N(kpHU, M), hUW = N(kpHU, -M), GuE = N(kpGu, M), GuW = N(kpGu, -M);
+    const T hVE = N(kpHV, Mv), hVW = N(kpHV, -Mv), GvE = N(kpGv, Mv), GvW = N(kpGv, -Mv);
+    const T Fb0 = N(kpFL, ob0), Fa1 = N(kpFL, oa1);
+    const T Fa0 = M1 ? FL[0] : N(kpFL, oa0), Fb1 = M1 ? FL[0] : N(kpFL, ob1);
+    const T FTp = N(kpFT, 1), FTmp = N(kpFTm, 1);
+    // ---------------- U point and F^u
+    T e, aFl;
+    if (M1) {
+      e = hP[1] * GsE;
+      e -= hPE * Gs[1];
+      e += hU[1] * (GuE - GuW);
+      e += (hUW - hUE) * Gu[1];
+      e += hV[1] * GvE;
+      e -= hVE * Gv[1];
+      e += hV[0] * N(kpGvm, 1);
+      e -= N(kpHVm, 1) * Gv[0];
+      aFl = zf * e + rdx * dDb;
+    } else {
+      e = (N(kpHP, oa0) * N(kpGs, ob0) - N(kpHP, ob0) * N(kpGs, oa0)) +
+          (N(kpHU, oa0) * N(kpGu, ob0) - N(kpHU, ob0) * N(kpGu, oa0)) +
+          (N(kpHU, oa1) * N(kpGu, ob1) - N(kpHU, ob1) * N(kpGu, oa1));
+      aFl = zf * e + zS * (N(kpHV, ocS) * N(kpGv, odS) - N(kpHV, odS) * N(kpGv, ocS)) +
+            zN * (N(kpHVm, ocN) * N(kpGvm, odN) - N(kpHVm, odN) * N(kpGvm, ocN)) + rdx * dDb;
+    }
+    {
+      const T ZE = Fb1 + Fb0, ZW = Fa1 + Fa0, YS = FT[1] + FTp, YN = FT[0] + FTmp;
+      const T Cu = yC + N(kpYC, 1), v = vs + N(kpVs, 1);
+      agU += hUW * ZW;
+      agU -= hUE * ZE;
+      agU += hU[0] * YN;
+      agU -= hU[2] * YS;
+      agU += cota * (Cu * U[1] - T(0.25) * yU[1] * v);
+      T hor = ZE * GuE;
+      hor -= ZW * GuW;
+      hor += YS * Gu[2];
+      hor -= YN * Gu[0];
+      bU = Cu * fs + aFl * Pu0 + agU * rPu[1];
+      aPu += aFl * U[1] - yU[1] * (dpsi * rdx);
+      arPu += agU * U[1] + hyU * hor;
+    }
+    // ---------------- Phi point
+    agP += hPW * Fa1;
+    agP -= hPE * Fb1;
+    horP += Fb1 * GsE;
+    horP -= Fa1 * GsW;
+    bP = aPh + agP * rP[1];
+    arP += agP * Ph[1] + hyP * horP;
+    // ---------------- V point
+    if (hasS) {
+      const T ZE = M1 ? FL[0] + FL[1] : rm * N(kpFL, ofE) + N(kpFLs, ofE);
+      const T ZW = (M1 ? Fa1 : rm * N(kpFL, ofW)) + N(kpFLs, ofW);
+      const T aFt = yvS * (eV + N(kpEU, -1)) + dDv;
+      agV += hVW * ZW;
+      agV -= hVE * ZE;
+      horV += ZE * GvE;
+      horV -= ZW * GvW;
+      bV = T(-0.25) * (cU + N(kpCU, -1)) + aFt * Pv0 + agV * rPv[1];
+      aPv += aFt * V[1] - yV[1] * (dpsv * rady);
+      arPv += agV * V[1] + hyV * horV;
+    }
+    xU = U[1];
+    xP = Ph[1];
+    xV = V[1];
+  };
+  int k = 0;
+  for (; k + 1 < K; k += 2) {
+    level(k, std::integral_constant<int, 0>{});
+    level(k + 1, std::integral_constant<int, 1>{});
+    if (R == 4) sl0 ^= 2;
+  }
+  if (k < K) level(k, std::integral_constant<int, 0>{});
+  {  // the last level has no level below
+    T accU = 0, accP = 0, accV = 0;
+    if (rmw && owner) {
+      accU = a.rU[q3];
+      accP = a.rPhi[q3];
+      if (hasS) accV = a.rV[qv];
+    }
+    write(accU, accP, accV);
   }
   if (owner) {
-    const unsigned n = r2 + c;
-    m.mub[n] = aPu * T(0.5) * rPuc - arPu * T(0.5) * rPuc * rPuc * rPuc;
-    m.mvb[n] = hasS ? aPv * T(0.5) * rPvc - arPv * T(0.5) * rPvc * rPvc * rPvc : T(0);
-    m.mcb[n] = -arP * T(0.5) * rPc * rPc * rPc;
+    const unsigned n = r2 + (unsigned)c;
+    m.mub[n] = aPu * T(0.5) * rPu[1] - arPu * T(0.5) * rPu[1] * rPu[1] * rPu[1];
+    m.mvb[n] = hasS ? aPv * T(0.5) * rPv[1] - arPv * T(0.5) * rPv[1] * rPv[1] * rPv[1] : T(0);
+    m.mcb[n] = -arP * T(0.5) * rP[1] * rP[1] * rP[1];
   }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64)
+    k_adj_rows(const __grid_constant__ Geom<T> g, const __grid_constant__ ColState<T> cs,
+               const __grid_constant__ AdjRowArgs<T> a, const __grid_constant__ AdjM<T> m,
+               const __grid_constant__ AdjOut<T> o, const int nany) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int4 item = a.items[blockIdx.x];
+  if ((int)blockIdx.x >= nany)
+    adj_row<T, true>(g, cs, a, m, o, item, smem);
+  else
+    adj_row<T, false>(g, cs, a, m, o, item, smem);
 }
 
 // pi-bar = direct psi part + m-bar, with m^u_i = (m_i + m_{i+1})/2 and

@@ -240,10 +240,11 @@ struct agcm_state {
   bool adj_ready = false;
   void* adj3[2] = {};   // Db aPhi                                  (K*J*I)
   void* adj2[5] = {};   // arPcol aPiD mub mvb mcb                  (J*I)
-  // rows of the adjoint gather: row-segment items (j << 8 | segment) of
-  // k_adj_rows, and the rows left to k_adj_gather
-  int* adj_items = nullptr;
-  int n_adj_items = 0;
+  // rows of the adjoint gather: row-segment items of k_adj_rows (the first
+  // n_adj_any of rows of any strides, the others of rows of stride 1), CTAs of
+  // adj_threads; and the rows left to k_adj_gather
+  int4* adj_items = nullptr;
+  int n_adj_items = 0, n_adj_any = 0, adj_threads = 32;
   int* adj_rows = nullptr;
   int n_adj_rows = 0;
   void* adj_part = nullptr;  // level-chunk partial sums of those rows (3 * chunks * rows * I)
@@ -1334,22 +1335,30 @@ int ensure_adj(agcm_state* s) {
   for (auto& p : s->adj2) p = get(n2);
   // rows whose adjoint halo fits a row segment go to k_adj_rows
   const agcm_grid* g = s->grid;
-  std::vector<int> items, rows;
+  std::vector<int4> items, ones;
+  std::vector<int> rows;
   for (int j = 0; j < g->J; ++j) {
-    const int H = agcm::adj_row_halo(g->Mu[j], j < g->J - 1 ? g->Mv[j] : 0, j > 0 ? g->Mv[j - 1] : 0);
-    int nseg = 0, S = 0;
-    if (H <= agcm::kAdjRowMaxH && H < g->I) agcm::adj_row_segments(g->I, H, &nseg, &S);
-    if (nseg > 0 && nseg <= 256) {
-      for (int q = 0; q < nseg; ++q)
-        if (q * S < g->I) items.push_back(j << 8 | q);
-    } else {
+    const int M = g->Mu[j], Mv = j < g->J - 1 ? g->Mv[j] : 0, Mvm = j > 0 ? g->Mv[j - 1] : 0;
+    const int H = agcm::adj_row_halo(M, Mv, Mvm);
+    int n = 0, S = 0;
+    agcm::row_segments(g->I, H, agcm::kRowB, &n, &S);
+    if (n == 0) {
       rows.push_back(j);
+      continue;
+    }
+    const bool one = M == 1 && Mv == 1 && Mvm == 1;
+    for (int q = 0; q < g->I; q += S) {
+      const int own = std::min(S, g->I - q);
+      (one ? ones : items).push_back(make_int4(j, q, own, H));
+      s->adj_threads = std::max(s->adj_threads, (own + 2 * H + 31) & ~31);
     }
   }
-  auto put_ints = [&](const std::vector<int>& v) -> int* {
-    if (v.empty()) return nullptr;
-    int* d = (int*)get(v.size() * sizeof(int));
-    if (d && cudaMemcpy(d, v.data(), v.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+  s->n_adj_any = (int)items.size();
+  items.insert(items.end(), ones.begin(), ones.end());
+  auto put_ints = [&](const auto& v) {
+    using E = std::decay_t<decltype(v[0])>;
+    E* d = v.empty() ? nullptr : (E*)get(v.size() * sizeof(E));
+    if (d && cudaMemcpy(d, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
     return d;
   };
   s->adj_items = put_ints(items);
@@ -1436,16 +1445,22 @@ int vjp(agcm_state* s, void* const x[4], const void* const y[4], void* const out
         G, s->adj_rows, s->n_adj_rows, nch, (const T*)s->adj_part, m);
   }
   if (s->n_adj_items > 0) {
-    constexpr size_t smem = agcm::adj_row_smem<T>();
-    static std::atomic<bool> attr{false};
-    if (!attr.load()) {
+    const size_t smem = agcm::adj_row_smem<T>(G.K);
+    static std::atomic<size_t> attr{0};  // the size set so far
+    if (attr.load() < smem) {
       CUDA_TRY(cudaFuncSetAttribute(agcm::k_adj_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      attr.store(true);
+      attr.store(smem);
     }
-    agcm::k_adj_rows<T><<<(unsigned)s->n_adj_items, agcm::kAdjRowB, smem, st>>>(
-        G, s->adj_items, (const T*)x[0], (const T*)x[1], (const T*)x[2], cs, (const T*)s->W, (const T*)s->psi,
-        (const T*)s->adj3[0], (const T*)s->adj3[1], (const T*)s->adj2[0], (const T*)y[0], (const T*)y[1],
-        (const T*)y[2], m, o);
+    const T* const r[3] = {sum ? o.rU : (accumulate ? o.oU : nullptr), sum ? o.rV : (accumulate ? o.oV : nullptr),
+                           sum ? o.rPhi : (accumulate ? o.oPhi : nullptr)};
+    bool vec = G.I % 4 == 0;
+    for (const void* p : {(const void*)x[0], (const void*)x[1], (const void*)x[2], (const void*)y[0], (const void*)y[1],
+                          (const void*)y[2], (const void*)r[0], (const void*)r[1], (const void*)r[2]})
+      vec = vec && ((uintptr_t)p & 15) == 0;
+    const agcm::AdjRowArgs<T> ra{(const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)y[0], (const T*)y[1],
+                                 (const T*)y[2], c.W, c.psi, c.Db, c.aPhi, c.arP, r[0], r[1], r[2], s->adj_items,
+                                 vec ? 1 : 0};
+    agcm::k_adj_rows<T><<<(unsigned)s->n_adj_items, s->adj_threads, smem, st>>>(G, cs, ra, m, o, s->n_adj_any);
   }
   if (fork) {
     CUDA_TRY(cudaEventRecord(s->ev_join[0], s->aux[0]));
