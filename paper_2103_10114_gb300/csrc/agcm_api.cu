@@ -334,9 +334,9 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
   return threads;
 }
 
-// Pairs, as long as they make two CTAs an SM (1440x720x30 FP32: 321 against
-// 428 us a stage with single rows, 720x360x30: 97 against 118, 405x203x26: 49
-// against 54); with fewer, single rows (256x128x30: 33.5 against 35 us; FP64
+// Pairs, as long as they make two CTAs an SM (before the set-up's loads were
+// gathered, 1440x720x30 FP32: 321 against 428 us a stage with single rows,
+// 720x360x30: 97 against 118, 405x203x26: 49 against 54); with fewer, single rows (256x128x30: 33.5 against 35 us; FP64
 // 128x64x8: 60 against 82 us).  Single rows in CTAs of the width that leaves
 // the fewest warps on the busiest of an SM's four schedulers, the narrowest
 // among equals (FP64 128x64x8, 64 threads: 52 us), up to three CTAs an SM.
@@ -440,7 +440,7 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   filtU.push_back(0);
   filtV.push_back(0);
   // the row-segment kernel's level table and row tables
-  std::vector<double> lev((size_t)K * agcm::kLevN, 0.0), Af(J), Ac(J), rvn(JV), rvs(JV), rAd(J);
+  std::vector<double> lev((size_t)K * agcm::kLevN, 0.0), rowtab((size_t)J * agcm::kRowTabN, 0.0), rAz(J);
   for (int k = 0; k < K; ++k) {
     double* L = lev.data() + (size_t)k * agcm::kLevN;
     L[agcm::kLevDs] = g->ds[k];
@@ -453,13 +453,18 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
     L[agcm::kLevRho] = rho[k];
   }
   for (int j = 0; j < J; ++j) {
-    Af[j] = g->A[j] * f0[j];
-    Ac[j] = g->A[j] * cota[j];
-    rAd[j] = 1.0 / g->A[j];
-  }
-  for (int j = 0; j < JV; ++j) {
-    rvn[j] = g->Av[j] / g->A[j];
-    rvs[j] = g->Av[j] / g->A[j + 1];
+    double* L = rowtab.data() + (size_t)j * agcm::kRowTabN;
+    L[agcm::kRtZf] = zf[j];
+    L[agcm::kRtR2A] = r2A[j];
+    L[agcm::kRtAf] = g->A[j] * f0[j];
+    L[agcm::kRtAc] = g->A[j] * cota[j];
+    if (j < JV) {
+      L[agcm::kRtYv] = yv[j];
+      L[agcm::kRtR2Av] = r2Av[j];
+      L[agcm::kRtRvn] = g->Av[j] / g->A[j];
+      L[agcm::kRtRvs] = g->Av[j] / g->A[j + 1];
+    }
+    rAz[j] = (double)(T)zf[j] / g->A[j];
   }
   std::vector<double> rt0pit((size_t)J * I);
   for (size_t n = 0; n < rt0pit.size(); ++n) rt0pit[n] = g->rts[n] / g->pit[n];
@@ -480,8 +485,7 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   std::vector<float4> ds3(K);
   for (int k = 0; k < K; ++k) ds3[k] = split3(g->ds[k]);
   size_t o_ds3 = put(ds3.data(), K * sizeof(float4));
-  size_t o_lev = putT(lev), o_Af = putT(Af), o_Ac = putT(Ac), o_rAd = putD(rAd);
-  size_t o_rvn = putT(rvn.empty() ? std::vector<double>{0} : rvn), o_rvs = putT(rvs.empty() ? std::vector<double>{0} : rvs);
+  size_t o_lev = putT(lev), o_rtab = putT(rowtab), o_rAz = putD(rAz);
   size_t o_rt0 = putT(rt0pit), o_pit = putT(g->pit);
   size_t o_bu = putI(filtU), o_bv = putI(filtV);
   agcm::Geom<T> G{};
@@ -537,11 +541,8 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   G.adl = (T)(kA * g->dlam);
   G.ds3 = (const float4*)(base + o_ds3);
   G.lev = (const T*)(base + o_lev);
-  G.Af = (const T*)(base + o_Af);
-  G.Ac = (const T*)(base + o_Ac);
-  G.rvn = (const T*)(base + o_rvn);
-  G.rvs = (const T*)(base + o_rvs);
-  G.rAd = (const double*)(base + o_rAd);
+  G.rowtab = (const T*)(base + o_rtab);
+  G.rAz = (const double*)(base + o_rAz);
   G.items = (const int4*)(base + o_it);
   *blob_out = d;
   *geom_out = G;
@@ -1520,8 +1521,8 @@ constexpr size_t kOffRaw = 0;                        // 6 row arrays s c cot A s
 constexpr size_t kOffRawLev = kOffRaw + 6 * kRowB;   // sh ds Hkk hk beta (double)
 constexpr size_t kOffPitRaw = kOffRawLev + 5 * kLevB;  // pi~, R T~_s (double)
 constexpr size_t kOffInt = kOffPitRaw + 2 * kColB;   // Mu Mv (int)
-constexpr size_t kOffRowT = kOffInt + 2 * kRowB;     // 16 typed row arrays, 1 / A_j (double)
-constexpr size_t kOffLevT = kOffRowT + 17 * kRowB;   // 7 typed level arrays, the level table of kLevN values
+constexpr size_t kOffRowT = kOffInt + 2 * kRowB;     // 12 typed row arrays, the row table of kRowTabN values, zf / A (double)
+constexpr size_t kOffLevT = kOffRowT + (13 + agcm::kRowTabN) * kRowB;   // 7 typed level arrays, the level table of kLevN values
 constexpr size_t kOffDs3 = kOffLevT + (7 + agcm::kLevN) * kLevB;   // dsigma in three FP32 parts
 constexpr size_t kOffColT = kOffDs3 + 2 * kLevB;                    // pit, rt0pit (typed)
 constexpr size_t kOffBar = kOffColT + 2 * kColB;     // Ubar, Vbar (double)
@@ -1545,7 +1546,8 @@ int g_static_prec[kStaticMaxDevices] = {};
 // Typed device tables from the raw FP64 ones (same formulas as the state path).
 template <class T>
 __global__ void k_static_geom(int I, int J, int K, const double* raw, const double* rawlev, const double* pitraw,
-                              const int* Mu, const int* Mv, T* rowT, double* rAd, T* levT, float4* ds3, T* colT,
+                              const int* Mu, const int* Mv, T* rowT, T* rowtab, double* rAz, T* levT,
+                              float4* ds3, T* colT,
                               size_t rowStride, size_t levStride, size_t colStride, double beta2) {
   const double* s = raw;
   const double* c = raw + rowStride;
@@ -1577,12 +1579,18 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
         rowT[9 * rowStride + j] = (T)(0.5 / Av[j]);
         rowT[10 * rowStride + j] = (T)(0.25 * A[j] / Av[j]);
         rowT[11 * rowStride + j] = (T)(0.25 * A[j + 1] / Av[j]);
-        rowT[12 * rowStride + j] = (T)(Av[j] / A[j]);
-        rowT[13 * rowStride + j] = (T)(Av[j] / A[j + 1]);
       }
-      rowT[14 * rowStride + j] = (T)(A[j] * (2.0 * kOmega * c[j]));
-      rowT[15 * rowStride + j] = (T)(A[j] * (cot[j] / kA));
-      rAd[j] = 1.0 / A[j];
+      T* L = rowtab + (size_t)j * agcm::kRowTabN;
+      const bool v = j < J - 1;
+      L[agcm::kRtZf] = rowT[2 * rowStride + j];
+      L[agcm::kRtR2A] = rowT[3 * rowStride + j];
+      L[agcm::kRtAf] = (T)(A[j] * (2.0 * kOmega * c[j]));
+      L[agcm::kRtAc] = (T)(A[j] * (cot[j] / kA));
+      L[agcm::kRtYv] = v ? rowT[7 * rowStride + j] : T(0);
+      L[agcm::kRtR2Av] = v ? rowT[9 * rowStride + j] : T(0);
+      L[agcm::kRtRvn] = v ? (T)(Av[j] / A[j]) : T(0);
+      L[agcm::kRtRvs] = v ? (T)(Av[j] / A[j + 1]) : T(0);
+      rAz[j] = (double)(T)(kA * dth / Mu[j]) / A[j];
     }
     if (n < (size_t)K) {
       const int k = (int)n;
@@ -1631,7 +1639,8 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   T* rowT = (T*)(base + kOffRowT);
   T* levT = (T*)(base + kOffLevT);
   T* colT = (T*)(base + kOffColT);
-  double* rAd = (double*)(base + kOffRowT + 16 * kRowB);
+  T* rowtab = (T*)(base + kOffRowT + 12 * kRowB);
+  double* rAz = (double*)(base + kOffRowT + (12 + agcm::kRowTabN) * kRowB);
   agcm::Geom<T> G{};
   const RowPlan plan = row_plan(g);
   std::vector<int4> items;  // host only
@@ -1655,7 +1664,7 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
       CUDA_TRY(cudaMemcpyAsync(base + kOffRowL, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
   }
   k_static_geom<T><<<nblocks(std::max<size_t>((size_t)I * J, (size_t)K), 256), 256, 0, st>>>(
-      I, J, K, raw, rawlev, pitraw, Mu, Mv, rowT, rAd, levT, (float4*)(base + kOffDs3), colT, rS, lS, cS, g->beta2);
+      I, J, K, raw, rawlev, pitraw, Mu, Mv, rowT, rowtab, rAz, levT, (float4*)(base + kOffDs3), colT, rS, lS, cS, g->beta2);
   CUDA_TRY(cudaGetLastError());
   }
   G.I = I; G.J = J; G.K = K;
@@ -1678,8 +1687,8 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   G.rt0pit = colT + cS;
   G.rady = (T)(1.0 / (kA * g->dth));
   G.adl = (T)(kA * g->dlam);
-  G.rvn = rowT + 12 * rS; G.rvs = rowT + 13 * rS; G.Af = rowT + 14 * rS; G.Ac = rowT + 15 * rS;
-  G.rAd = rAd;
+  G.rowtab = rowtab;
+  G.rAz = rAz;
   G.ds3 = (const float4*)(base + kOffDs3);
   G.lev = levT + 7 * lS;
   G.items = (const int4*)(base + kOffRowL);

@@ -44,11 +44,11 @@ struct Geom {
   const T* hk_rds;  // hk / dsigma_k (K)
   const T* rho;     // beta2 / beta_k: the delta kappa Phi/P part of the coefficient (K)
   const T* oms;     // 1 - sigma_hat_k (K): W_k = SD_k - (1 - sigma_hat_k) C
-  // the row-segment kernel's tables: per level kLevN values (kLev...), per row
-  // A_j f0, A_j cot(theta_j) / a (J), Av_j / A_j, Av_j / A_{j+1} (J-1), 1 / A_j in FP64 (J)
+  // the row-segment kernel's tables: kLevN values a level (kLev...), kRowTabN
+  // values a row (kRt...; zero where there is no V row), zf_j / A_j in FP64 (J)
   const T* lev;
-  const T *Af, *Ac, *rvn, *rvs;
-  const double* rAd;
+  const T* rowtab;
+  const double* rAz;
   // rows the low-latitude filter changes, entry 4 j + band (1 two-grid, 2 3-point)
   const int* filtU; // scalar / U rows
   const int* filtV; // V rows
@@ -77,6 +77,10 @@ struct Geom {
 // Values per level of Geom::lev: dsigma, 4 beta Hkk, 4 beta hk, 2 beta hk /
 // dsigma, 1 / dsigma, sigma_hat (the level's upper half level), rho, 2 beta Hkk.
 enum { kLevDs, kLevH4, kLevh4, kLevhr2, kLevRds, kLevSh, kLevRho, kLevH2, kLevN };
+
+// Values per row of Geom::rowtab: zf, 1 / (2 A), A f0, A cot(theta) / a; yv, 1 /
+// (2 Av), Av_j / A_j, Av_j / A_{j+1}.
+enum { kRtZf, kRtR2A, kRtAf, kRtAc, kRtYv, kRtR2Av, kRtRvn, kRtRvs, kRowTabN };
 
 __device__ __forceinline__ int wrapi(int i, int I) {
   return i < 0 ? i + I : (i >= I ? i - I : i);
