@@ -280,6 +280,7 @@ inline void leap1_band(const agcm_grid* g, int* lo, int* hi) {
 struct RowPlan {
   int B = agcm::kRowB;
   bool pair = true;
+  int nsm = 152;
 };
 
 // Work items of the row-segment stage kernel (agcm_row.cuh): pairs of
@@ -293,6 +294,8 @@ struct RowPlan {
 inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>* items, int off[3], int cnt[3],
                      int cls[agcm::kRowCls + 1]) {
   std::vector<int4> pairs, polar, single[agcm::kRowCls];
+  std::vector<int> polar_rows;
+  size_t nseg = 0;
   int threads = 32;
   for (int j = 0; j < g->J; ++j) {
     const bool hv = j < g->J - 1;
@@ -308,14 +311,22 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
       for (int q = 0; q < g->I; q += S) {
         const int own = std::min(S, g->I - q);
         list.push_back(make_int4((pair ? agcm::kRowPair : agcm::kRowAny) << 24 | j, q, own, H));
+        ++nseg;
         threads = std::max(threads, (own + 2 * H + 31) & ~31);
       }
       j += pair ? 1 : 0;
     } else {
       threads = agcm::kRowB;
-      for (int q = 0; q < g->I; q += agcm::kRowB) polar.push_back(make_int4(agcm::kRowPolar << 24 | j, q, agcm::kRowB, 0));
+      polar_rows.push_back(j);
     }
   }
+  // The rows next to the poles: in a grid of two waves of CTAs and more their
+  // work counts, else the latency of these few blocks does (33 against 22 us a
+  // stage at 256x128x30, 48 against 33 at 360x180x30; 294 against 314 at
+  // 1440x720x30 the other way).
+  const int cols = nseg >= (size_t)6 * plan.nsm ? agcm::kRowB : 32;
+  for (int j : polar_rows)
+    for (int q = 0; q < g->I; q += cols) polar.push_back(make_int4(agcm::kRowPolar << 24 | j, q, cols, 0));
   items->clear();
   auto put = [&](int kind, const std::vector<int4>& v) {
     if (cnt[kind] == 0) off[kind] = (int)items->size();
@@ -323,7 +334,9 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
     cnt[kind] += (int)v.size();
   };
   cnt[0] = cnt[1] = cnt[2] = 0;
+  off[0] = off[1] = off[2] = 0;
   put(agcm::kRowPolar, polar);
+  off[agcm::kRowPair] = (int)items->size();
   put(agcm::kRowPair, pairs);
   off[agcm::kRowAny] = (int)items->size();
   for (int c = 0; c < agcm::kRowCls; ++c) {
@@ -336,8 +349,9 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
 
 // Pairs, as long as they make two CTAs an SM (before the set-up's loads were
 // gathered, 1440x720x30 FP32: 321 against 428 us a stage with single rows,
-// 720x360x30: 97 against 118, 405x203x26: 49 against 54); with fewer, single rows (256x128x30: 33.5 against 35 us; FP64
-// 128x64x8: 60 against 82 us).  Single rows in CTAs of the width that leaves
+// 720x360x30: 97 against 118, 405x203x26: 49 against 54); with fewer, single
+// rows (256x128x30: 33.5 against 35 us; FP64 128x64x8: 60 against 82 us).
+// Single rows in CTAs of the width that leaves
 // the fewest warps on the busiest of an SM's four schedulers, the narrowest
 // among equals (FP64 128x64x8, 64 threads: 52 us), up to three CTAs an SM.
 inline RowPlan row_plan(const agcm_grid* g) {
@@ -346,8 +360,9 @@ inline RowPlan row_plan(const agcm_grid* g) {
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       nsm < 1) {
     cudaGetLastError();
-    nsm = 152;
+    nsm = p.nsm;
   }
+  p.nsm = nsm;
   std::vector<int4> items;
   int off[3], cnt[3], cls[agcm::kRowCls + 1];
   row_lists(g, p, &items, off, cnt, cls);
@@ -355,11 +370,14 @@ inline RowPlan row_plan(const agcm_grid* g) {
   p.pair = false;
   int best = 0;
   for (int B : {128, 96, 64}) {
-    RowPlan q;
+    RowPlan q = p;
     q.B = B;
     q.pair = false;
-    const int threads = row_lists(g, q, &items, off, cnt, cls);
-    const int per_sm = (int)((items.size() + nsm - 1) / nsm), cost = (per_sm * (threads / 32) + 3) / 4;
+    row_lists(g, q, &items, off, cnt, cls);
+    int n = 0, S = 0;
+    agcm::row_segments(g->I, 4, B, &n, &S);  // most rows: strides 1 and 3
+    const int per_sm = (int)((items.size() + nsm - 1) / nsm), warps = (std::min(S, g->I) + 8 + 31) / 32;
+    const int cost = (per_sm * warps + 3) / 4;
     if (B == 128 || (per_sm <= 3 && cost <= best)) {
       p.B = B;
       best = cost;

@@ -198,10 +198,7 @@ __global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_R
         } else if (kind == kRowAny) {
           row_segment<T, 2, 3, false, 1, false, false>(e.g, ra, w, smem);
         } else {
-          const int i = w.y + t;
-          if (i < e.g.I)
-            fused_column<T, 2>(e.g, i, item_row(w), ra.U, ra.V, ra.Phi, ra.pi, ra.Ubar, ra.Vbar, ra.Ub, ra.Vb, ra.Phib, ra.pib,
-                               ra.Uo, ra.Vo, ra.Phio, ra.pio, ra.Ubar_o, ra.Vbar_o, ra.Ubar_b, ra.Vbar_b, ra.cdt);
+          polar_columns<T, 2, 3, false>(e.g, ra, w, smem);
         }
       }
       cur = -1;  // the next stage rebuilds the member's arguments

@@ -70,13 +70,25 @@ constexpr int kTileX = 32;  // columns of one warp (one block) of the stage kern
 // Omega~ conversion, dpi/dt), 3 = both (the unsplit step).
 // NL: Eq. 1's delta kappa Phi/P term is on; every Phi/P that enters psi or
 // the Omega~ coefficient is scaled by 1 + rho_k Phi/P.
-template <class T, int MODE, int TERMS = 3, bool NL = false, bool L1 = false>
+//
+// NW > 1 and xch not null: the levels are shared out over NW warps of the
+// block (w = 0 the surface's), which hold the same 32 columns.  A warp first sums its levels'
+// contributions to the suffix sums, the warps exchange them through xch
+// ([NW][5][32] values of T, added in warp order), and each walks its own
+// levels with the sums of the warps below; the fields of the level below its
+// first and above its last are read once more.  The chain of K levels, which
+// is all the time that a few rows take, becomes K / NW levels and a short
+// pass.  act: false for a column past the row's end (computed, not stored).
+template <class T, int MODE, int TERMS = 3, bool NL = false, bool L1 = false, int NW = 1>
 __device__ __forceinline__ void fused_column(
     const Geom<T>& g, const int i, const int j, const T* __restrict__ U, const T* __restrict__ V,
     const T* __restrict__ Phi, const T* __restrict__ pi, const double* __restrict__ Ubar,
     const double* __restrict__ Vbar, const T* Ub, const T* Vb, const T* Phib, const T* pib, T* Uo, T* Vo, T* Phio,
-    T* pio, double* Ubar_o, double* Vbar_o, const double* Ubar_b, const double* Vbar_b, const T cdt) {
+    T* pio, double* Ubar_o, double* Vbar_o, const double* Ubar_b, const double* Vbar_b, const T cdt,
+    const int w = 0, T* xch = nullptr, const bool act = true) {
   const int I = g.I, J = g.J, K = g.K;
+  const bool split = NW > 1 && xch;
+  const int ke = split ? K - w * K / NW : K, kb = split ? K - (w + 1) * K / NW : 0;  // this warp's levels
   constexpr bool ADV = (TERMS & 1) != 0, ADA = (TERMS & 2) != 0;
   const bool hasS = L1 || j < J - 1;   // V row j exists, scalar row j+1 exists
   const bool hasN = L1 || j > 0;       // V row j-1 exists
@@ -169,7 +181,8 @@ __device__ __forceinline__ void fused_column(
     Cs = ((double)PugE * Ubar[rjp + gE] - (double)PugW * Ubar[rjp + gW]) * (double)rdxs +
          ((hasSS ? (double)svjp * (double)Pvs * Vbar[rjp + i] : 0.0) - (double)svj * (double)Pvc * Vbar[rj + i]) *
              (double)rdys;
-  if (MODE == 0)
+  if (NW > 1 && (w > 0 || !act)) {
+  } else if (MODE == 0)
     pio[rj + i] = ADA ? (T)(-Cc) : T(0);
   else {
     const double pb = (MODE == 1) ? (double)pi[rj + i] : (double)pib[rj + i];
@@ -189,24 +202,72 @@ __device__ __forceinline__ void fused_column(
   double ubar = 0.0, vbar = 0.0;
   T dubar = T(0), dvbar = T(0);
 
+  if (split) {
+    // the warps' sums over their levels, and the levels below this warp's
+    T p[5] = {0, 0, 0, 0, 0};
+#pragma unroll 2
+    for (int k = ke - 1; k >= kb; --k) {
+      const T* Uk = U + (size_t)k * plane;
+      const T* Phk = Phi + (size_t)k * plane;
+      const T* Vk = V + (size_t)k * vplane;
+      const T dsk = g.ds[k], hk = g.hk[k], rho = NL ? g.rho[k] : T(0);
+      const T Ftc = hasS ? Pvc * Vk[rj + i] : T(0), Ftp = hasS ? Pvp * Vk[rj + ip] : T(0);
+      const T Ftn = hasN ? Pvn * Vk[rjm + i] : T(0), Ftnp = hasN ? Pvnp * Vk[rjm + ip] : T(0);
+      const T Fts = hasSS ? Pvs * Vk[rjp + i] : T(0);
+      p[0] += dsk * ((PufE * Uk[rj + fE] - PufW * Uk[rj + fW]) * rdx + (svj * Ftc - svjm * Ftn) * rdy);
+      p[1] += dsk * ((PufE1 * Uk[rj + fE1] - PufW1 * Uk[rj + fW1]) * rdx + (svj * Ftp - svjm * Ftnp) * rdy);
+      if (hasS)
+        p[2] += dsk * ((PugE * Uk[rjp + gE] - PugW * Uk[rjp + gW]) * rdxs + (svjp * Fts - svj * Ftc) * rdys);
+      auto B = [&](T G) { return NL ? G * (one + rho * G) : G; };
+      p[3] += hk * (B(rPE1 * Phk[rj + fE1]) - B(rPW1 * Phk[rj + fW1]));
+      if (hasS) p[4] += hk * (B(rPs * Phk[rjp + i]) - B(rPc * Phk[rj + i]));
+    }
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int q = 0; q < 5; ++q) xch[(w * 5 + q) * 32 + lane] = p[q];
+    __syncthreads();
+    for (int v = 0; v < w; ++v) {
+      SD += xch[(v * 5 + 0) * 32 + lane];
+      SDp += xch[(v * 5 + 1) * 32 + lane];
+      SDs += xch[(v * 5 + 2) * 32 + lane];
+      dSU += xch[(v * 5 + 3) * 32 + lane];
+      dSV += xch[(v * 5 + 4) * 32 + lane];
+    }
+    if (ke < K && kb < ke) {
+      const T om = g.oms[ke];
+      Wb = SD - om * Cf;
+      Wbp = SDp - om * Cpf;
+      Wbs = SDs - om * Csf;
+      GsB = Phi[(size_t)ke * plane + rj + i] * rPc;
+      GuB = U[(size_t)ke * plane + rj + i] * rPuc;
+      GvB = hasS ? V[(size_t)ke * vplane + rj + i] * rPvc : T(0);
+    }
+  }
+
   // software pipeline: the geometry of a level is loaded one iteration before
   // its level is computed, and the base state of a level one iteration before
   // that level is completed and written
-  T q_ds = g.ds[K - 1], q_H = g.Hkk[K - 1], q_hk = g.hk[K - 1], q_hr = g.hk_rds[K - 1], q_r2 = g.r2ds[K - 1];
-  T q_om = g.oms[K - 1];
-  T q_rho = NL ? g.rho[K - 1] : T(0);
-  double q_dsd = g.dsd[K - 1];
+  const int kf = max(ke - 1, 0);
+  T q_ds = g.ds[kf], q_H = g.Hkk[kf], q_hk = g.hk[kf], q_hr = g.hk_rds[kf], q_r2 = g.r2ds[kf];
+  T q_om = g.oms[kf];
+  T q_rho = NL ? g.rho[kf] : T(0);
+  double q_dsd = g.dsd[kf];
   T p_r2 = 0, p_ds = 0;   // level below: 1/(2 dsigma), dsigma
   double p_dsd = 0.0;
   T pbU = 0, pbV = 0, pbPh = 0;  // level below: base values
   const size_t o_own = (size_t)rj + i;
   int it = 0;
-  for (int k = K - 1; k >= -1; --k, ++it) {
+  for (int k = ke - 1; k >= kb - 1; --k, ++it) {
     T Gsc = 0, Guc = 0, Gvc = 0, Wt = 0, Wtp = 0, Wts = 0;
     T nPPh = 0, nPU = 0, nPV = 0;
     T c_r2 = 0, c_ds = 0, nbU = 0, nbV = 0, nbPh = 0;
     double c_dsd = 0.0;
-    if (k >= 0) {
+    if (NW > 1 && k >= 0 && k < kb) {  // the level above the warp's last: its G only
+      Gsc = Phi[(size_t)k * plane + o_own] * rPc;
+      Guc = U[(size_t)k * plane + o_own] * rPuc;
+      Gvc = hasS ? V[(size_t)k * vplane + o_own] * rPvc : T(0);
+    }
+    if (k >= kb) {
       if (MODE == 2) {  // base of this level, used when it is completed next iteration
         nbU = Ub[(size_t)k * plane + o_own];
         nbPh = Phib[(size_t)k * plane + o_own];
@@ -326,7 +387,7 @@ __device__ __forceinline__ void fused_column(
       }
     }
     // ---- complete level k+1 with its top-face vertical term (needs G_k) and write it
-    if (k + 1 <= K - 1) {
+    if (k + 1 <= ke - 1) {
       const int kk = k + 1;
       const T r2dsk1 = p_r2;
       const T TPh = PPh + (ADV ? Wb * Gsc * r2dsk1 * rPc : T(0));
@@ -334,8 +395,10 @@ __device__ __forceinline__ void fused_column(
       const size_t o = (size_t)kk * plane + rj + i;
       const T bPh = MODE == 0 ? T(0) : pbPh, bU = MODE == 0 ? T(0) : pbU;
       const T oPh = bPh + cdt * TPh, oU = bU + cdt * TU;
-      Phio[o] = oPh;
-      Uo[o] = oU;
+      if (NW == 1 || act) {
+        Phio[o] = oPh;
+        Uo[o] = oU;
+      }
       if (kInc) {
         dubar += p_ds * (oU - bU);
       } else {
@@ -346,7 +409,7 @@ __device__ __forceinline__ void fused_column(
         const size_t ov = (size_t)kk * vplane + rj + i;
         const T bV = MODE == 0 ? T(0) : pbV;
         const T oV = bV + cdt * TV;
-        Vo[ov] = oV;
+        if (NW == 1 || act) Vo[ov] = oV;
         if (kInc)
           dvbar += p_ds * (oV - bV);
         else
@@ -369,7 +432,25 @@ __device__ __forceinline__ void fused_column(
     pbV = nbV;
     pbPh = nbPh;
   }
-  if (Ubar_o) {
+  if (MODE != 0 && split) {
+    const int lane = threadIdx.x & 31;
+    __syncthreads();  // every warp has read the sums
+    xch[(w * 5 + 0) * 32 + lane] = kInc ? dubar : (T)ubar;
+    xch[(w * 5 + 1) * 32 + lane] = kInc ? dvbar : (T)vbar;
+    __syncthreads();
+    if (w > 0) return;
+    for (int v = 1; v < NW; ++v) {
+      const T a = xch[(v * 5 + 0) * 32 + lane], b = xch[(v * 5 + 1) * 32 + lane];
+      if (kInc) {
+        dubar += a;
+        dvbar += b;
+      } else {
+        ubar += (double)a;
+        vbar += (double)b;
+      }
+    }
+  }
+  if (Ubar_o && (NW == 1 || act)) {
     if (kInc) {
       ubar = Ubar_b[rj + i] + (double)dubar;
       if (hasS) vbar = Vbar_b[rj + i] + (double)dvbar;
