@@ -72,29 +72,16 @@ struct AdjCol {
 // vertical advection of the levels h-1, h at the points whose face means hold
 // W(j, i)) and of -C give Cbar and the suffix sums that form Dbar_k.
 //
-// Both forms below hold 32 columns per block and split each column's levels
-// into groups (threadIdx.y): walk 1 forms a group's partial sums, the block
-// exchanges them through shared memory (every sum in group order, so the
-// result is the same on every run), and walk 2 forms each level's outputs
-// with the prefix and suffix offsets of the other groups.  The sums run in
-// the state's precision: FP64 issues at 1/64 of the FP32 rate on this GPU,
-// and per level and column they would be the bulk of the pass.
-//   k_adj_col    groups of at most kColL levels (K <= 8 kColL): walk 1
-//                keeps each level's values in shared memory for walk 2;
-//   k_adj_col_w  any K, kColG groups: walk 2 re-forms each level (its loads
-//                hit L1).
-#ifndef AGCM_COLL
-#define AGCM_COLL 8
-#endif
-constexpr int kColL = AGCM_COLL;
-#ifndef AGCM_COLG
-#define AGCM_COLG 2
-#endif
-constexpr int kColG = AGCM_COLG;
+// The sums run in the state's precision: FP64 issues at 1/64 of the FP32 rate
+// on this GPU, and per level and column they would be the bulk of the pass.
+//   k_adj_col    a row segment per block, rows staged in shared memory, one
+//                walk down and one up the levels, each level's D and adjoint
+//                of W kept in shared memory between them;
+//   k_adj_col_w  more levels than shared memory holds: 32 columns and kColG
+//                groups of levels per block, stencil read through L1.
+constexpr int kColG = 2;
 
-// The per-column pieces shared by the two forms.  ST: the level tables are
-// read from a copy in shared memory (8 values per level: ds, Hkk, hk, hk_rds,
-// r2ds, 1 - sh, rho), else from the grid's tables in global memory.
+// Level tables: ds, Hkk, hk, hk_rds, r2ds, 1 - sh, rho.
 enum { kLds, kLHkk, kLhk, kLhkr, kLr2ds, kLoms, kLrho, kLN = 8 };
 template <class T>
 __device__ __forceinline__ void col_tables(const Geom<T>& g, T* lt, int tid, int nthreads) {
@@ -110,10 +97,10 @@ __device__ __forceinline__ void col_tables(const Geom<T>& g, T* lt, int tid, int
     L[7] = T(0);
   }
 }
-template <class T, bool ST>
+// The per-column pieces of k_adj_col_w.
+template <class T>
 struct ColCtx {
   const Geom<T>& g;
-  const T* lt = nullptr;  // shared-memory level tables (ST)
   const T *U, *V, *Phi, *yU, *yV, *yPhi;
   // element offsets fit 32 bits: nlon * nlat * nlev <= 4e9
   unsigned plane, vplane, r2;
@@ -122,17 +109,13 @@ struct ColCtx {
   T rdx, rdy, rady, svS, svN, Pue, Puw, rPc, rPui, rPum, PvS, PvN, rPvS, rPvN;
 
   __device__ T tab(int k, int f) const {
-    if constexpr (ST) {
-      return lt[kLN * k + f];
-    } else {
-      const T* p = f == kLds ? g.ds : f == kLHkk ? g.Hkk : f == kLhk ? g.hk : f == kLhkr ? g.hk_rds
-                 : f == kLr2ds ? g.r2ds : f == kLoms ? g.oms : g.rho;
-      return ldg(p + k);
-    }
+    const T* p = f == kLds ? g.ds : f == kLHkk ? g.Hkk : f == kLhk ? g.hk : f == kLhkr ? g.hk_rds
+               : f == kLr2ds ? g.r2ds : f == kLoms ? g.oms : g.rho;
+    return ldg(p + k);
   }
-  __device__ ColCtx(const Geom<T>& g_, const T* lt_, const T* U_, const T* V_, const T* Phi_,
+  __device__ ColCtx(const Geom<T>& g_, const T* U_, const T* V_, const T* Phi_,
                     const ColState<T>& cs, const T* yU_, const T* yV_, const T* yPhi_, int i, int j)
-      : g(g_), lt(lt_), U(U_), V(V_), Phi(Phi_), yU(yU_), yV(yV_), yPhi(yPhi_) {
+      : g(g_), U(U_), V(V_), Phi(Phi_), yU(yU_), yV(yV_), yPhi(yPhi_) {
     const int I = g.I, J = g.J;
     plane = (unsigned)J * (unsigned)I;
     vplane = (unsigned)(J - 1) * (unsigned)I;
@@ -160,25 +143,6 @@ struct ColCtx {
     PvN = hasN ? ldg(cs.Pv + n - I) : T(0);
     rPvS = hasS ? ldg(cs.rPv + n) : T(0);
     rPvN = hasN ? ldg(cs.rPv + n - I) : T(0);
-  }
-  // an L2 prefetch of the rows a level reads (no registers held: the level
-  // is loaded one level later)
-  __device__ void prefetch(int k) const {
-    const unsigned o3 = (unsigned)k * plane + r2 + ic, ov = (unsigned)k * vplane + r2 + ic;
-    const int I = g.I;
-    auto pf = [](const T* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); };
-    pf(U + o3);
-    pf(yU + o3);
-    pf(Phi + o3);
-    pf(yPhi + o3);
-    if (hasS) {
-      pf(V + ov);
-      pf(yV + ov);
-    }
-    if (hasN) {
-      pf(V + ov - I);
-      pf(yV + ov - I);
-    }
   }
   // the values of one level: D, the adjoint of psi, Phi, ybar_Phi and the
   // products y / P, x / P of the five points whose vertical advection holds
@@ -246,8 +210,6 @@ struct ColCtx {
   }
 };
 
-__device__ __forceinline__ int gy_off(int gy, int lane) { return gy * 32 + lane; }
-
 // Group sums of one column: sum ds D, sum pb, sum sh aW, sum aW, sum hk B, sum hk_rds xb.
 template <class T>
 struct ColSums {
@@ -281,8 +243,8 @@ __device__ __forceinline__ ColSums<T> col_exchange(T* red, int G, int gy, int la
 // The suffix quantities of level k: W_k, psi_k, Dbar_k.  q*: this group's
 // sums up to level k (qD before it, the others including it), s*: this
 // group's totals, r: the other groups' offsets.
-template <class T, bool ST>
-__device__ __forceinline__ void col_suffix(const ColCtx<T, ST>& c, const AdjCol<T>& o, int k, unsigned q3, T D, T B,
+template <class T>
+__device__ __forceinline__ void col_suffix(const ColCtx<T>& c, const AdjCol<T>& o, int k, unsigned q3, T D, T B,
                                            T xb, T qD, T qB, T qX, T qA, T sD, T sB, T sX, T sA,
                                            const ColSums<T>& r, T ps) {
   const T ds = c.tab(k, kLds), Hkk = c.tab(k, kLHkk);
@@ -292,104 +254,251 @@ __device__ __forceinline__ void col_suffix(const ColCtx<T, ST>& c, const AdjCol<
   o.Db[q3] = ds * (r.Cb - SW) - c.rPc * (Hkk * xb + ds * SX);
 }
 
-// Four 256-thread blocks per SM (64 registers; the FP64 form keeps two):
-// at 720 x 360 x 30 FP32 0.124 ms against 0.159 ms for two blocks (106
-// registers), the pass being bound by load latency.
-#ifndef AGCM_COLB
-#define AGCM_COLB 4
-#endif
-#ifndef AGCM_COLU
-#define AGCM_COLU 8
-#endif
-constexpr int kColU = AGCM_COLU;
+// One row segment per block, one thread per column.  The rows of U, ybar_U,
+// V and ybar_V (V rows j-1, j), Phi and ybar_Phi arrive level by level in a
+// ring of shared-memory slots, two 16-byte copies a thread, on the way down;
+// that walk forms D, the gathered adjoints of psi and W, the prefix sums and
+// with them the adjoint of Phi, and keeps D and the adjoint of W; the walk up
+// forms W, psi and Dbar from the suffix sums, reading Phi and ybar_Phi once
+// more (from L2).  Rows whose divergence pair lies outside the halo (kind 1)
+// read the pair from global memory a level ahead.
+// Bound by load latency (16 warps an SM, 95 registers) in FP32 and by the FP64
+// pipe in FP64.  Per launch of the reverse pass, before (32 columns and four
+// groups of eight levels per block, stencil through L1) and now: 720 x 360 x 30
+// FP32 108 -> 82 us (7.8 M points, 40 B a point at the copy rate 46 us), FP64
+// 1503 -> 1108; 256 x 128 x 30 FP64 201 -> 193, FP32 20 either way; 128 x 64 x
+// 16 FP32 13.5 -> 11.1, FP64 39 -> 48 (one warp a scheduler: its levels are one
+// chain of FP64 issue); 128 x 64 x 120 FP32 71 -> 42, FP64 368 -> 313.  Ring of two slots 107, three 90 (five blocks 82, but
+// 256 x 128 and 405 x 203 4 to 7 % slower); groups of six levels 83.  FP64
+// keeps the adjoint of W in Dbar's place instead of shared memory: 80 KB a
+// block would hold two blocks (1209).
+constexpr int kColRaw = 8;  // U, yU, V j-1, V j, yV j-1, yV j, Phi, yPhi
+constexpr int kColPad = 64;  // before the ring: a halo column's pair reaches at most H <= 32 to the west of it
+constexpr int kColB = 8;  // levels of a partial sum
 template <class T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? AGCM_COLB : 2) k_adj_col(Geom<T> g, const T* __restrict__ U, const T* __restrict__ V,
-                                                 const T* __restrict__ Phi, const T* __restrict__ pi, ColState<T> cs,
-                                                 const T* __restrict__ yU, const T* __restrict__ yV,
-                                                 const T* __restrict__ yPhi, const T* __restrict__ ypi,
-                                                 AdjCol<T> o) {
-  extern __shared__ __align__(16) unsigned char col_smem[];
-  T* const red = reinterpret_cast<T*>(col_smem);  // [7][G][32]: group sums, then arp
-  const int I = g.I, K = g.K, G = blockDim.y;
-  // each level's D, psi adjoint, Phi, ybar_Phi and W adjoint: [5][kColL][G][32];
-  // then the level tables [K][8]
-  T* const lv = red + 7 * G * 32 + gy_off(threadIdx.y, threadIdx.x);
-  T* const lt = red + (7 + 5 * kColL) * G * 32;
-  const int lstride = G * 32;
-  const int lane = threadIdx.x, gy = threadIdx.y;
-  const int i = blockIdx.x * 32 + lane, j = blockIdx.y;
-  const bool col = i < I;
-  col_tables(g, lt, gy * 32 + lane, G * 32);
-  __syncthreads();
-  const ColCtx<T, true> c(g, lt, U, V, Phi, cs, yU, yV, yPhi, col ? i : 0, j);
-  const int kb = min(K, gy * kColL), ke = min(K, kb + kColL);
-  const unsigned n = c.r2 + c.ic;
-  // ---- walk 1: every level's values into shared memory, and the group sums
-  auto vD = [&](int l) -> T& { return lv[(0 * kColL + l) * lstride]; };
-  auto vP = [&](int l) -> T& { return lv[(1 * kColL + l) * lstride]; };
-  auto vPh = [&](int l) -> T& { return lv[(2 * kColL + l) * lstride]; };
-  auto vY = [&](int l) -> T& { return lv[(3 * kColL + l) * lstride]; };
-  auto vA = [&](int l) -> T& { return lv[(4 * kColL + l) * lstride]; };
-  T s[6] = {0, 0, 0, 0, 0, 0};
-  typename ColCtx<T, true>::Lev cv{}, pv{};
-  if (kb > 0 && kb < ke) c.level(kb - 1, pv);
-#pragma unroll kColU
-  for (int l = 0; l < kColL; ++l) {
-    const int k = kb + l;
-    if (k < ke) {
-      if (k + 1 < ke) c.prefetch(k + 1);
-      c.level(k, cv);
-      const T aw = k > 0 ? c.adj_w(k, cv, pv) : T(0);
-      vD(l) = cv.D;
-      vP(l) = cv.pb;
-      vPh(l) = cv.ph;
-      vY(l) = cv.yx;
-      vA(l) = aw;
-      s[0] += c.tab(k, kLds) * cv.D;
-      s[1] += cv.pb;
-      s[2] += (T(1) - c.tab(k, kLoms)) * aw;  // sh_k aW_k (aW = 0 at k = 0)
-      s[3] += aw;
-      s[4] += c.tab(k, kLhk) * c.Bk(k, cv.ph);
-      s[5] += c.tab(k, kLhkr) * c.xbk(k, cv.ph, cv.yx);
-      pv = cv;
-    }
-  }
-  ColSums<T> r = col_exchange(red, G, gy, lane, s);
-  // ---- walk 2: the outputs of every level, from shared memory (each thread
-  // reads back only what it wrote)
-  T arp = 0;
-  if (col && kb < ke) {
-    r.Cb -= ldg(ypi + n);
-    const T ps = ldg(g.rt0pit + n) * ldg(pi + n);
-    T qD = 0, qB = 0, qX = 0, qA = 0, Q = r.Q, pre = r.pre;
-#pragma unroll kColU
-    for (int l = 0; l < kColL; ++l) {
-      const int k = kb + l;
-      if (k < ke) {
-        const unsigned q3 = (unsigned)k * c.plane + n;
-        const T D = vD(l), pb = vP(l), ph = vPh(l), yx = vY(l);
-        o.aPhi[q3] = c.adj_phi(k, D, pb, ph, yx, Q, pre, arp);
-        const T dsk = c.tab(k, kLds);
-        Q += dsk * D;
-        pre += pb;
-        const T B = c.Bk(k, ph), xb = c.xbk(k, ph, yx);
-        const T qD0 = qD;
-        qD += dsk * D;
-        qB += c.tab(k, kLhk) * B;
-        qX += c.tab(k, kLhkr) * xb;
-        qA += vA(l);
-        col_suffix(c, o, k, q3, D, B, xb, qD0, qB, qX, qA, s[0], s[4], s[5], s[3], r, ps);
+struct ColRing {
+  static constexpr int R = sizeof(T) == 4 ? 4 : 2;      // slots
+  static constexpr int kKeep = sizeof(T) == 4 ? 2 : 1;  // arrays kept over the levels
+  static constexpr int kCtas = sizeof(T) == 4 ? 4 : 3;  // blocks per SM
+};
+template <class T>
+constexpr size_t adj_col_smem(int K) {
+  return sizeof(T) * (kColPad + (size_t)kRowB * (ColRing<T>::R * kColRaw + ColRing<T>::kKeep * K) + (size_t)kLN * K);
+}
+// Halo of row j's column pass: the divergence pair and the column to the west.
+__host__ __device__ inline int adj_col_halo(int M) { return ((M + 1) / 2 + 3) & ~3; }
+template <class T>
+struct AdjColArgs {
+  const T *U, *V, *Phi, *pi;        // x
+  const T *yU, *yV, *yPhi, *ypi;    // ybar
+  const int4* items;                // kind << 24 | row j, first own column, own columns, halo
+  int vec;                          // 1: every row is 16-byte aligned
+};
+template <class T>
+__global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
+    k_adj_col(const __grid_constant__ Geom<T> g, const __grid_constant__ ColState<T> cs,
+              const __grid_constant__ AdjColArgs<T> a, const __grid_constant__ AdjCol<T> o) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  constexpr int R = ColRing<T>::R, NTP = kRowB, kKeep = ColRing<T>::kKeep;
+  const int I = g.I, J = g.J, K = g.K;
+  const int4 item = a.items[blockIdx.x];
+  const bool wide = item.x >> 24;
+  const int j = item.x & 0xffffff, c0 = item.y, own = item.z, H = item.w;
+  const bool hasS = j < J - 1, hasN = j > 0, nl = g.nl != 0;
+  const int M = g.Mu[j];
+  const int NT = own + 2 * H, NTW = (NT + 31) & ~31;
+  const int t = threadIdx.x;
+  if (t >= NTW) leave();
+  const bool owner = t >= H && t < H + own;
+  int cstart = c0 - H;
+  while (cstart < 0) cstart += I;
+  int c = cstart + t;
+  while (c >= I) c -= I;
+  T* const ring = reinterpret_cast<T*>(smem) + kColPad;
+  T* const kept = ring + (size_t)R * kColRaw * NTP + t;          // D, the adjoint of W of every level
+  T* const lt = ring + (size_t)(R * kColRaw + kKeep * K) * NTP;  // level tables
+  col_tables(g, lt, t, NTW);
+  // element offsets fit 32 bits: nlon * nlat * nlev <= 4e9
+  const unsigned plane = (unsigned)J * (unsigned)I, vplane = (unsigned)(J - 1) * (unsigned)I;
+  const unsigned r2 = (unsigned)j * (unsigned)I;
+  // a quarter of the threads each: a chunk of four columns of two rows
+  const int tr = NTW >> 2, cr = t / tr, cc = 4 * (t - cr * tr);
+  int c4 = cstart + cc;
+  while (c4 >= I) c4 -= I;
+  const int sw = min(I - c4, 4);  // the first element past the periodic seam
+  const bool vr = cr == 1 || cr == 2;  // V, yV; quarters 0 and 3: U, yU and Phi, yPhi
+  const bool in = cc < NT, ok0 = in && (!vr || hasN), ok1 = in && (!vr || hasS);
+  const T* const f0 = cr == 0 ? a.U : (cr == 1 ? a.V : (cr == 2 ? a.yV : a.Phi));
+  const T* const f1 = cr == 0 ? a.yU : (cr == 1 ? a.V : (cr == 2 ? a.yV : a.yPhi));
+  const unsigned so = r2 + (unsigned)c4;
+  const unsigned o0 = vr ? (ok0 ? so - I : 0u) : so, o1 = vr ? (ok1 ? so : 0u) : so;
+  const unsigned ring_s = smem_addr(ring) + (unsigned)((2 * cr * NTP + cc) * (int)sizeof(T));
+  auto issue_level = [&](int k, int s) __attribute__((always_inline)) {
+    const unsigned p = (unsigned)k * (vr ? vplane : plane), d = ring_s + (unsigned)(s * kColRaw * NTP * (int)sizeof(T));
+    if (a.vec) {
+#pragma unroll
+      for (int e = 0; e < 4; e += 16 / (int)sizeof(T)) {
+        copy16_g2s(d + e * sizeof(T), f0 + (p + o0 + e), true, ok0);
+        copy16_g2s(d + (NTP + e) * sizeof(T), f1 + (p + o1 + e), true, ok1);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const unsigned x = e < sw ? e : e - I;
+        copy_elem_g2s<sizeof(T)>(d + e * sizeof(T), f0 + (p + (ok0 ? o0 + x : 0u)), true, ok0);
+        copy_elem_g2s<sizeof(T)>(d + (NTP + e) * sizeof(T), f1 + (p + (ok1 ? o1 + x : 0u)), true, ok1);
       }
     }
+  };
+  for (int s = 0; s < R; ++s) {
+    if (s < K) issue_level(s, s);
+    copy_commit();
   }
-  T* const rarp = red + 6 * G * 32;
-  rarp[gy * 32 + lane] = arp;
-  __syncthreads();
-  if (gy == 0 && col) {
-    T a = 0;
-    for (int q = 0; q < G; ++q) a += rarp[q * 32 + lane];
-    o.arP[n] = a;
-    o.aPiD[n] = r.psum * ldg(g.rt0pit + n);
+  // ---- the factors of the column
+  const int de = (M - 1) / 2, dw = -(M + 1) / 2;
+  const unsigned n = r2 + (unsigned)c;
+  int ue = c + de, uw = c + dw;
+  ue = ue >= I ? ue - I : ue;
+  uw = uw < 0 ? uw + I : uw;
+  const T rdx = g.rdx[j], rdy = g.rdy[j], rady = g.rady;
+  const T svS = hasS ? ldg(g.sv + j) : T(0), svN = hasN ? ldg(g.sv + j - 1) : T(0);
+  const T PuE = ldg(cs.Pu + r2 + ue), PuW = ldg(cs.Pu + r2 + uw);
+  const T PvS = hasS ? ldg(cs.Pv + n) : T(0), PvN = hasN ? ldg(cs.Pv + n - I) : T(0);
+  const T bS = svS * PvS, bN = svN * PvN;
+  const T rPc = ldg(cs.rP + n), rPu = ldg(cs.rPu + n), rPm = ldg(cs.rPu + r2 + (c > 0 ? c - 1 : I - 1));
+  const T rPvS = hasS ? ldg(cs.rPv + n) : T(0), rPvN = hasN ? ldg(cs.rPv + n - I) : T(0);
+  const T ps = ldg(g.rt0pit + n) * ldg(a.pi + n), rt = ldg(g.rt0pit + n), yp = ldg(a.ypi + n);
+  T wu[4] = {0, 0, 0, 0};  // wide rows: U, yU at the pair, a level ahead
+  if (wide) {
+    wu[0] = ldg(a.U + r2 + ue);
+    wu[1] = ldg(a.U + r2 + uw);
+    wu[2] = ldg(a.yU + r2 + ue);
+    wu[3] = ldg(a.yU + r2 + uw);
+  }
+  // ---- down: D, the adjoints of psi and W, prefix sums
+  // sums over the levels in groups of kColB, each in two parts (whole groups,
+  // the group so far): one chain of K roundings would be less exact
+  T Q0 = 0, Q1 = 0, pre0 = 0, pre1 = 0, Cb0 = 0, Cb1 = 0, arp0 = 0, arp = 0;
+  T r0 = 0;  // 1 / (2 dsigma) of the level above
+  T pq[5] = {0, 0, 0, 0, 0}, px[5] = {0, 0, 0, 0, 0};  // y / P, x / P of the level above
+  copy_wait<R - 1>();
+  row_sync(NTW);
+  int slot = 0;
+  for (int k = 0; k < K; ++k) {
+    const T* const raw = ring + (size_t)slot * (kColRaw * NTP) + t;
+    const T* const L = lt + kLN * k;
+    T Ue, Uw, ye, yw;
+    if (wide) {
+      Ue = wu[0];
+      Uw = wu[1];
+      ye = wu[2];
+      yw = wu[3];
+      if (k + 1 < K) {
+        const unsigned q = (unsigned)(k + 1) * plane + r2;
+        wu[0] = ldg(a.U + q + ue);
+        wu[1] = ldg(a.U + q + uw);
+        wu[2] = ldg(a.yU + q + ue);
+        wu[3] = ldg(a.yU + q + uw);
+      }
+    } else {
+      Ue = raw[de];
+      Uw = raw[dw];
+      ye = raw[NTP + de];
+      yw = raw[NTP + dw];
+    }
+    const T VN = raw[2 * NTP], VS = raw[3 * NTP], yVN = raw[4 * NTP], yVS = raw[5 * NTP];
+    const T ph = raw[6 * NTP], yx = raw[7 * NTP];
+    // metric factors outside: folded into P they would put one rounding of
+    // each into the sum over all levels
+    const T D = rdx * (PuE * Ue - PuW * Uw) + rdy * (bS * VS - bN * VN);
+    const T pb = rdx * (PuE * ye - PuW * yw) + rady * (PvS * yVS - PvN * yVN);
+    // the points whose vertical advection holds W(j, i): Phi (j, i), and in a
+    // face mean (weight 1/2, in q) U (j, i-1), U (j, i), V (j-1, i), V (j, i)
+    const T q[5] = {yx * rPc, raw[NTP - 1] * (T(0.5) * rPm), raw[NTP] * (T(0.5) * rPu), yVN * (T(0.5) * rPvN),
+                    yVS * (T(0.5) * rPvS)};
+    const T x[5] = {ph * rPc, raw[-1] * rPm, raw[0] * rPu, VN * rPvN, VS * rPvS};
+    T u = 0, d = 0;
+#pragma unroll
+    for (int e = 0; e < 5; ++e) {
+      u += q[e] * px[e];
+      d += pq[e] * x[e];
+      pq[e] = q[e];
+      px[e] = x[e];
+    }
+    const T r1 = L[kLr2ds], aw = r1 * u - r0 * d;  // the adjoint of W_k (0 at k = 0)
+    r0 = r1;
+    kept[(size_t)k * NTP] = D;
+    if (kKeep > 1)
+      kept[(size_t)(K + k) * NTP] = aw;
+    else if (owner)
+      o.Db[(unsigned)k * plane + n] = aw;  // read back below
+    Cb1 += (T(1) - L[kLoms]) * aw;
+    const T Q = Q0 + Q1, pre = pre0 + pre1;
+    // the prefix quantities: the adjoints of Phi and 1/P
+    const T Hkk = L[kLHkk], Sk = Hkk * D + L[kLhkr] * Q, Bb = Hkk * pb + L[kLhk] * pre;
+    T ap = Bb;
+    if (!nl) {
+      arp += Bb * ph - yx * Sk;
+    } else {
+      const T rho = L[kLrho], G = rPc * ph;
+      ap = Bb * (T(1) + T(2) * rho * G) - yx * rPc * rho * Sk;  // dB/dG = 1 + 2 rho G
+      arp += ap * ph - yx * (T(1) + rho * G) * Sk;
+    }
+    if (owner) o.aPhi[(unsigned)k * plane + n] = ap * rPc;
+    Q1 += L[kLds] * D;
+    pre1 += pb;
+    if (k % kColB == kColB - 1) {
+      Q0 += Q1;
+      pre0 += pre1;
+      Cb0 += Cb1;
+      arp0 += arp;
+      Q1 = pre1 = Cb1 = arp = T(0);
+    }
+    copy_wait<R - 2>();
+    row_sync(NTW);
+    if (k + R < K) issue_level(k + R, slot);
+    copy_commit();
+    slot = slot + 1 == R ? 0 : slot + 1;
+  }
+  if (!owner) return;
+  // ---- up: W, psi, Dbar from the suffix sums
+  o.arP[n] = arp0 + arp;
+  o.aPiD[n] = (pre0 + pre1) * rt;
+  const T C = Q0 + Q1, Cb = (Cb0 + Cb1) - yp;
+  T SD0 = 0, S0 = 0, SW0 = 0, SX0 = 0;
+  constexpr int B = kColB;  // Phi and ybar_Phi of a group are loaded together
+  for (int kt = K - 1; kt >= 0; kt -= B) {
+    T ph[B], yx[B], kA[B];
+#pragma unroll
+    for (int e = 0; e < B; ++e) {
+      const unsigned q = (unsigned)max(kt - e, 0) * plane + n;
+      ph[e] = ldg(a.Phi + q);
+      yx[e] = ldg(a.yPhi + q);
+      if (kKeep == 1) kA[e] = o.Db[q];
+    }
+    T SD = 0, S = 0, SW = 0, SX = 0;  // of this group
+#pragma unroll
+    for (int e = 0; e < B; ++e) {
+      const int k = kt - e;
+      if (k >= 0) {
+        const T* const L = lt + kLN * k;
+        const unsigned q = (unsigned)k * plane + n;
+        const T D = kept[(size_t)k * NTP], aw = kKeep > 1 ? kept[(size_t)(K + k) * NTP] : kA[e];
+        const T ds = L[kLds], Hkk = L[kLHkk];
+        const T f = nl ? T(1) + L[kLrho] * (rPc * ph[e]) : T(1), Bk = rPc * ph[e] * f, xb = yx[e] * f;
+        SD += ds * D;
+        if (k > 0) o.W[q] = (SD0 + SD) - L[kLoms] * C;
+        o.psi[q] = Hkk * Bk + (S0 + S) + ps;
+        o.Db[q] = ds * (Cb - (SW0 + SW)) - rPc * (Hkk * xb + ds * (SX0 + SX));
+        S += L[kLhk] * Bk;
+        SW += aw;
+        SX += L[kLhkr] * xb;
+      }
+    }
+    SD0 += SD;
+    S0 += S;
+    SW0 += SW;
+    SX0 += SX;
   }
 }
 
@@ -405,12 +514,12 @@ __global__ void __launch_bounds__(32 * kColG) k_adj_col_w(Geom<T> g, const T* __
   const int lane = threadIdx.x, gy = threadIdx.y;
   const int i = blockIdx.x * 32 + lane, j = blockIdx.y;
   const bool col = i < I;
-  const ColCtx<T, false> c(g, nullptr, U, V, Phi, cs, yU, yV, yPhi, col ? i : 0, j);
+  const ColCtx<T> c(g, U, V, Phi, cs, yU, yV, yPhi, col ? i : 0, j);
   const int L = (K + kColG - 1) / kColG;
   const int kb = min(K, gy * L), ke = min(K, kb + L);
   const unsigned n = c.r2 + c.ic;
   T s[6] = {0, 0, 0, 0, 0, 0};
-  typename ColCtx<T, false>::Lev cv{}, pv{};
+  typename ColCtx<T>::Lev cv{}, pv{};
   if (kb < ke) {
     if (kb > 0) c.level(kb - 1, pv);
     for (int k = kb; k < ke; ++k) {
@@ -809,7 +918,7 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
   constexpr int R = AdjRing<T>::R, NTP = kRowB;
   const int I = g.I, J = g.J, K = g.K;
   const int j = item.x & 0xffffff, c0 = item.y, own = item.z, H = item.w;
-  const bool hasS = M1 || j < J - 1, hasN = M1 || j > 0, hasSS = j + 1 < J - 1;
+  const bool hasS = M1 || j < J - 1, hasN = M1 || j > 0;
   const int M = M1 ? 1 : g.Mu[j], Mv = M1 ? 1 : (hasS ? g.Mv[j] : 1), Mvm = M1 ? 1 : (hasN ? g.Mv[j - 1] : 1);
   const int NT = own + 2 * H, NTW = (NT + 31) & ~31;
   const int t = threadIdx.x;

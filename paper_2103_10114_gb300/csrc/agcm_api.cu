@@ -245,6 +245,8 @@ struct agcm_state {
   // adj_threads; and the rows left to k_adj_gather
   int4* adj_items = nullptr;
   int n_adj_items = 0, n_adj_any = 0, adj_threads = 32;
+  int4* col_items = nullptr;  // row-segment items of k_adj_col, CTAs of col_threads
+  int n_col_items = 0, col_threads = 32;
   int* adj_rows = nullptr;
   int n_adj_rows = 0;
   void* adj_part = nullptr;  // level-chunk partial sums of those rows (3 * chunks * rows * I)
@@ -1382,6 +1384,21 @@ int ensure_adj(agcm_state* s) {
   };
   s->adj_items = put_ints(items);
   s->n_adj_items = (int)items.size();
+  std::vector<int4> citems;  // the rows that read their pair from global memory first
+  for (int wide = 1; wide >= 0; --wide)
+    for (int j = 0; j < g->J; ++j) {
+      int H = agcm::adj_col_halo(g->Mu[j]), n = 0, S = 0;
+      agcm::row_segments(g->I, H, agcm::kRowB, &n, &S);
+      if ((n == 0) != (wide != 0)) continue;
+      if (wide) agcm::row_segments(g->I, H = 4, agcm::kRowB, &n, &S);
+      for (int q = 0; q < g->I; q += S) {
+        const int own = std::min(S, g->I - q);
+        citems.push_back(make_int4(wide << 24 | j, q, own, H));
+        s->col_threads = std::max(s->col_threads, (own + 2 * H + 31) & ~31);
+      }
+    }
+  s->col_items = put_ints(citems);
+  s->n_col_items = (int)citems.size();
   s->adj_rows = put_ints(rows);
   s->n_adj_rows = (int)rows.size();
   if (!rows.empty()) {
@@ -1418,18 +1435,20 @@ int vjp(agcm_state* s, void* const x[4], const void* const y[4], void* const out
   const agcm::AdjCol<T> c{(T*)s->W, (T*)s->psi, (T*)s->adj3[0], (T*)s->adj3[1], (T*)s->adj2[0], (T*)s->adj2[1]};
   s->prof.begin(KID_ADJ_COL, st);
   const dim3 cgrid((unsigned)((G.I + 31) / 32), (unsigned)G.J);
-  // level groups of at most kColL levels, 32 x ng threads (the kernel's bound is 256)
-  const int ng = (G.K + agcm::kColL - 1) / agcm::kColL;
-  if (ng <= 8) {
-    const size_t smem = ((7 + 5 * agcm::kColL) * ng * 32 + agcm::kLN * G.K) * sizeof(T);
+  const size_t csmem = agcm::adj_col_smem<T>(G.K);
+  // up to some 200 levels.  The other form at 128 x 64 x 120: FP32 71 us against
+  // 42, FP64 368 against 313; at 256 x 128 x 100 94 against 107, 1091 against 792.
+  if (csmem <= 227 * 1024) {
     static std::atomic<size_t> attr{0};  // the size set so far
-    if (attr.load() < smem) {
-      CUDA_TRY(cudaFuncSetAttribute(agcm::k_adj_col<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      attr.store(smem);
+    if (attr.load() < csmem) {
+      CUDA_TRY(cudaFuncSetAttribute(agcm::k_adj_col<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
+      attr.store(csmem);
     }
-    agcm::k_adj_col<T><<<cgrid, dim3(32, ng), smem, st>>>(
-        G, (const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)x[3], cs, (const T*)y[0], (const T*)y[1],
-        (const T*)y[2], (const T*)y[3], c);
+    bool vec = G.I % 4 == 0;
+    for (int f = 0; f < 3; ++f) vec = vec && ((uintptr_t)x[f] & 15) == 0 && ((uintptr_t)y[f] & 15) == 0;
+    const agcm::AdjColArgs<T> ca{(const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)x[3], (const T*)y[0],
+                                 (const T*)y[1], (const T*)y[2], (const T*)y[3], s->col_items, vec ? 1 : 0};
+    agcm::k_adj_col<T><<<(unsigned)s->n_col_items, s->col_threads, csmem, st>>>(G, cs, ca, c);
   } else {
     agcm::k_adj_col_w<T><<<cgrid, dim3(32, agcm::kColG), 0, st>>>(
         G, (const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)x[3], cs, (const T*)y[0], (const T*)y[1],
