@@ -282,6 +282,7 @@ inline void leap1_band(const agcm_grid* g, int* lo, int* hi) {
 struct RowPlan {
   int B = agcm::kRowB;
   bool pair = true;
+  bool two = true;  // with pairs: two short remainders may share a CTA
   int nsm = 152;
 };
 
@@ -295,7 +296,7 @@ struct RowPlan {
 // item.
 inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>* items, int off[3], int cnt[3],
                      int cls[agcm::kRowCls + 1]) {
-  std::vector<int4> pairs, polar, single[agcm::kRowCls];
+  std::vector<int4> pairs, polar, single[agcm::kRowCls], half;
   std::vector<int> polar_rows;
   size_t nseg = 0;
   int threads = 32;
@@ -310,10 +311,29 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
     if (n > 0) {
       const int c = eq && !plan.pair && Mu <= 7 ? agcm::kRowCls - 1 - Mu / 2 : 0;
       std::vector<int4>& list = pair ? pairs : single[c];
-      for (int q = 0; q < g->I; q += S) {
-        const int own = std::min(S, g->I - q);
-        list.push_back(make_int4((pair ? agcm::kRowPair : agcm::kRowAny) << 24 | j, q, own, H));
-        ++nseg;
+      const int kind = (pair ? agcm::kRowPair : agcm::kRowAny) << 24;
+      int end = g->I;
+      nseg += (size_t)n;
+      // full segments and half a CTA, where that takes no more warps than equal segments
+      const int full = (agcm::kRowB - 2 * H) & ~3, rem = g->I % full, nf = g->I / full;
+      auto warps = [&](int own) { return (own + 2 * H + 31) / 32; };
+      if (plan.two && plan.pair && plan.B == agcm::kRowB && rem > 0 && rem + 2 * H <= agcm::kRowB / 2 &&
+          nf * warps(full) + warps(rem) <= n * warps(S)) {
+        end = nf * full;
+        S = full;
+        threads = agcm::kRowB;
+        auto other = std::find_if(half.begin(), half.end(), [&](const int4& v) { return v.x >> 24 == kind >> 24 && v.w == H; });
+        if (other == half.end()) {
+          half.push_back(make_int4(kind | j, end, rem, H));
+        } else {
+          other->w |= (j + 1) << 8;
+          list.push_back(*other);
+          half.erase(other);
+        }
+      }
+      for (int q = 0; q < end; q += S) {
+        const int own = std::min(S, end - q);
+        list.push_back(make_int4(kind | j, q, own, H));
         threads = std::max(threads, (own + 2 * H + 31) & ~31);
       }
       j += pair ? 1 : 0;
@@ -322,6 +342,7 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
       polar_rows.push_back(j);
     }
   }
+  for (const int4& v : half) (v.x >> 24 == agcm::kRowPair ? pairs : single[0]).push_back(v);
   // The rows next to the poles: in a grid of two waves of CTAs and more their
   // work counts, else the latency of these few blocks does (33 against 22 us a
   // stage at 256x128x30, 48 against 33 at 360x180x30; 294 against 314 at
@@ -356,7 +377,12 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
 // Single rows in CTAs of the width that leaves
 // the fewest warps on the busiest of an SM's four schedulers, the narrowest
 // among equals (FP64 128x64x8, 64 threads: 52 us), up to three CTAs an SM.
-inline RowPlan row_plan(const agcm_grid* g) {
+// Remainders of two rows in one CTA where that saves a wave of CTAs (per_sm on
+// an SM) or there are many (405x203x26 FP32: 497 -> 452 CTAs for 456 places, 44
+// -> 36 us a stage; 750x375x20: 81 -> 78; 1000x500x20: 115 -> 111); with the
+// same few waves the equal segments' lighter CTAs are as good (640x320x30: 78.4
+// against 79.4 us, 500x250x30: 53.0 against 53.8).
+inline RowPlan row_plan(const agcm_grid* g, int per_sm) {
   RowPlan p;
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -367,8 +393,15 @@ inline RowPlan row_plan(const agcm_grid* g) {
   p.nsm = nsm;
   std::vector<int4> items;
   int off[3], cnt[3], cls[agcm::kRowCls + 1];
+  p.two = false;
   row_lists(g, p, &items, off, cnt, cls);
-  if ((long long)g->I * g->J >= kRowMinCols && (int)items.size() >= 2 * nsm) return p;
+  if ((long long)g->I * g->J >= kRowMinCols && (int)items.size() >= 2 * nsm) {
+    const size_t slots = (size_t)per_sm * nsm, n = items.size();
+    p.two = true;
+    row_lists(g, p, &items, off, cnt, cls);
+    p.two = n >= 5 * slots || (items.size() + slots - 1) / slots < (n + slots - 1) / slots;
+    return p;
+  }
   p.pair = false;
   int best = 0;
   for (int B : {128, 96, 64}) {
@@ -509,7 +542,7 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   size_t o_rt0 = putT(rt0pit), o_pit = putT(g->pit);
   size_t o_bu = putI(filtU), o_bv = putI(filtV);
   agcm::Geom<T> G{};
-  const RowPlan plan = row_plan(g);
+  const RowPlan plan = row_plan(g, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64);
   std::vector<int4> items;
   G.rowT = row_lists(g, plan, &items, G.off, G.cnt, G.cls);
   G.nitems = (int)items.size();
@@ -1679,7 +1712,7 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   T* rowtab = (T*)(base + kOffRowT + 12 * kRowB);
   double* rAz = (double*)(base + kOffRowT + (12 + agcm::kRowTabN) * kRowB);
   agcm::Geom<T> G{};
-  const RowPlan plan = row_plan(g);
+  const RowPlan plan = row_plan(g, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64);
   std::vector<int4> items;  // host only
   G.rowT = row_lists(g, plan, &items, G.off, G.cnt, G.cls);
   G.nitems = (int)items.size();
@@ -1839,7 +1872,9 @@ void fill_desc(agcm_ensemble* e) {
     const agcm_grid* g = e->members[m]->grid;
     std::vector<int4> items;
     int off[3], cnt[3], cls[agcm::kRowCls + 1];
-    row_lists(g, row_plan(g), &items, off, cnt, cls);
+    RowPlan plan = row_plan(g, AGCM_ROW_MINB);
+    plan.two = false;  // the member's number stands in the item
+    row_lists(g, plan, &items, off, cnt, cls);
     for (int4 it : items) {
       it.w |= (int)m << 8;
       e->host_items.push_back(it);
