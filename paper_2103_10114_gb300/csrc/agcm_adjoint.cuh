@@ -321,11 +321,12 @@ __global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
   // element offsets fit 32 bits: nlon * nlat * nlev <= 4e9
   const unsigned plane = (unsigned)J * (unsigned)I, vplane = (unsigned)(J - 1) * (unsigned)I;
   const unsigned r2 = (unsigned)j * (unsigned)I;
-  // a quarter of the threads each: a chunk of four columns of two rows
-  const int tr = NTW >> 2, cr = t / tr, cc = 4 * (t - cr * tr);
+  // a quarter of the threads each: four columns of two rows, as the stage
+  // kernel stages them (next to each other, or tr apart where rows are not aligned)
+  const int tr = NTW >> 2, cr = t / tr, cc = (a.vec ? 4 : 1) * (t - cr * tr);
   int c4 = cstart + cc;
   while (c4 >= I) c4 -= I;
-  const int sw = min(I - c4, 4);  // the first element past the periodic seam
+  const unsigned turns = a.vec ? 0u : row_turns(c4, tr, I);
   const bool vr = cr == 1 || cr == 2;  // V, yV; quarters 0 and 3: U, yU and Phi, yPhi
   const bool in = cc < NT, ok0 = in && (!vr || hasN), ok1 = in && (!vr || hasS);
   const T* const f0 = cr == 0 ? a.U : (cr == 1 ? a.V : (cr == 2 ? a.yV : a.Phi));
@@ -344,9 +345,9 @@ __global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
     } else {
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const unsigned x = e < sw ? e : e - I;
-        copy_elem_g2s<sizeof(T)>(d + e * sizeof(T), f0 + (p + (ok0 ? o0 + x : 0u)), true, ok0);
-        copy_elem_g2s<sizeof(T)>(d + (NTP + e) * sizeof(T), f1 + (p + (ok1 ? o1 + x : 0u)), true, ok1);
+        const unsigned x = e * tr - (turns >> 8 * e & 255u) * I, de = d + (unsigned)(e * tr * (int)sizeof(T));
+        copy_elem_g2s<sizeof(T)>(de, f0 + (p + (ok0 ? o0 + x : 0u)), true, ok0);
+        copy_elem_g2s<sizeof(T)>(de + NTP * sizeof(T), f1 + (p + (ok1 ? o1 + x : 0u)), true, ok1);
       }
     }
   };
@@ -939,15 +940,16 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
   // Staged rows of a level: 3 f + r, field f = U, Phi, V, yU, yPhi, yV, row r =
   // j-1, j, j+1; then 18, 19 psi, 20, 21 Dbar, 22, 23 W at j, j+1, 24 the
   // adjoint of Phi, 25..27 the stage sum's U, Phi, V of the level above.  A
-  // quarter of the threads each: a thread one chunk of four columns of seven
-  // rows.  Rows outside the grid are zeros.
-  const int tr = NTW >> 2, cr = t / tr, cc = 4 * (t - cr * tr);
+  // quarter of the threads each: a thread four columns of seven rows, next to
+  // each other, or tr apart where rows are not aligned.  Rows outside the grid
+  // are zeros.
+  const int tr = NTW >> 2, cr = t / tr, cc = (a.vec ? 4 : 1) * (t - cr * tr);
   int c4 = cstart + cc;
   while (c4 >= I) c4 -= I;
-  const int sw = min(I - c4, 4);  // the first element past the periodic seam
+  const unsigned turns = a.vec ? 0u : row_turns(c4, tr, I);
   const int jr = cr < 3 ? j + cr - 1 : j;
   const bool in = cc < NT, ok3 = in && jr >= 0 && jr < J, okv = in && jr >= 0 && jr < J - 1;
-  const bool oks = in && hasS, okr = in && cc >= H && cc < H + own;
+  const bool oks = in && hasS, okr = in && (!a.vec || (cc >= H && cc < H + own));
   const unsigned so = (unsigned)(ok3 ? jr : j) * (unsigned)I + (unsigned)c4, ro = r2 + (unsigned)c4;
   const unsigned ring_s = smem_addr(ring);
   auto chunk = [&](auto vec, int row, int s, const T* src, bool ok) __attribute__((always_inline)) {
@@ -958,7 +960,8 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
     } else {
 #pragma unroll
       for (int e = 0; e < 4; ++e)
-        copy_elem_g2s<sizeof(T)>(d + e * sizeof(T), src + (e < sw ? e : e - I), true, ok);
+        copy_elem_g2s<sizeof(T)>(d + (unsigned)(e * tr * (int)sizeof(T)), src + (e * tr - (int)(turns >> 8 * e & 255u) * I),
+                                 true, ok);
     }
   };
   auto issue_form = [&](auto vec, int k, int s) __attribute__((always_inline)) {
