@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
     k_adj_col(const __grid_constant__ Geom<T> g, const __grid_constant__ ColState<T> cs,
               const __grid_constant__ AdjColArgs<T> a, const __grid_constant__ AdjCol<T> o) {
   extern __shared__ __align__(128) unsigned char smem[];
+  pdl_launch();
   constexpr int R = ColRing<T>::R, NTP = kRowB, kKeep = ColRing<T>::kKeep;
   const int I = g.I, J = g.J, K = g.K;
   const int4 item = a.items[blockIdx.x];
@@ -351,6 +352,7 @@ __global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
       }
     }
   };
+  pdl_wait();  // the launches before this one have written the P family and ybar
   for (int s = 0; s < R; ++s) {
     if (s < K) issue_level(s, s);
     copy_commit();
@@ -996,6 +998,7 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
     else
       issue_form(std::false_type{}, k, s);
   };
+  pdl_wait();  // the column pass is done
   for (int s = 0; s < R; ++s) {
     if (s < K) issue_level(s, s);
     copy_commit();
@@ -1259,6 +1262,7 @@ __global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_R
                const __grid_constant__ AdjRowArgs<T> a, const __grid_constant__ AdjM<T> m,
                const __grid_constant__ AdjOut<T> o, const int nany) {
   extern __shared__ __align__(128) unsigned char smem[];
+  pdl_launch();
   const int4 item = a.items[blockIdx.x];
   if ((int)blockIdx.x >= nany)
     adj_row<T, true>(g, cs, a, m, o, item, smem);
@@ -1272,8 +1276,10 @@ template <class T>
 __global__ void __launch_bounds__(256) k_adj_colstate(Geom<T> g, AdjM<T> m, const T* __restrict__ aPiD,
                                                       AdjOut<T> o) {
   const int I = g.I, J = g.J;
+  pdl_launch();
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= I * J) return;
+  pdl_wait();
   const int j = n / I, i = n - j * I;
   T mb = m.mcb[n] + T(0.5) * (m.mub[n] + m.mub[j * I + wrapi(i - 1, I)]);
   if (j < J - 1) mb += T(0.5) * m.mvb[n];

@@ -220,7 +220,7 @@ struct agcm_state {
   void* x[3][4] = {};
   // adjoint forward-recompute scratch (allocated with the adjoint workspace):
   // P, rP, Pu, rPu, Pv, rPv (2-D), W ((K+1) planes), psi
-  void* col[6] = {};
+  void* col[6] = {};  // P family of the three stage states, last stage first
   void* W = nullptr;
   void* psi = nullptr;
   // FP64 vertical means sum_k dsigma U_k and V_k of x[0..2] (J*I each), the
@@ -1382,7 +1382,7 @@ int ensure_adj(agcm_state* s) {
     return p;
   };
   // forward recompute (phases A, B) at the stage states
-  for (auto& p : s->col) p = get(n2);
+  for (auto& p : s->col) p = get(3 * n2);  // of the three stage states
   s->W = get(nw);
   s->psi = get(n3);
   for (auto& p : s->adj3) p = get(n3);
@@ -1449,22 +1449,43 @@ int ensure_adj(agcm_state* s) {
   return AGCM_OK;
 }
 
+// A launch; dependent: it may start before the launch before it has ended (the
+// kernel waits for that itself).
+template <class... P, class... A>
+cudaError_t launch(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, bool dependent, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+template <class T>
+agcm::ColState<T> colstate_of(const agcm_state* s) {
+  return {(T*)s->col[0], (T*)s->col[1], (T*)s->col[2], (T*)s->col[3], (T*)s->col[4], (T*)s->col[5]};
+}
+
 // out = (accumulate ? out : 0) + scale * J(x)^T y, J the Jacobian of T at x;
 // with sum != nullptr also sum = sum_in + scale * J(x)^T y (sum_in defaults
 // to sum itself).  No atomics and no
-// zeroing: the P family, the column pass (phase B at x and its transpose),
+// zeroing, the P family (of all stages, `stage` this one) being there: the
+// column pass (phase B at x and its transpose),
 // the gathered adjoint of every point (row segments, and the rows past their
-// halo on the second stream), the adjoint of pi.
+// halo on the second stream), the adjoint of pi.  Each kernel's launch and
+// set-up overlap the end of the one before it (dependent launches).
 template <class T>
-int vjp(agcm_state* s, void* const x[4], const void* const y[4], void* const out[4], double scale, int accumulate,
+int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void* const out[4], double scale, int accumulate,
         cudaStream_t st, void* const* sum = nullptr, const void* const* sum_in = nullptr) {
   if (!sum_in) sum_in = sum;
   const agcm::Geom<T>& G = geom_of<T>(s);
   const size_t n2 = s->n2;
-  agcm::ColState<T> cs{(T*)s->col[0], (T*)s->col[1], (T*)s->col[2], (T*)s->col[3], (T*)s->col[4], (T*)s->col[5]};
-  s->prof.begin(KID_COLSTATE, st);
-  agcm::k_colstate<T><<<nblocks(n2, 256), 256, 0, st>>>(G, (const T*)x[3], cs);
-  s->prof.end(st);
+  const agcm::ColState<T> cs = colstate_of<T>(s).at(stage * n2);
   const agcm::AdjCol<T> c{(T*)s->W, (T*)s->psi, (T*)s->adj3[0], (T*)s->adj3[1], (T*)s->adj2[0], (T*)s->adj2[1]};
   s->prof.begin(KID_ADJ_COL, st);
   const dim3 cgrid((unsigned)((G.I + 31) / 32), (unsigned)G.J);
@@ -1481,7 +1502,7 @@ int vjp(agcm_state* s, void* const x[4], const void* const y[4], void* const out
     for (int f = 0; f < 3; ++f) vec = vec && ((uintptr_t)x[f] & 15) == 0 && ((uintptr_t)y[f] & 15) == 0;
     const agcm::AdjColArgs<T> ca{(const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)x[3], (const T*)y[0],
                                  (const T*)y[1], (const T*)y[2], (const T*)y[3], s->col_items, vec ? 1 : 0};
-    agcm::k_adj_col<T><<<(unsigned)s->n_col_items, s->col_threads, csmem, st>>>(G, cs, ca, c);
+    CUDA_TRY(launch(agcm::k_adj_col<T>, dim3((unsigned)s->n_col_items), s->col_threads, csmem, st, true, G, cs, ca, c));
   } else {
     agcm::k_adj_col_w<T><<<cgrid, dim3(32, agcm::kColG), 0, st>>>(
         G, (const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)x[3], cs, (const T*)y[0], (const T*)y[1],
@@ -1531,7 +1552,8 @@ int vjp(agcm_state* s, void* const x[4], const void* const y[4], void* const out
     const agcm::AdjRowArgs<T> ra{(const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)y[0], (const T*)y[1],
                                  (const T*)y[2], c.W, c.psi, c.Db, c.aPhi, c.arP, r[0], r[1], r[2], s->adj_items,
                                  vec ? 1 : 0};
-    agcm::k_adj_rows<T><<<(unsigned)s->n_adj_items, s->adj_threads, smem, st>>>(G, cs, ra, m, o, s->n_adj_any);
+    CUDA_TRY(launch(agcm::k_adj_rows<T>, dim3((unsigned)s->n_adj_items), s->adj_threads, smem, st, true, G, cs, ra, m, o,
+                    s->n_adj_any));
   }
   if (fork) {
     CUDA_TRY(cudaEventRecord(s->ev_join[0], s->aux[0]));
@@ -1539,7 +1561,7 @@ int vjp(agcm_state* s, void* const x[4], const void* const y[4], void* const out
   }
   s->prof.end(st);
   s->prof.begin(KID_ADJ_COLSTATE, st);
-  agcm::k_adj_colstate<T><<<nblocks(n2, 256), 256, 0, st>>>(G, m, (const T*)s->adj2[1], o);
+  CUDA_TRY(launch(agcm::k_adj_colstate<T>, dim3(nblocks(n2, 256)), 256, 0, st, !fork, G, m, (const T*)s->adj2[1], o));
   s->prof.end(st);
   CUDA_TRY(cudaGetLastError());
   return AGCM_OK;
@@ -1557,11 +1579,15 @@ int adjoint_step(agcm_state* s, const void* const lam_in[4], void* const lam_out
   if ((rc = fused_stage<T, 2>(s, 1, s->x[2], 2, 0.5 * dt, st))) return rc;
   void* const* mu2 = s->mu[0];
   void* const* mu1 = s->mu[1];
+  s->prof.begin(KID_COLSTATE, st);
+  const agcm::ColPi<T> states{{(const T*)s->x[2][3], (const T*)s->x[1][3], (const T*)s->x[0][3]}};
+  agcm::k_colstate<T><<<dim3(nblocks(s->n2, 256), 3), 256, 0, st>>>(geom_of<T>(s), states, colstate_of<T>(s));
+  s->prof.end(st);
   // each product also adds itself to lam_out (no separate accumulation
   // pass); the first forms lam_out = lam_in + mu2 (no copy of lam_in)
-  if ((rc = vjp<T>(s, s->x[2], lam_in, mu2, dt, 0, st, lam_out, lam_in))) return rc;
-  if ((rc = vjp<T>(s, s->x[1], mu2, mu1, 0.5 * dt, 0, st, lam_out))) return rc;
-  return vjp<T>(s, s->x[0], mu1, lam_out, 0.5 * dt, 1, st);
+  if ((rc = vjp<T>(s, 0, s->x[2], lam_in, mu2, dt, 0, st, lam_out, lam_in))) return rc;
+  if ((rc = vjp<T>(s, 1, s->x[1], mu2, mu1, 0.5 * dt, 0, st, lam_out))) return rc;
+  return vjp<T>(s, 2, s->x[0], mu1, lam_out, 0.5 * dt, 1, st);
 }
 
 }  // namespace

@@ -17,11 +17,18 @@ namespace agcm {
 template <class T>
 struct ColState {  // phase-A outputs, J*I each (Pv/rPv: (J-1)*I)
   T *P, *rP, *Pu, *rPu, *Pv, *rPv;
+  __host__ __device__ ColState at(size_t n) const { return {P + n, rP + n, Pu + n, rPu + n, Pv + n, rPv + n}; }
+};
+template <class T>
+struct ColPi {  // pi of the three stage states, one launch for all
+  const T* pi[3];
 };
 
 template <class T>
-__global__ void __launch_bounds__(256) k_colstate(Geom<T> g, const T* __restrict__ pi, ColState<T> cs) {
+__global__ void __launch_bounds__(256) k_colstate(Geom<T> g, ColPi<T> states, ColState<T> cs) {
   const int I = g.I, J = g.J;
+  const T* __restrict__ pi = states.pi[blockIdx.y];
+  cs = cs.at((size_t)blockIdx.y * I * J);
   const int n = blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= I * J) return;
   const int j = n / I, i = n - j * I;
