@@ -284,6 +284,7 @@ struct RowPlan {
   bool pair = true;
   bool two = true;  // with pairs: two short remainders may share a CTA
   int nsm = 152;
+  size_t slots = 0;  // CTAs that the GPU holds at a time (0: the rows next to the poles are not cut to fit)
 };
 
 // Work items of the row-segment stage kernel (agcm_row.cuh): pairs of
@@ -347,7 +348,12 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
   // work counts, else the latency of these few blocks does (33 against 22 us a
   // stage at 256x128x30, 48 against 33 at 360x180x30; 294 against 314 at
   // 1440x720x30 the other way).
-  const int cols = nseg >= (size_t)6 * plan.nsm ? agcm::kRowB : 32;
+  // Half as many columns, twice the groups of levels, where that fits beside
+  // the rows in one wave (256x128x30: 23.4 -> 21.3 us a stage, 16 levels 18.3 ->
+  // 17.6, 12 levels 17.2 -> 17.9; 405x203x26, which it would take to a second
+  // wave, 35 -> 45).
+  const bool fits = g->K >= 16 && nseg + polar_rows.size() * (size_t)((g->I + 15) / 16) <= plan.slots;
+  const int cols = nseg >= (size_t)6 * plan.nsm ? agcm::kRowB : (fits ? 16 : 32);
   for (int j : polar_rows)
     for (int q = 0; q < g->I; q += cols) polar.push_back(make_int4(agcm::kRowPolar << 24 | j, q, cols, 0));
   items->clear();
@@ -391,15 +397,17 @@ inline RowPlan row_plan(const agcm_grid* g, int per_sm) {
     nsm = p.nsm;
   }
   p.nsm = nsm;
+  const size_t slots = (size_t)per_sm * nsm;
   std::vector<int4> items;
   int off[3], cnt[3], cls[agcm::kRowCls + 1];
   p.two = false;
   row_lists(g, p, &items, off, cnt, cls);
   if ((long long)g->I * g->J >= kRowMinCols && (int)items.size() >= 2 * nsm) {
-    const size_t slots = (size_t)per_sm * nsm, n = items.size();
+    const size_t n = items.size();
     p.two = true;
     row_lists(g, p, &items, off, cnt, cls);
     p.two = n >= 5 * slots || (items.size() + slots - 1) / slots < (n + slots - 1) / slots;
+    p.slots = slots;
     return p;
   }
   p.pair = false;
@@ -418,6 +426,7 @@ inline RowPlan row_plan(const agcm_grid* g, int per_sm) {
       best = cost;
     }
   }
+  p.slots = slots;
   return p;
 }
 

@@ -71,24 +71,26 @@ constexpr int kTileX = 32;  // columns of one warp (one block) of the stage kern
 // NL: Eq. 1's delta kappa Phi/P term is on; every Phi/P that enters psi or
 // the Omega~ coefficient is scaled by 1 + rho_k Phi/P.
 //
-// NW > 1 and xch not null: the levels are shared out over NW warps of the
-// block (w = 0 the surface's), which hold the same 32 columns.  A warp first sums its levels'
-// contributions to the suffix sums, the warps exchange them through xch
-// ([NW][5][32] values of T, added in warp order), and each walks its own
-// levels with the sums of the warps below; the fields of the level below its
+// POL: a row next to a pole, in a block of the row-segment kernel.  xch not
+// null: the levels are shared out over nw groups of threads of the block (w = 0
+// the surface's), which hold the same columns (lane).  A group first sums its
+// levels' contributions to the suffix sums, the groups exchange them through xch
+// ([nw][5][columns] values of T, added in group order), and each walks its own
+// levels with the sums of the groups below; the fields of the level below its
 // first and above its last are read once more.  The chain of K levels, which
-// is all the time that a few rows take, becomes K / NW levels and a short
+// is all the time that a few rows take, becomes K / nw levels and a short
 // pass.  act: false for a column past the row's end (computed, not stored).
-template <class T, int MODE, int TERMS = 3, bool NL = false, bool L1 = false, int NW = 1>
+template <class T, int MODE, int TERMS = 3, bool NL = false, bool L1 = false, bool POL = false>
 __device__ __forceinline__ void fused_column(
     const Geom<T>& g, const int i, const int j, const T* __restrict__ U, const T* __restrict__ V,
     const T* __restrict__ Phi, const T* __restrict__ pi, const double* __restrict__ Ubar,
     const double* __restrict__ Vbar, const T* Ub, const T* Vb, const T* Phib, const T* pib, T* Uo, T* Vo, T* Phio,
     T* pio, double* Ubar_o, double* Vbar_o, const double* Ubar_b, const double* Vbar_b, const T cdt,
-    const int w = 0, T* xch = nullptr, const bool act = true) {
+    const int w = 0, const int nw = 1, const int lane = 0, T* xch = nullptr, const bool act = true) {
   const int I = g.I, J = g.J, K = g.K;
-  const bool split = NW > 1 && xch;
-  const int ke = split ? K - w * K / NW : K, kb = split ? K - (w + 1) * K / NW : 0;  // this warp's levels
+  const bool split = POL && xch;
+  const int ncol = split ? (int)blockDim.x / nw : 0;
+  const int ke = split ? K - w * K / nw : K, kb = split ? K - (w + 1) * K / nw : 0;  // this thread's levels
   constexpr bool ADV = (TERMS & 1) != 0, ADA = (TERMS & 2) != 0;
   const bool hasS = L1 || j < J - 1;   // V row j exists, scalar row j+1 exists
   const bool hasN = L1 || j > 0;       // V row j-1 exists
@@ -181,7 +183,7 @@ __device__ __forceinline__ void fused_column(
     Cs = ((double)PugE * Ubar[rjp + gE] - (double)PugW * Ubar[rjp + gW]) * (double)rdxs +
          ((hasSS ? (double)svjp * (double)Pvs * Vbar[rjp + i] : 0.0) - (double)svj * (double)Pvc * Vbar[rj + i]) *
              (double)rdys;
-  if (NW > 1 && (w > 0 || !act)) {
+  if (POL && (w > 0 || !act)) {
   } else if (MODE == 0)
     pio[rj + i] = ADA ? (T)(-Cc) : T(0);
   else {
@@ -203,7 +205,7 @@ __device__ __forceinline__ void fused_column(
   T dubar = T(0), dvbar = T(0);
 
   if (split) {
-    // the warps' sums over their levels, and the levels below this warp's
+    // the groups' sums over their levels, and the levels below this group's
     T p[5] = {0, 0, 0, 0, 0};
 #pragma unroll 2
     for (int k = ke - 1; k >= kb; --k) {
@@ -222,16 +224,15 @@ __device__ __forceinline__ void fused_column(
       p[3] += hk * (B(rPE1 * Phk[rj + fE1]) - B(rPW1 * Phk[rj + fW1]));
       if (hasS) p[4] += hk * (B(rPs * Phk[rjp + i]) - B(rPc * Phk[rj + i]));
     }
-    const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int q = 0; q < 5; ++q) xch[(w * 5 + q) * 32 + lane] = p[q];
+    for (int q = 0; q < 5; ++q) xch[(w * 5 + q) * ncol + lane] = p[q];
     __syncthreads();
     for (int v = 0; v < w; ++v) {
-      SD += xch[(v * 5 + 0) * 32 + lane];
-      SDp += xch[(v * 5 + 1) * 32 + lane];
-      SDs += xch[(v * 5 + 2) * 32 + lane];
-      dSU += xch[(v * 5 + 3) * 32 + lane];
-      dSV += xch[(v * 5 + 4) * 32 + lane];
+      SD += xch[(v * 5 + 0) * ncol + lane];
+      SDp += xch[(v * 5 + 1) * ncol + lane];
+      SDs += xch[(v * 5 + 2) * ncol + lane];
+      dSU += xch[(v * 5 + 3) * ncol + lane];
+      dSV += xch[(v * 5 + 4) * ncol + lane];
     }
     if (ke < K && kb < ke) {
       const T om = g.oms[ke];
@@ -262,7 +263,7 @@ __device__ __forceinline__ void fused_column(
     T nPPh = 0, nPU = 0, nPV = 0;
     T c_r2 = 0, c_ds = 0, nbU = 0, nbV = 0, nbPh = 0;
     double c_dsd = 0.0;
-    if (NW > 1 && k >= 0 && k < kb) {  // the level above the warp's last: its G only
+    if (POL && k >= 0 && k < kb) {  // the level above the group's last: its G only
       Gsc = Phi[(size_t)k * plane + o_own] * rPc;
       Guc = U[(size_t)k * plane + o_own] * rPuc;
       Gvc = hasS ? V[(size_t)k * vplane + o_own] * rPvc : T(0);
@@ -395,7 +396,7 @@ __device__ __forceinline__ void fused_column(
       const size_t o = (size_t)kk * plane + rj + i;
       const T bPh = MODE == 0 ? T(0) : pbPh, bU = MODE == 0 ? T(0) : pbU;
       const T oPh = bPh + cdt * TPh, oU = bU + cdt * TU;
-      if (NW == 1 || act) {
+      if (!POL || act) {
         Phio[o] = oPh;
         Uo[o] = oU;
       }
@@ -409,7 +410,7 @@ __device__ __forceinline__ void fused_column(
         const size_t ov = (size_t)kk * vplane + rj + i;
         const T bV = MODE == 0 ? T(0) : pbV;
         const T oV = bV + cdt * TV;
-        if (NW == 1 || act) Vo[ov] = oV;
+        if (!POL || act) Vo[ov] = oV;
         if (kInc)
           dvbar += p_ds * (oV - bV);
         else
@@ -433,14 +434,13 @@ __device__ __forceinline__ void fused_column(
     pbPh = nbPh;
   }
   if (MODE != 0 && split) {
-    const int lane = threadIdx.x & 31;
-    __syncthreads();  // every warp has read the sums
-    xch[(w * 5 + 0) * 32 + lane] = kInc ? dubar : (T)ubar;
-    xch[(w * 5 + 1) * 32 + lane] = kInc ? dvbar : (T)vbar;
+    __syncthreads();  // every group has read the sums
+    xch[(w * 5 + 0) * ncol + lane] = kInc ? dubar : (T)ubar;
+    xch[(w * 5 + 1) * ncol + lane] = kInc ? dvbar : (T)vbar;
     __syncthreads();
     if (w > 0) return;
-    for (int v = 1; v < NW; ++v) {
-      const T a = xch[(v * 5 + 0) * 32 + lane], b = xch[(v * 5 + 1) * 32 + lane];
+    for (int v = 1; v < nw; ++v) {
+      const T a = xch[(v * 5 + 0) * ncol + lane], b = xch[(v * 5 + 1) * ncol + lane];
       if (kInc) {
         dubar += a;
         dvbar += b;
@@ -450,7 +450,7 @@ __device__ __forceinline__ void fused_column(
       }
     }
   }
-  if (Ubar_o && (NW == 1 || act)) {
+  if (Ubar_o && (!POL || act)) {
     if (kInc) {
       ubar = Ubar_b[rj + i] + (double)dubar;
       if (hasS) vbar = Vbar_b[rj + i] + (double)dvbar;
