@@ -335,9 +335,8 @@ def main():
     # dominant kernel and its algorithmic bytes (one stage: 6/9/9 words per point -> 8 on average)
     name, (kms, kn) = max(prof.items(), key=lambda kv: kv[1][0])
     stage_bytes = pts * 8 * esz
-    # the profiler brackets each stage (the stride-1 row band and the other
-    # rows, two concurrent launches) with one pair of events: the roofline's
-    # unit is the stage
+    # the profiler brackets each stage with one pair of events: the roofline's
+    # unit is the stage (one launch here)
     n_stages = 3 * args.steps
     stage_ms = kms / n_stages
     achieved = stage_bytes / (stage_ms / 1e3) / 1e9 if name == "k_fused_stage" else None

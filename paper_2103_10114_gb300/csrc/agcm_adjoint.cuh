@@ -7,7 +7,8 @@
 //
 //   k_colstate    (agcm_phases.cuh) phase A at x: m = pi~ + pi, P = sqrt(m) and
 //                 its U/V-point values and reciprocals.
-//   k_adj_col     32 columns x level groups per block: phase B at x (the
+//   k_adj_col     one row segment per block, rows staged in shared memory, a
+//                 walk down and one up the levels: phase B at x (the
 //                 leap divergence D_k of Eq. 6, its column sum C, the sigma
 //                 mass flux W_h = sh_h C - sum_{k<h} ds_k D_k of Alg. 1 /
 //                 Alg. 2, the Omega~ factor S_k and the hydrostatic psi)

@@ -376,11 +376,10 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
   return threads;
 }
 
-// Pairs, as long as they make two CTAs an SM (before the set-up's loads were
-// gathered, 1440x720x30 FP32: 321 against 428 us a stage with single rows,
-// 720x360x30: 97 against 118, 405x203x26: 49 against 54); with fewer, single
-// rows (256x128x30: 33.5 against 35 us; FP64 128x64x8: 60 against 82 us).
-// Single rows in CTAs of the width that leaves
+// Pairs, as long as they make two CTAs an SM (720x360x30 FP32: 87 us a stage
+// against 114 with single rows, 512x256x26: 50 against 64, 405x203x26: 49
+// against 52); with fewer, single rows (256x128x30: 23.5 against 28.4 us; FP64
+// 128x64x8: 60 against 82 us).  Single rows in CTAs of the width that leaves
 // the fewest warps on the busiest of an SM's four schedulers, the narrowest
 // among equals (FP64 128x64x8, 64 threads: 52 us), up to three CTAs an SM.
 // Remainders of two rows in one CTA where that saves a wave of CTAs (per_sm on
@@ -737,7 +736,7 @@ int launch_fused(const agcm::Geom<T>& G, const void* const xs[4], const double* 
   const bool rowpath = choice != 1 && G.nitems > 0 && (choice == 2 || (long long)G.I * G.J >= kRowMinCols) && smem <= 227 * 1024;
   auto rows = [&](auto nl) -> int {
     if (rowpath) {
-      // 16-byte aligned rows are staged by bulk copies, others element by element
+      // 16-byte aligned rows are staged by 16-byte copies, others element by element
       bool vec = G.I % 4 == 0 && a16(xs[0]) && a16(xs[1]) && a16(xs[2]);
       if (MODE == 2) vec = vec && a16(xb[0]) && a16(xb[1]) && a16(xb[2]);
       agcm::RowArgs<T> ra{(const T*)xs[0], (const T*)xs[1], (const T*)xs[2], (const T*)xs[3], ub, vb,
@@ -1899,8 +1898,7 @@ void fill_desc(agcm_ensemble* e) {
     begin += d[m].nbx * ((s->grid->J + e->rows_per_item - 1) / e->rows_per_item);
   }
   e->nitems = begin;
-  // row-segment persistent launch: every member's row-segment items (any
-  // stride class), then 256-column chunks of the rows left to the column body
+  // row-segment persistent launch: every member's items
   e->host_items.clear();
   e->rows_smem = 0;
   for (size_t m = 0; m < e->members.size(); ++m) {

@@ -6,18 +6,16 @@ Two ways to advance the members, both captured whole in one CUDA graph:
 * "persistent": one launch of the ensemble kernel (agcm_ensemble_step), in
   one of two forms: one-warp blocks running the column body on items of 32
   columns of 1, 2 or 4 consecutive rows (its launch shape: how many blocks are
-  resident per SM, and the row tile); or 256-thread blocks (warps_per_block
-  8) running the row-segment body on (member, row segment) items, with the
-  rows near the poles on the column body;
+  resident per SM, and the row tile); or 128-thread blocks (warps_per_block
+  8 asks for them) running the row-segment body on (member, row segment)
+  items, with the rows near the poles on the column body;
 * "streams": each member stepped by the single-state kernel (agcm_step) with
   the members spread round-robin over N CUDA streams, so small members run
   side by side.  The single-state kernel reads its grid tables from the launch
-  parameters and fits in 80-96 registers, where the persistent kernel, which
-  reads each member's tables through a descriptor, needs 168.  "streams-row"
-  does the same with every member on the row-segment stage kernel
-  (agcm_state_set_stage_kernel 2): a small member alone would not fill the
-  GPU with row segments and takes the column kernel, but side by side with
-  the others its row segments are the cheaper work per point.
+  parameters, where the persistent kernel reads each member's through a
+  descriptor.  "streams-row" does the same with every member on the
+  row-segment stage kernel (agcm_state_set_stage_kernel 2), which the smallest
+  members (under 4096 columns) otherwise leave to the column kernel.
 
 The best choice depends on the member mix and the GPU, so `autotune` times
 each candidate on the ensemble itself and keeps the fastest (cached per
