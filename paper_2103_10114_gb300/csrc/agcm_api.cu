@@ -501,7 +501,7 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   filtU.push_back(0);
   filtV.push_back(0);
   // the row-segment kernel's level table and row tables
-  std::vector<double> lev((size_t)K * agcm::kLevN, 0.0), rowtab((size_t)J * agcm::kRowTabN, 0.0), rAz(J);
+  std::vector<double> lev((size_t)K * agcm::kLevN, 0.0), rowtab((size_t)J * agcm::kRowTabN, 0.0), rAz(2 * (size_t)J);
   for (int k = 0; k < K; ++k) {
     double* L = lev.data() + (size_t)k * agcm::kLevN;
     L[agcm::kLevDs] = g->ds[k];
@@ -525,7 +525,8 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
       L[agcm::kRtRvn] = g->Av[j] / g->A[j];
       L[agcm::kRtRvs] = g->Av[j] / g->A[j + 1];
     }
-    rAz[j] = (double)(T)zf[j] / g->A[j];
+    rAz[2 * j] = (double)(T)zf[j] / g->A[j];
+    rAz[2 * j + 1] = j > 0 ? agcm::edge_units((T)yv[j - 1], (T)zf[j - 1], (T)zf[j]) : 0.0;
   }
   std::vector<double> rt0pit((size_t)J * I);
   for (size_t n = 0; n < rt0pit.size(); ++n) rt0pit[n] = g->rts[n] / g->pit[n];
@@ -1626,7 +1627,7 @@ constexpr size_t kOffRawLev = kOffRaw + 6 * kRowB;   // sh ds Hkk hk beta (doubl
 constexpr size_t kOffPitRaw = kOffRawLev + 5 * kLevB;  // pi~, R T~_s (double)
 constexpr size_t kOffInt = kOffPitRaw + 2 * kColB;   // Mu Mv (int)
 constexpr size_t kOffRowT = kOffInt + 2 * kRowB;     // 12 typed row arrays, the row table of kRowTabN values, zf / A (double)
-constexpr size_t kOffLevT = kOffRowT + (13 + agcm::kRowTabN) * kRowB;   // 7 typed level arrays, the level table of kLevN values
+constexpr size_t kOffLevT = kOffRowT + (14 + agcm::kRowTabN) * kRowB;   // 7 typed level arrays, the level table of kLevN values
 constexpr size_t kOffDs3 = kOffLevT + (7 + agcm::kLevN) * kLevB;   // dsigma in three FP32 parts
 constexpr size_t kOffColT = kOffDs3 + 2 * kLevB;                    // pit, rt0pit (typed)
 constexpr size_t kOffBar = kOffColT + 2 * kColB;     // Ubar, Vbar (double)
@@ -1694,7 +1695,9 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
       L[agcm::kRtR2Av] = v ? rowT[9 * rowStride + j] : T(0);
       L[agcm::kRtRvn] = v ? (T)(Av[j] / A[j]) : T(0);
       L[agcm::kRtRvs] = v ? (T)(Av[j] / A[j + 1]) : T(0);
-      rAz[j] = (double)(T)(kA * dth / Mu[j]) / A[j];
+      const T zf = (T)(kA * dth / Mu[j]);
+      rAz[2 * j] = (double)zf / A[j];
+      rAz[2 * j + 1] = j > 0 ? agcm::edge_units((T)(kA * dlam * sv[j - 1]), (T)(kA * dth / Mu[j - 1]), zf) : 0.0;
     }
     if (n < (size_t)K) {
       const int k = (int)n;

@@ -1,0 +1,25 @@
+"""Mass of an FP32 run: what crosses a row edge leaves one row and enters the
+other, also where the rows' strides differ.  Over 300 steps the start of the
+jet moves some 1e-3 of the mass between the latitudes; a face length that
+differs by an FP32 rounding (6e-8) between the two rows of an edge shows as
+some 6e-11 of the total, the rounding of pi itself (6e-8 of |pi| ~ 1e-2 over
+sqrt(points)) below 2e-11 on these grids."""
+import pytest
+
+from paper_2103_10114_gb300 import agcm, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("grid", [(720, 360, 10), (405, 203, 6)], ids=lambda g: "%dx%dx%d" % g)
+def test_mass_is_kept_across_stride_changes(cuda_ok, grid):
+    agcm.build()
+    I, J, K = grid
+    st = inputs.baroclinic_jet(I, J, K, seed=3, noise=1e-3, terrain_seed=2)
+    g = agcm.Grid(I, J, K, phis=st["phis"])
+    s = agcm.State(g, agcm.AGCM_FP32)
+    s.load(st)
+    before = s.diagnostics()["mass"]
+    s.step(300, g.dt(100.0))
+    assert abs(s.diagnostics()["mass"] / before - 1.0) <= 4e-11
+    s.close()
