@@ -284,6 +284,7 @@ struct RowPlan {
   bool pair = true;
   bool two = true;  // with pairs: two short remainders may share a CTA
   int nsm = 152;
+  bool column = false;  // the column kernel is the faster one
   size_t slots = 0;  // CTAs that the GPU holds at a time (0: the rows next to the poles are not cut to fit)
 };
 
@@ -387,7 +388,7 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
 // -> 36 us a stage; 750x375x20: 81 -> 78; 1000x500x20: 115 -> 111); with the
 // same few waves the equal segments' lighter CTAs are as good (640x320x30: 78.4
 // against 79.4 us, 500x250x30: 53.0 against 53.8).
-inline RowPlan row_plan(const agcm_grid* g, int per_sm) {
+inline RowPlan row_plan(const agcm_grid* g, int per_sm, bool fp64) {
   RowPlan p;
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -426,6 +427,11 @@ inline RowPlan row_plan(const agcm_grid* g, int per_sm) {
     }
   }
   p.slots = slots;
+  // FP64: one warp's chain of FP64 issue is the time of a stage on such a grid;
+  // where the column kernel's warps are one to a scheduler and the row
+  // segments' two, the column kernel's is the shorter (180x90x30: 207 against
+  // 221 us a stage)
+  p.column = fp64 && best >= 2 && (long long)((g->I + 31) / 32) * g->J <= 4LL * nsm;
   return p;
 }
 
@@ -551,10 +557,11 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   size_t o_rt0 = putT(rt0pit), o_pit = putT(g->pit);
   size_t o_bu = putI(filtU), o_bv = putI(filtV);
   agcm::Geom<T> G{};
-  const RowPlan plan = row_plan(g, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64);
+  const RowPlan plan = row_plan(g, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64, sizeof(T) == 8);
   std::vector<int4> items;
   G.rowT = row_lists(g, plan, &items, G.off, G.cnt, G.cls);
   G.nitems = (int)items.size();
+  G.column = plan.column;
   items.push_back(make_int4(0, 0, 0, 0));
   size_t o_it = put(items.data(), items.size() * sizeof(int4));
 
@@ -734,7 +741,7 @@ int launch_fused(const agcm::Geom<T>& G, const void* const xs[4], const double* 
   // a state's own choice (agcm_state_set_stage_kernel), else the process's
   const int choice = state_choice > 0 ? state_choice : g_stage_choice.load(std::memory_order_relaxed);
   const size_t smem = agcm::row_smem_bytes<T>(G.K);
-  const bool rowpath = choice != 1 && G.nitems > 0 && (choice == 2 || (long long)G.I * G.J >= kRowMinCols) && smem <= 227 * 1024;
+  const bool rowpath = choice != 1 && G.nitems > 0 && (choice == 2 || ((long long)G.I * G.J >= kRowMinCols && !G.column)) && smem <= 227 * 1024;
   auto rows = [&](auto nl) -> int {
     if (rowpath) {
       // 16-byte aligned rows are staged by 16-byte copies, others element by element
@@ -1749,10 +1756,11 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   T* rowtab = (T*)(base + kOffRowT + 12 * kRowB);
   double* rAz = (double*)(base + kOffRowT + (12 + agcm::kRowTabN) * kRowB);
   agcm::Geom<T> G{};
-  const RowPlan plan = row_plan(g, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64);
+  const RowPlan plan = row_plan(g, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64, sizeof(T) == 8);
   std::vector<int4> items;  // host only
   G.rowT = row_lists(g, plan, &items, G.off, G.cnt, G.cls);
   G.nitems = (int)items.size();
+  G.column = plan.column;
   if (tables) {
   const std::vector<double>* rows[6] = {&g->s, &g->c, &g->cot, &g->A, &g->sv, &g->Av};
   for (int q = 0; q < 6; ++q)
@@ -1908,7 +1916,7 @@ void fill_desc(agcm_ensemble* e) {
     const agcm_grid* g = e->members[m]->grid;
     std::vector<int4> items;
     int off[3], cnt[3], cls[agcm::kRowCls + 1];
-    RowPlan plan = row_plan(g, AGCM_ROW_MINB);
+    RowPlan plan = row_plan(g, AGCM_ROW_MINB, false);
     plan.two = false;  // the member's number stands in the item
     row_lists(g, plan, &items, off, cnt, cls);
     for (int4 it : items) {

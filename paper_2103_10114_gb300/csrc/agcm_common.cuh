@@ -73,6 +73,7 @@ struct Geom {
   const int4* items;
   int off[3], cnt[3], cls[kRowCls + 1], nitems;
   int rowT;  // threads of a CTA that holds every item
+  int column;  // 1: the column kernel unless the row kernel is asked for
 };
 
 // Values per level of Geom::lev: dsigma, 4 beta Hkk, 4 beta hk, 2 beta hk /
