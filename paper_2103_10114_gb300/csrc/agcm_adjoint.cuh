@@ -366,18 +366,18 @@ __global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
   uw = uw < 0 ? uw + I : uw;
   const T rdx = g.rdx[j], rdy = g.rdy[j], rady = g.rady;
   const T svS = hasS ? ldg(g.sv + j) : T(0), svN = hasN ? ldg(g.sv + j - 1) : T(0);
-  const T PuE = ldg(cs.Pu + r2 + ue), PuW = ldg(cs.Pu + r2 + uw);
-  const T PvS = hasS ? ldg(cs.Pv + n) : T(0), PvN = hasN ? ldg(cs.Pv + n - I) : T(0);
+  const T PuE = cs.Pu[r2 + ue], PuW = cs.Pu[r2 + uw];
+  const T PvS = hasS ? cs.Pv[n] : T(0), PvN = hasN ? cs.Pv[n - I] : T(0);
   const T bS = svS * PvS, bN = svN * PvN;
-  const T rPc = ldg(cs.rP + n), rPu = ldg(cs.rPu + n), rPm = ldg(cs.rPu + r2 + (c > 0 ? c - 1 : I - 1));
-  const T rPvS = hasS ? ldg(cs.rPv + n) : T(0), rPvN = hasN ? ldg(cs.rPv + n - I) : T(0);
-  const T ps = ldg(g.rt0pit + n) * ldg(a.pi + n), rt = ldg(g.rt0pit + n), yp = ldg(a.ypi + n);
+  const T rPc = cs.rP[n], rPu = cs.rPu[n], rPm = cs.rPu[r2 + (c > 0 ? c - 1 : I - 1)];
+  const T rPvS = hasS ? cs.rPv[n] : T(0), rPvN = hasN ? cs.rPv[n - I] : T(0);
+  const T ps = ldg(g.rt0pit + n) * a.pi[n], rt = ldg(g.rt0pit + n), yp = a.ypi[n];
   T wu[4] = {0, 0, 0, 0};  // wide rows: U, yU at the pair, a level ahead
   if (wide) {
-    wu[0] = ldg(a.U + r2 + ue);
-    wu[1] = ldg(a.U + r2 + uw);
-    wu[2] = ldg(a.yU + r2 + ue);
-    wu[3] = ldg(a.yU + r2 + uw);
+    wu[0] = a.U[r2 + ue];
+    wu[1] = a.U[r2 + uw];
+    wu[2] = a.yU[r2 + ue];
+    wu[3] = a.yU[r2 + uw];
   }
   // ---- down: D, the adjoints of psi and W, prefix sums
   // sums over the levels in groups of kColB, each in two parts (whole groups,
@@ -399,10 +399,10 @@ __global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
       yw = wu[3];
       if (k + 1 < K) {
         const unsigned q = (unsigned)(k + 1) * plane + r2;
-        wu[0] = ldg(a.U + q + ue);
-        wu[1] = ldg(a.U + q + uw);
-        wu[2] = ldg(a.yU + q + ue);
-        wu[3] = ldg(a.yU + q + uw);
+        wu[0] = a.U[q + ue];
+        wu[1] = a.U[q + uw];
+        wu[2] = a.yU[q + ue];
+        wu[3] = a.yU[q + uw];
       }
     } else {
       Ue = raw[de];
@@ -476,8 +476,8 @@ __global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
 #pragma unroll
     for (int e = 0; e < B; ++e) {
       const unsigned q = (unsigned)max(kt - e, 0) * plane + n;
-      ph[e] = ldg(a.Phi + q);
-      yx[e] = ldg(a.yPhi + q);
+      ph[e] = a.Phi[q];
+      yx[e] = a.yPhi[q];
       if (kKeep == 1) kA[e] = o.Db[q];
     }
     T SD = 0, S = 0, SW = 0, SX = 0;  // of this group
@@ -1013,17 +1013,17 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
     const int jj = j - 1 + r;
     const bool ok = jj >= 0 && jj < J, kv = jj >= 0 && jj < J - 1;
     const unsigned n = ok ? (unsigned)jj * (unsigned)I + (unsigned)c : r2 + (unsigned)c;
-    rP[r] = ok ? ldg(cs.rP + n) : T(0);
-    rPu[r] = ok ? ldg(cs.rPu + n) : T(0);
+    rP[r] = ok ? cs.rP[n] : T(0);
+    rPu[r] = ok ? cs.rPu[n] : T(0);
     kP[r] = ok ? -ldg(g.r2A + jj) * rP[r] : T(0);
     kU[r] = ok ? T(-0.5) * ldg(g.r2A + jj) * rPu[r] : T(0);
-    const T Pu = ok && r > 0 ? ldg(cs.Pu + n) : T(0);
+    const T Pu = ok && r > 0 ? cs.Pu[n] : T(0);
     if (r == 1) Pu0 = Pu;
     // row j+1's flux carries V row j's face length
     if (r > 0) aF[r - 1] = r == 1 ? ldg(g.zf + j) * Pu : (hasS ? ldg(g.zfv + j) * Pu : T(0));
-    rPv[r] = kv ? ldg(cs.rPv + n) : T(0);
+    rPv[r] = kv ? cs.rPv[n] : T(0);
     kV[r] = kv ? T(-0.5) * ldg(g.r2Av + jj) * rPv[r] : T(0);
-    const T Pv = kv ? ldg(cs.Pv + n) : T(0);
+    const T Pv = kv ? cs.Pv[n] : T(0);
     if (r == 1) Pv0 = Pv;
     b[r] = kv ? ldg(g.yv + jj) * Pv : T(0);
   }
@@ -1044,7 +1044,7 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
 
   // ---- carries: sums over the levels, and of the level above: h / dsigma and
   // G, the adjoints so far, x and -ybar / (2 A) / dsigma (late terms)
-  T aPu = 0, arPu = 0, aPv = 0, arPv = 0, arP = owner ? ldg(a.arPcol + r2 + c) : T(0);
+  T aPu = 0, arPu = 0, aPv = 0, arPv = 0, arP = owner ? a.arPcol[r2 + c] : T(0);
   T hvU = 0, hvP = 0, hvV = 0, GuP = 0, GsP = 0, GvP = 0;
   T bU = 0, bP = 0, bV = 0, xU = 0, xP = 0, xV = 0, yrU = 0, yrP = 0, yrV = 0;
   const bool rmw = a.rU != nullptr;
@@ -1274,7 +1274,7 @@ __global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_R
 // pi-bar = direct psi part + m-bar, with m^u_i = (m_i + m_{i+1})/2 and
 // m^v_j = (m_j + m_{j+1})/2 transposed as gathers.
 template <class T>
-__global__ void __launch_bounds__(256) k_adj_colstate(Geom<T> g, AdjM<T> m, const T* __restrict__ aPiD,
+__global__ void __launch_bounds__(256) k_adj_colstate(Geom<T> g, AdjM<T> m, const T* aPiD,
                                                       AdjOut<T> o) {
   const int I = g.I, J = g.J;
   pdl_launch();
