@@ -949,22 +949,22 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
   const int tr = NTW >> 2, cr = t / tr, cc = (a.vec ? 4 : 1) * (t - cr * tr);
   int c4 = cstart + cc;
   while (c4 >= I) c4 -= I;
-  const unsigned turns = a.vec ? 0u : row_turns(c4, tr, I);
+  const unsigned turns = own_columns(cc, a.vec ? 1 : tr, H, own) | (a.vec ? 0u : row_turns(c4, tr, I));
   const int jr = cr < 3 ? j + cr - 1 : j;
   const bool in = cc < NT, ok3 = in && jr >= 0 && jr < J, okv = in && jr >= 0 && jr < J - 1;
-  const bool oks = in && hasS, okr = in && (!a.vec || (cc >= H && cc < H + own));
+  const bool oks = in && hasS;
   const unsigned so = (unsigned)(ok3 ? jr : j) * (unsigned)I + (unsigned)c4, ro = r2 + (unsigned)c4;
   const unsigned ring_s = smem_addr(ring);
-  auto chunk = [&](auto vec, int row, int s, const T* src, bool ok) __attribute__((always_inline)) {
+  auto chunk = [&](auto vec, int row, int s, const T* src, bool ok, bool inplace = false) __attribute__((always_inline)) {
     const unsigned d = ring_s + (unsigned)(((s * kAdjRaw + row) * NTP + cc) * (int)sizeof(T));
     if constexpr (decltype(vec)::value) {
 #pragma unroll
-      for (int e = 0; e < 4; e += 16 / (int)sizeof(T)) copy16_g2s(d + e * sizeof(T), src + e, true, ok);
+      for (int e = 0; e < 4; e += 16 / (int)sizeof(T)) copy16_g2s(d + e * sizeof(T), src + e, true, ok && (!inplace || turns & 128u));
     } else {
 #pragma unroll
       for (int e = 0; e < 4; ++e)
-        copy_elem_g2s<sizeof(T)>(d + (unsigned)(e * tr * (int)sizeof(T)), src + (e * tr - (int)(turns >> 8 * e & 255u) * I),
-                                 true, ok);
+        copy_elem_g2s<sizeof(T)>(d + (unsigned)(e * tr * (int)sizeof(T)), src + (e * tr - (int)(turns >> 8 * e & 127u) * I),
+                                 true, ok && (!inplace || turns >> 8 * e & 128u));
     }
   };
   auto issue_form = [&](auto vec, int k, int s) __attribute__((always_inline)) {
@@ -980,7 +980,7 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
       if (a.rU && k > 0) {  // quarter cr: field U, Phi, V
         const T* const r = cr == 0 ? a.rU : (cr == 1 ? a.rPhi : a.rV);
         const unsigned q = cr == 2 ? (hasS ? pv - vplane + ro : 0u) : p3 - plane + ro;
-        chunk(vec, 25 + cr, s, r + q, okr && (cr < 2 || hasS));
+        chunk(vec, 25 + cr, s, r + q, in && (cr < 2 || hasS), true);
       }
     } else {
       const unsigned q = p3 + ro, qs = oks ? q + I : q;
