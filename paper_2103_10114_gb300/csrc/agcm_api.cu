@@ -89,6 +89,16 @@ void dev_free(void* p) {
     cudaFree(p);
 }
 
+// A table from host memory into fresh device memory, there when this returns.
+// cudaMemcpy from pageable memory may return while the last of it is on its
+// way, and nothing orders a launch on a non-blocking stream behind it; and
+// memory from a caching allocator may still be written by what its last owner
+// queued on a stream of its own.
+bool upload(void* d, const void* h, size_t bytes) {
+  return cudaDeviceSynchronize() == cudaSuccess && cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
+         cudaStreamSynchronize(nullptr) == cudaSuccess;
+}
+
 // ---------------------------------------------------------------- constants
 // Reading R2: only the Earth radius is fixed by the paper (zonal grid-size table).
 constexpr double kA = 6.371e6;
@@ -567,7 +577,7 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
 
   void* d = dev_alloc(host.size());
   if (!d) return fail(AGCM_ENOMEM, "device allocation of %zu bytes for the grid tables failed", host.size());
-  if (cudaMemcpy(d, host.data(), host.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
+  if (!upload(d, host.data(), host.size())) {
     dev_free(d);
     return fail(AGCM_ECUDA, "copy of the grid tables failed: %s", cudaGetErrorString(cudaGetLastError()));
   }
@@ -1167,6 +1177,7 @@ int agcm_state_create(const agcm_grid_t* g, int precision, int nmembers, agcm_st
     delete s;
     return fail(AGCM_ENOMEM, "device allocation for a %zu x %zu x %zu state failed", I, J, K);
   }
+  cudaDeviceSynchronize();  // as in upload
   for (int c = 0; c < 3; ++c)
     for (int f = 0; f < 4; ++f) {
       size_t n = f == 1 ? std::max<size_t>(s->nv, 1) : (f == 3 ? s->n2 : s->n3);
@@ -1428,7 +1439,7 @@ int ensure_adj(agcm_state* s) {
   auto put_ints = [&](const auto& v) {
     using E = std::decay_t<decltype(v[0])>;
     E* d = v.empty() ? nullptr : (E*)get(v.size() * sizeof(E));
-    if (d && cudaMemcpy(d, v.data(), v.size() * sizeof(E), cudaMemcpyHostToDevice) != cudaSuccess) ok = false;
+    if (d && !upload(d, v.data(), v.size() * sizeof(E))) ok = false;
     return d;
   };
   s->adj_items = put_ints(items);
@@ -2029,8 +2040,7 @@ int agcm_ensemble_create(agcm_state_t* const* members, int n, agcm_ensemble_t** 
   e->d_desc = dev_alloc(e->host_desc.size());
   e->d_items = dev_alloc(std::max<size_t>(e->host_items.size(), 1) * sizeof(int4));
   if (e->d_items && !e->host_items.empty() &&
-      cudaMemcpy(e->d_items, e->host_items.data(), e->host_items.size() * sizeof(int4), cudaMemcpyHostToDevice) !=
-          cudaSuccess) {
+      !upload(e->d_items, e->host_items.data(), e->host_items.size() * sizeof(int4))) {
     dev_free(e->d_items);
     e->d_items = nullptr;
   }
