@@ -70,8 +70,10 @@ int agcm_version(void);
  * Device memory hook.  By default the library calls cudaMalloc/cudaFree.
  * A caller may route every allocation through its own allocator (the Python
  * binding routes them through PyTorch's caching allocator).  `alloc` returns
- * NULL on failure, which the library reports as AGCM_ENOMEM.  Pass NULLs to
- * restore the default.  Not thread-safe against concurrent state creation.
+ * NULL on failure, which the library reports as AGCM_ENOMEM.  Memory of any
+ * alignment will do: a block that is not 16-byte aligned is freed again and one
+ * of 255 bytes more is asked for instead.  Pass NULLs to restore the default.
+ * Not thread-safe against concurrent state creation.
  */
 typedef void* (*agcm_alloc_fn)(uint64_t bytes, void* ctx);
 typedef void (*agcm_free_fn)(void* ptr, void* ctx);

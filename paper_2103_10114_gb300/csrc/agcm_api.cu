@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "../../include/agcm.h"
+#include "agcm_host.h"
 #include "agcm_common.cuh"
 #include "agcm_phases.cuh"
 #include "agcm_fused.cuh"
@@ -71,9 +72,13 @@ agcm_alloc_fn g_alloc = nullptr;
 agcm_free_fn g_free = nullptr;
 void* g_alloc_ctx = nullptr;
 
+agcm::AlignedBlocks& g_blocks = *new agcm::AlignedBlocks;  // never destroyed: states may outlive static destructors
+
 void* dev_alloc(size_t bytes) {
   if (bytes == 0) bytes = 256;
-  if (g_alloc) return g_alloc((uint64_t)bytes, g_alloc_ctx);
+  if (g_alloc)
+    return g_blocks.take(
+        bytes, [](size_t n) { return g_alloc((uint64_t)n, g_alloc_ctx); }, [](void* p) { g_free(p, g_alloc_ctx); });
   void* p = nullptr;
   if (cudaMalloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -83,6 +88,7 @@ void* dev_alloc(size_t bytes) {
 }
 void dev_free(void* p) {
   if (!p) return;
+  p = g_blocks.release(p);
   if (g_free)
     g_free(p, g_alloc_ctx);
   else
