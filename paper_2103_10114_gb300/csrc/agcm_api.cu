@@ -105,6 +105,18 @@ bool upload(void* d, const void* h, size_t bytes) {
          cudaStreamSynchronize(nullptr) == cudaSuccess;
 }
 
+// Lets `kern` be launched with that much dynamic shared memory on the current device.
+agcm::SharedLimits& g_shared = *new agcm::SharedLimits;
+template <class Kern>
+cudaError_t allow_shared(Kern kern, size_t bytes) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return g_shared.raise(dev, (const void*)kern, bytes, [&](size_t n) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n);
+  });
+}
+
 // ---------------------------------------------------------------- constants
 // Reading R2: only the Earth radius is fixed by the paper (zonal grid-size table).
 constexpr double kA = 6.371e6;
@@ -767,11 +779,7 @@ int launch_fused(const agcm::Geom<T>& G, const void* const xs[4], const double* 
                           (const T*)xb[0], (const T*)xb[1], (const T*)xb[2], (const T*)xb[3], (T*)out[0],
                           (T*)out[1], (T*)out[2], (T*)out[3], ubo, vbo, ubb, vbb, (T)cdt, vec ? 1 : 0, gap(xs[2], xs[0]), gap(xs[1], xs[0]), MODE == 2 ? gap(xb[1], xb[0]) : 0, 0};
       auto kern = agcm::k_row_stage<T, MODE, TERMS, decltype(nl)::value>;
-      static std::atomic<size_t> attr{0};  // per instantiation: the size set so far
-      if (attr.load() < smem) {
-        CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        attr.store(smem);
-      }
+      CUDA_TRY(allow_shared(kern, smem));
       auto go = [&](int off, int n, cudaStream_t q, bool dependent) -> int {
         agcm::RowArgs<T> rc = ra;
         rc.first = off;
@@ -1273,7 +1281,7 @@ int agcm_filter(agcm_state_t* s, double r, void* stream) {
     const int wpb = (int)std::max<size_t>(1, std::min<size_t>(8, (96 * 1024) / row_bytes));
     const size_t smem = (size_t)wpb * row_bytes;
     auto kern = agcm::k_filter<T, VW>;
-    CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CUDA_TRY(allow_shared(kern, smem));
     int dev = 0, nsm = 0, occ = 0;
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -1526,11 +1534,7 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
   // up to some 200 levels.  The other form at 128 x 64 x 120: FP32 71 us against
   // 42, FP64 368 against 313; at 256 x 128 x 100 94 against 107, 1091 against 792.
   if (csmem <= 227 * 1024) {
-    static std::atomic<size_t> attr{0};  // the size set so far
-    if (attr.load() < csmem) {
-      CUDA_TRY(cudaFuncSetAttribute(agcm::k_adj_col<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csmem));
-      attr.store(csmem);
-    }
+    CUDA_TRY(allow_shared(agcm::k_adj_col<T>, csmem));
     bool vec = G.I % 4 == 0;
     for (int f = 0; f < 3; ++f) vec = vec && ((uintptr_t)x[f] & 15) == 0 && ((uintptr_t)y[f] & 15) == 0;
     const agcm::AdjColArgs<T> ca{(const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)x[3], (const T*)y[0],
@@ -1571,11 +1575,7 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
   }
   if (s->n_adj_items > 0) {
     const size_t smem = agcm::adj_row_smem<T>(G.K);
-    static std::atomic<size_t> attr{0};  // the size set so far
-    if (attr.load() < smem) {
-      CUDA_TRY(cudaFuncSetAttribute(agcm::k_adj_rows<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      attr.store(smem);
-    }
+    CUDA_TRY(allow_shared(agcm::k_adj_rows<T>, smem));
     const T* const r[3] = {sum ? o.rU : (accumulate ? o.oU : nullptr), sum ? o.rV : (accumulate ? o.oV : nullptr),
                            sum ? o.rPhi : (accumulate ? o.oPhi : nullptr)};
     bool vec = G.I % 4 == 0;
@@ -1972,7 +1972,7 @@ int ensemble_step(agcm_ensemble* e, int nsteps, const double* dt, cudaStream_t s
   if (e->warps_per_block == 8) {  // the row-segment persistent launch
     auto kr = agcm::k_ensemble_rows<T>;
     if (e->rows_smem > 227 * 1024) return fail(AGCM_EINVAL, "ensemble member with too many levels for the row launch");
-    CUDA_TRY(cudaFuncSetAttribute(kr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->rows_smem));
+    CUDA_TRY(allow_shared(kr, e->rows_smem));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kr, agcm::kRowB, e->rows_smem));
     if (occ < 1) return fail(AGCM_EINVAL, "row-segment ensemble kernel does not fit");
     const int per_sm = e->blocks_per_sm > 0 ? std::min(e->blocks_per_sm, occ) : occ;

@@ -2,8 +2,10 @@
 #pragma once
 #include <cstddef>
 #include <cstdint>
+#include <map>
 #include <mutex>
 #include <unordered_map>
+#include <utility>
 
 namespace agcm {
 
@@ -40,6 +42,27 @@ class AlignedBlocks {
  private:
   std::mutex mu_;
   std::unordered_map<void*, void*> hook_;
+};
+
+// The dynamic shared memory each kernel may be launched with, which is set per
+// device and must hold for every thread that is about to launch: it is only
+// ever raised, by one thread at a time.
+class SharedLimits {
+ public:
+  // set(bytes) makes the limit `bytes` on device dev and returns 0 if it could.
+  template <class Set>
+  auto raise(int dev, const void* kernel, size_t bytes, Set set) -> decltype(set(bytes)) {
+    std::lock_guard<std::mutex> lk(mu_);
+    size_t& now = size_[{dev, kernel}];
+    if (now >= bytes) return {};
+    const auto rc = set(bytes);
+    if (rc == decltype(set(bytes)){}) now = bytes;
+    return rc;
+  }
+
+ private:
+  std::mutex mu_;
+  std::map<std::pair<int, const void*>, size_t> size_;
 };
 
 }  // namespace agcm
