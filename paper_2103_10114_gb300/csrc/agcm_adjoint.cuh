@@ -599,13 +599,14 @@ __device__ __forceinline__ P* opaque(P* p) {
 }
 
 // The gathered adjoint of one column (j, i) at the levels of one chunk of
-// kAdjLevChunk levels (blockIdx.z): the U point (j, i), the Phi point (j, i)
+// lev levels (blockIdx.z): the U point (j, i), the Phi point (j, i)
 // and, for j < J-1, the V point (j, i).  Each neighbour value is read through
 // L1.  This is the general form for any stride; k_adj_rows below takes the
 // rows whose strides are small, and this kernel the nrows rows in `rows`.
 // The level sums of the 2-D factors' adjoints are written per chunk to
-// part[3][nchunks][nrows][I] and added in chunk order by k_adj_fold.
-constexpr int kAdjLevChunk = 1;  // few rows: the more chunks the shorter the launch (256x128x30: 282 against 297 us a reverse step with 4)
+// part[3][nchunks][nrows][I] and added in chunk order by k_adj_fold.  Chunks of
+// one level, as long as the grid's z holds them: for few rows, the more chunks
+// the shorter the launch (256x128x30: 282 against 297 us a reverse step with 4).
 // Offsets in row j (stride M = Mu_j):  a0 = i - (M-1)/2, b0 = i + (M+1)/2 =
 // a0 + M (the pair whose face flux is F^u(i) for a Phi point, one of the two
 // for a U point), a1 = i - (M+1)/2, b1 = i + (M-1)/2 = a1 + M (the other U
@@ -615,13 +616,13 @@ __global__ void __launch_bounds__(kAdjTileX* kAdjTileY, 4) k_adj_gather(
     Geom<T> g, const T* __restrict__ U, const T* __restrict__ V, const T* __restrict__ Phi, ColState<T> cs,
     const T* __restrict__ W, const T* __restrict__ psi, const T* __restrict__ Db, const T* __restrict__ aPhi,
     const T* __restrict__ arPcol, const T* __restrict__ yU, const T* __restrict__ yV, const T* __restrict__ yPhi,
-    const int* __restrict__ rows, int nrows, T* __restrict__ part, AdjOut<T> o) {
+    const int* __restrict__ rows, int nrows, int lev, T* __restrict__ part, AdjOut<T> o) {
   const int I = g.I, J = g.J, K = g.K;
   const int i = blockIdx.x * kAdjTileX + (int)(threadIdx.x % kAdjTileX);
   const int jq = blockIdx.y * kAdjTileY + (int)(threadIdx.x / kAdjTileX);
   if (i >= I || jq >= nrows) return;
   const int j = ldg(rows + jq);
-  const int kb = blockIdx.z * kAdjLevChunk, ke = min(K, kb + kAdjLevChunk);
+  const int kb = blockIdx.z * lev, ke = min(K, kb + lev);
   const size_t plane = (size_t)J * I, vplane = (size_t)(J - 1) * I;
   const bool hasS = j < J - 1, hasN = j > 0, hasSS = j + 1 < J - 1;
   const int M = ldg(g.Mu + j);

@@ -67,6 +67,9 @@ std::mutex g_grid_mu;
 // give every SM one CTA.
 constexpr long long kRowMinCols = 4096;
 
+constexpr size_t kMaxShared = 227 * 1024;  // of a block
+constexpr int kMaxGridZ = 65535;
+
 // ---------------------------------------------------------------- allocator
 agcm_alloc_fn g_alloc = nullptr;
 agcm_free_fn g_free = nullptr;
@@ -277,6 +280,7 @@ struct agcm_state {
   int n_col_items = 0, col_threads = 32;
   int* adj_rows = nullptr;
   int n_adj_rows = 0;
+  int adj_lev = 1, adj_chunks = 1;  // their levels of a chunk, chunks
   void* adj_part = nullptr;  // level-chunk partial sums of those rows (3 * chunks * rows * I)
   void* mu[2][4] = {};  // stage adjoints mu2, mu1
 };
@@ -769,7 +773,7 @@ int launch_fused(const agcm::Geom<T>& G, const void* const xs[4], const double* 
   // a state's own choice (agcm_state_set_stage_kernel), else the process's
   const int choice = state_choice > 0 ? state_choice : g_stage_choice.load(std::memory_order_relaxed);
   const size_t smem = agcm::row_smem_bytes<T>(G.K);
-  const bool rowpath = choice != 1 && G.nitems > 0 && (choice == 2 || ((long long)G.I * G.J >= kRowMinCols && !G.column)) && smem <= 227 * 1024;
+  const bool rowpath = choice != 1 && G.nitems > 0 && (choice == 2 || ((long long)G.I * G.J >= kRowMinCols && !G.column)) && smem <= kMaxShared;
   auto rows = [&](auto nl) -> int {
     if (rowpath) {
       // 16-byte aligned rows are staged by 16-byte copies, others element by element
@@ -1428,8 +1432,10 @@ int ensure_adj(agcm_state* s) {
   s->psi = get(n3);
   for (auto& p : s->adj3) p = get(n3);
   for (auto& p : s->adj2) p = get(n2);
-  // rows whose adjoint halo fits a row segment go to k_adj_rows
+  // rows whose adjoint halo fits a row segment go to k_adj_rows, while a block
+  // holds its table of the levels (up to some 39,000 in FP32, 17,000 in FP64)
   const agcm_grid* g = s->grid;
+  const bool staged = (s->prec == AGCM_FP64 ? agcm::adj_row_smem<double>(g->K) : agcm::adj_row_smem<float>(g->K)) <= kMaxShared;
   std::vector<int4> items, ones;
   std::vector<int> rows;
   for (int j = 0; j < g->J; ++j) {
@@ -1437,7 +1443,7 @@ int ensure_adj(agcm_state* s) {
     const int H = agcm::adj_row_halo(M, Mv, Mvm);
     int n = 0, S = 0;
     agcm::row_segments(g->I, H, agcm::kRowB, &n, &S);
-    if (n == 0) {
+    if (n == 0 || !staged) {
       rows.push_back(j);
       continue;
     }
@@ -1476,8 +1482,9 @@ int ensure_adj(agcm_state* s) {
   s->adj_rows = put_ints(rows);
   s->n_adj_rows = (int)rows.size();
   if (!rows.empty()) {
-    const size_t nch = (size_t)(g->K + agcm::kAdjLevChunk - 1) / agcm::kAdjLevChunk;
-    s->adj_part = get(3 * nch * rows.size() * g->I * e);
+    s->adj_lev = (g->K + kMaxGridZ - 1) / kMaxGridZ;
+    s->adj_chunks = (g->K + s->adj_lev - 1) / s->adj_lev;
+    s->adj_part = get(3 * (size_t)s->adj_chunks * rows.size() * g->I * e);
   }
   for (int c = 0; c < 2; ++c) {
     s->mu[c][0] = get(n3);
@@ -1533,7 +1540,7 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
   const size_t csmem = agcm::adj_col_smem<T>(G.K);
   // up to some 200 levels.  The other form at 128 x 64 x 120: FP32 71 us against
   // 42, FP64 368 against 313; at 256 x 128 x 100 94 against 107, 1091 against 792.
-  if (csmem <= 227 * 1024) {
+  if (csmem <= kMaxShared) {
     CUDA_TRY(allow_shared(agcm::k_adj_col<T>, csmem));
     bool vec = G.I % 4 == 0;
     for (int f = 0; f < 3; ++f) vec = vec && ((uintptr_t)x[f] & 15) == 0 && ((uintptr_t)y[f] & 15) == 0;
@@ -1563,15 +1570,14 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
   }
   if (s->n_adj_rows > 0) {
     cudaStream_t q = fork ? s->aux[0] : st;
-    const int nch = (G.K + agcm::kAdjLevChunk - 1) / agcm::kAdjLevChunk;
     const dim3 agrid((unsigned)((G.I + agcm::kAdjTileX - 1) / agcm::kAdjTileX),
-                     (unsigned)((s->n_adj_rows + agcm::kAdjTileY - 1) / agcm::kAdjTileY), (unsigned)nch);
+                     (unsigned)((s->n_adj_rows + agcm::kAdjTileY - 1) / agcm::kAdjTileY), (unsigned)s->adj_chunks);
     agcm::k_adj_gather<T><<<agrid, agcm::kAdjTileX * agcm::kAdjTileY, 0, q>>>(
         G, (const T*)x[0], (const T*)x[1], (const T*)x[2], cs, (const T*)s->W, (const T*)s->psi,
         (const T*)s->adj3[0], (const T*)s->adj3[1], (const T*)s->adj2[0], (const T*)y[0], (const T*)y[1],
-        (const T*)y[2], s->adj_rows, s->n_adj_rows, (T*)s->adj_part, o);
+        (const T*)y[2], s->adj_rows, s->n_adj_rows, s->adj_lev, (T*)s->adj_part, o);
     agcm::k_adj_fold<T><<<nblocks((size_t)s->n_adj_rows * G.I, 256), 256, 0, q>>>(
-        G, s->adj_rows, s->n_adj_rows, nch, (const T*)s->adj_part, m);
+        G, s->adj_rows, s->n_adj_rows, s->adj_chunks, (const T*)s->adj_part, m);
   }
   if (s->n_adj_items > 0) {
     const size_t smem = agcm::adj_row_smem<T>(G.K);
@@ -1971,7 +1977,7 @@ int ensemble_step(agcm_ensemble* e, int nsteps, const double* dt, cudaStream_t s
   const int threads = 32 * e->warps_per_block;
   if (e->warps_per_block == 8) {  // the row-segment persistent launch
     auto kr = agcm::k_ensemble_rows<T>;
-    if (e->rows_smem > 227 * 1024) return fail(AGCM_EINVAL, "ensemble member with too many levels for the row launch");
+    if (e->rows_smem > kMaxShared) return fail(AGCM_EINVAL, "ensemble member with too many levels for the row launch");
     CUDA_TRY(allow_shared(kr, e->rows_smem));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kr, agcm::kRowB, e->rows_smem));
     if (occ < 1) return fail(AGCM_EINVAL, "row-segment ensemble kernel does not fit");
