@@ -26,7 +26,15 @@ static int own_columns_once() {
     }
   return 0;
 }
-int main() { return own_columns_once(); }
+// A block holds the rows of as many levels as the row-segment ensemble has ever
+// taken: 4449 in FP32, 1732 in FP64.
+static int levels_of_a_block() {
+  const size_t most = 227 * 1024;
+  if (row_smem_bytes<float>(4449) > most) return puts("FP32 levels"), 1;
+  if (row_smem_bytes<double>(1732) > most) return puts("FP64 levels"), 1;
+  return 0;
+}
+int main() { return own_columns_once() | levels_of_a_block(); }
 """
 
 
