@@ -552,19 +552,13 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
     L[agcm::kLevRho] = rho[k];
   }
   for (int j = 0; j < J; ++j) {
-    double* L = rowtab.data() + (size_t)j * agcm::kRowTabN;
-    L[agcm::kRtZf] = zf[j];
-    L[agcm::kRtR2A] = r2A[j];
-    L[agcm::kRtAf] = g->A[j] * f0[j];
-    L[agcm::kRtAc] = g->A[j] * cota[j];
-    if (j < JV) {
-      L[agcm::kRtYv] = yv[j];
-      L[agcm::kRtR2Av] = r2Av[j];
-      L[agcm::kRtRvn] = g->Av[j] / g->A[j];
-      L[agcm::kRtRvs] = g->Av[j] / g->A[j + 1];
-    }
-    rAz[2 * j] = (double)(T)zf[j] / g->A[j];
-    rAz[2 * j + 1] = j > 0 ? agcm::edge_units((T)yv[j - 1], (T)zf[j - 1], (T)zf[j]) : 0.0;
+    const agcm::RowTab t = agcm::row_tab(j, J, kA * g->dlam, kA * g->dth, g->A.data(), g->sv.data(), g->Av.data(),
+                                         g->Mu.data(), [&](int r) { return 2.0 * kOmega * g->c[r]; },
+                                         [&](int r) { return g->cot[r] / kA; });
+    std::copy(t.v, t.v + agcm::kRowTabN, rowtab.begin() + (size_t)j * agcm::kRowTabN);
+    const double z = kA * g->dth / g->Mu[j];
+    rAz[2 * j] = z / g->A[j];
+    rAz[2 * j + 1] = j > 0 ? agcm::edge_units<T>(kA * g->dlam * g->sv[j - 1], kA * g->dth / g->Mu[j - 1], z) : 0.0;
   }
   std::vector<double> rt0pit((size_t)J * I);
   for (size_t n = 0; n < rt0pit.size(); ++n) rt0pit[n] = g->rts[n] / g->pit[n];
@@ -1715,19 +1709,12 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
         rowT[10 * rowStride + j] = (T)(0.25 * A[j] / Av[j]);
         rowT[11 * rowStride + j] = (T)(0.25 * A[j + 1] / Av[j]);
       }
-      T* L = rowtab + (size_t)j * agcm::kRowTabN;
-      const bool v = j < J - 1;
-      L[agcm::kRtZf] = rowT[2 * rowStride + j];
-      L[agcm::kRtR2A] = rowT[3 * rowStride + j];
-      L[agcm::kRtAf] = (T)(A[j] * (2.0 * kOmega * c[j]));
-      L[agcm::kRtAc] = (T)(A[j] * (cot[j] / kA));
-      L[agcm::kRtYv] = v ? rowT[7 * rowStride + j] : T(0);
-      L[agcm::kRtR2Av] = v ? rowT[9 * rowStride + j] : T(0);
-      L[agcm::kRtRvn] = v ? (T)(Av[j] / A[j]) : T(0);
-      L[agcm::kRtRvs] = v ? (T)(Av[j] / A[j + 1]) : T(0);
-      const T zf = (T)(kA * dth / Mu[j]);
-      rAz[2 * j] = (double)zf / A[j];
-      rAz[2 * j + 1] = j > 0 ? agcm::edge_units((T)(kA * dlam * sv[j - 1]), (T)(kA * dth / Mu[j - 1]), zf) : 0.0;
+      const agcm::RowTab t = agcm::row_tab(j, J, kA * dlam, kA * dth, A, sv, Av, Mu,
+                                           [&](int r) { return 2.0 * kOmega * c[r]; }, [&](int r) { return cot[r] / kA; });
+      for (int q = 0; q < agcm::kRowTabN; ++q) rowtab[(size_t)j * agcm::kRowTabN + q] = (T)t.v[q];
+      const double z = kA * dth / Mu[j];
+      rAz[2 * j] = z / A[j];
+      rAz[2 * j + 1] = j > 0 ? agcm::edge_units<T>(kA * dlam * sv[j - 1], kA * dth / Mu[j - 1], z) : 0.0;
     }
     if (n < (size_t)K) {
       const int k = (int)n;

@@ -45,8 +45,7 @@ struct Geom {
   const T* rho;     // beta2 / beta_k: the delta kappa Phi/P part of the coefficient (K)
   const T* oms;     // 1 - sigma_hat_k (K): W_k = SD_k - (1 - sigma_hat_k) C
   // the row-segment kernel's tables: kLevN values a level (kLev...), kRowTabN
-  // values a row (kRt...; zero where there is no V row); in FP64 zf_j / A_j and
-  // edge_units of the V edge j-1 (J x 2)
+  // values a row (kRt...); in FP64 z_j / A_j and edge_units of the V edge j-1 (J x 2)
   const T* lev;
   const T* rowtab;
   const double* rAz;
@@ -80,9 +79,38 @@ struct Geom {
 // dsigma, 1 / dsigma, sigma_hat (the level's upper half level), rho, 2 beta Hkk.
 enum { kLevDs, kLevH4, kLevh4, kLevhr2, kLevRds, kLevSh, kLevRho, kLevH2, kLevN };
 
-// Values per row of Geom::rowtab: zf, 1 / (2 A), A f0, A cot(theta) / a; yv, 1 /
-// (2 Av), Av_j / A_j, Av_j / A_{j+1}.
-enum { kRtZf, kRtR2A, kRtAf, kRtAc, kRtYv, kRtR2Av, kRtRvn, kRtRvs, kRowTabN };
+// Values per row of Geom::rowtab, lengths in units of the row's z = a dth / Mu_j,
+// each formed in FP64 and rounded once: z / (2 A_j), z / (2 Av_j); the V edges'
+// lengths a dlam sin(theta^v) of V rows j, j-1; A_j f0, A_j cot(theta) / a; Av_j /
+// A_j, Av_j / A_{j+1}.  Then, for a row of any strides, of its southern neighbour
+// in the same units: V row j+1's length, z of row j+1, A_{j+1} f0, A_{j+1}
+// cot(theta) / a.  Zero where there is no such row.
+enum { kRtPh, kRtV, kRtYv, kRtYn, kRtAf, kRtAc, kRtRvn, kRtRvs, kRtOwn, kRtYs = kRtOwn, kRtZs, kRtAfs, kRtAcs, kRowTabN };
+struct RowTab {
+  double v[kRowTabN];
+};
+// Row j's values; A, sv, Av and f0(j), c(j) = cot(theta_j) / a in FP64; V rows 0 .. J-2.
+template <class F0, class Cot>
+__host__ __device__ inline RowTab row_tab(int j, int J, double adlam, double adth, const double* A, const double* sv,
+                                          const double* Av, const int* Mu, F0 f0, Cot c) {
+  RowTab t{};
+  const double z = adth / Mu[j];
+  t.v[kRtPh] = 0.5 * z / A[j];
+  t.v[kRtAf] = A[j] * f0(j) / z;
+  t.v[kRtAc] = A[j] * c(j) / z;
+  if (j > 0) t.v[kRtYn] = adlam * sv[j - 1] / z;
+  if (j < J - 1) {
+    t.v[kRtV] = 0.5 * z / Av[j];
+    t.v[kRtYv] = adlam * sv[j] / z;
+    t.v[kRtRvn] = Av[j] / A[j];
+    t.v[kRtRvs] = Av[j] / A[j + 1];
+    t.v[kRtZs] = (double)Mu[j] / Mu[j + 1];
+    t.v[kRtAfs] = A[j + 1] * f0(j + 1) / z;
+    t.v[kRtAcs] = A[j + 1] * c(j + 1) / z;
+  }
+  if (j < J - 2) t.v[kRtYs] = adlam * sv[j + 1] / z;
+  return t;
+}
 
 __device__ __forceinline__ int wrapi(int i, int I) {
   return i < 0 ? i + I : (i >= I ? i - I : i);
@@ -97,16 +125,15 @@ __device__ __forceinline__ T ldg(const T* p) {
 __device__ __forceinline__ double sqrt_t(double x) { return sqrt(x); }
 __device__ __forceinline__ float sqrt_t(float x) { return sqrtf(x); }
 
-// A row's column integrals take a V edge's length y in units of the row's z:
-// the rounded product of y and the rounded 1 / z.  What the rows of an edge
-// make of it differs where their strides do; edge_units is what the row above
-// (zn) makes of it over what the row below (z) does, less 1.  Without it the
-// mass that crossed such an edge changed by some 3e-8 of itself: 1.4e-10 of the
-// total in 500 steps of 1440x720x30 FP32, 4e-12 with it.
+// A row's column integrals take a V edge's length y in units of the row's z,
+// rounded to T.  What the rows of an edge make of it differs where their strides
+// do; edge_units is what the row above (zn) makes of it over what the row below
+// (z) does, less 1.  Without it the mass that crossed such an edge changed by
+// some 3e-8 of itself: 1.4e-10 of the total in 500 steps of 1440x720x30 FP32,
+// 4e-12 with it.
 template <class T>
-__host__ __device__ inline double edge_units(T y, T zn, T z) {
-  const T wn = y * (T(1) / zn), w = y * (T(1) / z);
-  return ((double)zn * (double)wn) / ((double)z * (double)w) - 1.0;
+__host__ __device__ inline double edge_units(double y, double zn, double z) {
+  return (zn * (double)(T)(y / zn)) / (z * (double)(T)(y / z)) - 1.0;
 }
 
 // a + b = s + e exactly (TwoSum, Knuth), and a sum of FP32 numbers in three
