@@ -558,7 +558,11 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
     std::copy(t.v, t.v + agcm::kRowTabN, rowtab.begin() + (size_t)j * agcm::kRowTabN);
     const double z = kA * g->dth / g->Mu[j];
     rAz[2 * j] = z / g->A[j];
-    rAz[2 * j + 1] = j > 0 ? agcm::edge_units<T>(kA * g->dlam * g->sv[j - 1], kA * g->dth / g->Mu[j - 1], z) : 0.0;
+    auto edge = [&](int r) {  // V edge j - 1 as row r takes it
+      return agcm::edge_length<T>(agcm::row_on_columns(r, J, g->Mu.data(), g->Mv.data()), g->sv[j - 1], g->A[r], g->s[r],
+                                  kA * g->dth / g->Mu[r], kA, g->dlam, g->dth);
+    };
+    rAz[2 * j + 1] = j > 0 ? agcm::edge_units(edge(j - 1), edge(j)) : 0.0;
   }
   std::vector<double> rt0pit((size_t)J * I);
   for (size_t n = 0; n < rt0pit.size(); ++n) rt0pit[n] = g->rts[n] / g->pit[n];
@@ -1714,7 +1718,11 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
       for (int q = 0; q < agcm::kRowTabN; ++q) rowtab[(size_t)j * agcm::kRowTabN + q] = (T)t.v[q];
       const double z = kA * dth / Mu[j];
       rAz[2 * j] = z / A[j];
-      rAz[2 * j + 1] = j > 0 ? agcm::edge_units<T>(kA * dlam * sv[j - 1], kA * dth / Mu[j - 1], z) : 0.0;
+      auto edge = [&](int r) {  // V edge j - 1 as row r takes it
+        return agcm::edge_length<T>(agcm::row_on_columns(r, J, Mu, Mv), sv[j - 1], A[r], s[r], kA * dth / Mu[r], kA, dlam,
+                                    dth);
+      };
+      rAz[2 * j + 1] = j > 0 ? agcm::edge_units(edge(j - 1), edge(j)) : 0.0;
     }
     if (n < (size_t)K) {
       const int k = (int)n;

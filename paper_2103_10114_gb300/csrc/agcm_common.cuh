@@ -45,7 +45,7 @@ struct Geom {
   const T* rho;     // beta2 / beta_k: the delta kappa Phi/P part of the coefficient (K)
   const T* oms;     // 1 - sigma_hat_k (K): W_k = SD_k - (1 - sigma_hat_k) C
   // the row-segment kernel's tables: kLevN values a level (kLev...), kRowTabN
-  // values a row (kRt...); in FP64 z_j / A_j and edge_units of the V edge j-1 (J x 2)
+  // values a row (kRt...); in FP64 z_j / A_j and edge_units of V edge j-1 (J x 2)
   const T* lev;
   const T* rowtab;
   const double* rAz;
@@ -125,16 +125,20 @@ __device__ __forceinline__ T ldg(const T* p) {
 __device__ __forceinline__ double sqrt_t(double x) { return sqrt(x); }
 __device__ __forceinline__ float sqrt_t(float x) { return sqrtf(x); }
 
-// A row's column integrals take a V edge's length y in units of the row's z,
-// rounded to T.  What the rows of an edge make of it differs where their strides
-// do; edge_units is what the row above (zn) makes of it over what the row below
-// (z) does, less 1.  Without it the mass that crossed such an edge changed by
-// some 3e-8 of itself: 1.4e-10 of the total in 500 steps of 1440x720x30 FP32,
-// 4e-12 with it.
+// The length of V edge e = j or j - 1 as row j's column integrals take it: a
+// dlam sin(theta^v) in units of the row's z = a dth / Mu_j, rounded to T; on a row
+// left to the column body (cols), sin(theta^v) and 1 / (a sin(theta) dth) rounded
+// to T, times the cell's area.
 template <class T>
-__host__ __device__ inline double edge_units(double y, double zn, double z) {
-  return (zn * (double)(T)(y / zn)) / (z * (double)(T)(y / z)) - 1.0;
+__host__ __device__ inline double edge_length(bool cols, double sv, double A, double s, double z, double a, double dlam,
+                                              double dth) {
+  return cols ? A * ((double)(T)sv * (double)(T)(1.0 / (a * s * dth))) : z * (double)(T)(a * dlam * sv / z);
 }
+// What the row above makes of an edge over what the row below does, less 1.
+// Without it the mass that crosses an edge between rows of different strides
+// changes by some 3e-8 of itself: 1.4e-10 of the total in 500 steps of
+// 1440x720x30 FP32, 4e-12 with it.
+__host__ __device__ inline double edge_units(double above, double below) { return above / below - 1.0; }
 
 // a + b = s + e exactly (TwoSum, Knuth), and a sum of FP32 numbers in three
 // FP32 terms.  Products that go in are formed by __fmul_rn: a multiply-add

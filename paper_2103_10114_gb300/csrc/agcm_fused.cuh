@@ -170,6 +170,8 @@ __device__ __forceinline__ void fused_column(
     cotas = g.cota[j + 1];
   }
   const T rady = g.rady;
+  constexpr bool kEdge = POL && sizeof(T) == 4 && ADA;
+  const double eN = kEdge ? g.rAz[2 * j + 1] : 0.0;
 
   // ---- column integrals C (FP64) at the own column, i+1 and j+1
   const double Cc = ((double)PufE * Ubar[rj + fE] - (double)PufW * Ubar[rj + fW]) * (double)rdx +
@@ -183,12 +185,15 @@ __device__ __forceinline__ void fused_column(
     Cs = ((double)PugE * Ubar[rjp + gE] - (double)PugW * Ubar[rjp + gW]) * (double)rdxs +
          ((hasSS ? (double)svjp * (double)Pvs * Vbar[rjp + i] : 0.0) - (double)svj * (double)Pvc * Vbar[rj + i]) *
              (double)rdys;
-  if (POL && (w > 0 || !act)) {
-  } else if (MODE == 0)
-    pio[rj + i] = ADA ? (T)(-Cc) : T(0);
-  else {
-    const double pb = (MODE == 1) ? (double)pi[rj + i] : (double)pib[rj + i];
-    pio[rj + i] = ADA ? (T)(pb - (double)cdt * Cc) : (T)pb;
+  if (!POL || (w == nw - 1 && act)) {  // the last group: the first has the means to finish
+    // what leaves the row above enters this one (edge_units)
+    const double Cm = kEdge && hasN ? Cc - eN * ((double)svjm * (double)Pvn * Vbar[rjm + i] * (double)rdy) : Cc;
+    if (MODE == 0) {
+      pio[rj + i] = ADA ? (T)(-Cm) : T(0);
+    } else {
+      const double pb = (MODE == 1) ? (double)pi[rj + i] : (double)pib[rj + i];
+      pio[rj + i] = ADA ? (T)(pb - (double)cdt * Cm) : (T)pb;
+    }
   }
   const T Cf = (T)Cc, Cpf = (T)Cp, Csf = (T)Cs;
 

@@ -4,6 +4,7 @@ jet moves some 1e-3 of the mass between the latitudes; a face length that
 differs by an FP32 rounding (6e-8) between the two rows of an edge shows as
 some 6e-11 of the total, the rounding of pi itself (6e-8 of |pi| ~ 1e-2 over
 sqrt(points)) below 2e-11 on these grids."""
+import numpy as np
 import pytest
 
 from paper_2103_10114_gb300 import agcm, inputs
@@ -18,6 +19,25 @@ def test_mass_is_kept_across_stride_changes(cuda_ok, grid):
     st = inputs.baroclinic_jet(I, J, K, seed=3, noise=1e-3, terrain_seed=2)
     g = agcm.Grid(I, J, K, phis=st["phis"])
     s = agcm.State(g, agcm.AGCM_FP32)
+    s.load(st)
+    before = s.diagnostics()["mass"]
+    s.step(300, g.dt(100.0))
+    assert abs(s.diagnostics()["mass"] / before - 1.0) <= 4e-11
+    s.close()
+
+
+def test_mass_is_kept_across_the_edges_of_the_column_body(cuda_ok):
+    """The same where every third row has a stride above 31 and is left to the
+    column body, which takes its edges' lengths from other tables: two of three
+    edges lie between the two bodies."""
+    agcm.build()
+    I, J, K = 360, 180, 6
+    mu, mv = (np.array(v) for v in agcm.Grid(I, J, K).leap())
+    mu[1::3] = np.maximum(mu[1::3], 45)
+    st = inputs.baroclinic_jet(I, J, K, seed=3, noise=1e-3, terrain_seed=2)
+    g = agcm.Grid(I, J, K, leap_u=mu, leap_v=mv, phis=st["phis"])
+    s = agcm.State(g, agcm.AGCM_FP32)
+    s.set_stage_kernel(agcm.STAGE_ROW)
     s.load(st)
     before = s.diagnostics()["mass"]
     s.step(300, g.dt(100.0))
