@@ -377,16 +377,22 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
     }
   }
   for (const int4& v : half) (v.x >> 24 == agcm::kRowPair ? pairs : single[0]).push_back(v);
-  // The rows next to the poles: in a grid of two waves of CTAs and more their
-  // work counts, else the latency of these few blocks does (33 against 22 us a
-  // stage at 256x128x30, 48 against 33 at 360x180x30; 294 against 314 at
-  // 1440x720x30 the other way).
+  // The rows left to the column body, next to the poles or wherever strides are
+  // wide.  A few of them are latency: 32 columns a block, the levels shared out
+  // over four groups (33 against 22 us a stage at 256x128x30 FP32, 48 against 33
+  // at 360x180x30 with 128 columns a block).  Beside two waves of CTAs and more,
+  // or where they are many themselves, they are work, of which the groups make
+  // more: 128 columns (294 against 314 us at 1440x720x30; with 73 wide rows at
+  // 720x360x30 129 against 180, with 21 at 405x203x20 41 against 48; 11 rows
+  // there, 143 items, 41.5 against 40.3, 45 rows at 256x128x30 51 against 39).
   // Half as many columns, twice the groups of levels, where that fits beside
   // the rows in one wave (256x128x30: 23.4 -> 21.3 us a stage, 16 levels 18.3 ->
   // 17.6, 12 levels 17.2 -> 17.9; 405x203x26, which it would take to a second
   // wave, 35 -> 45).
-  const bool fits = g->K >= 16 && nseg + polar_rows.size() * (size_t)((g->I + 15) / 16) <= plan.slots;
-  const int cols = nseg >= (size_t)6 * plan.nsm ? agcm::kRowB : (fits ? 16 : 32);
+  auto blocks = [&](int c) { return polar_rows.size() * (size_t)((g->I + c - 1) / c); };
+  const bool fits = g->K >= 16 && nseg + blocks(16) <= plan.slots;
+  const bool few = plan.slots == 0 || 2 * blocks(32) <= plan.slots || 2 * (nseg + blocks(32)) <= 3 * plan.slots;
+  const int cols = nseg >= (size_t)6 * plan.nsm || !few ? agcm::kRowB : (fits ? 16 : 32);
   for (int j : polar_rows)
     for (int q = 0; q < g->I; q += cols) polar.push_back(make_int4(agcm::kRowPolar << 24 | j, q, cols, 0));
   items->clear();
@@ -420,8 +426,18 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
 // -> 36 us a stage; 750x375x20: 81 -> 78; 1000x500x20: 115 -> 111); with the
 // same few waves the equal segments' lighter CTAs are as good (640x320x30: 78.4
 // against 79.4 us, 500x250x30: 53.0 against 53.8).
+//
+// The column kernel where two rows in five or more are left to its body, which
+// runs with more warps an SM there than in the row kernel: with half of the rows
+// wide 183 against 191 us a stage at 720x360x30 FP32, 48.5 against 63 at
+// 405x203x20, 46 against 53 at 256x128x30, 189 against 214 at 256x128x16 FP64
+// (512x256x12 FP64 561 against 485); with a third 185 against 163, 49 against 44,
+// 46 against 39, 190 against 210; with all 188 against 295.
 inline RowPlan row_plan(const agcm_grid* g, int per_sm, bool fp64) {
   RowPlan p;
+  int wide = 0;
+  for (int j = 0; j < g->J; ++j) wide += agcm::row_on_columns(j, g->J, g->Mu.data(), g->Mv.data());
+  p.column = 5LL * wide >= 2LL * g->J;
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       nsm < 1) {
@@ -463,7 +479,7 @@ inline RowPlan row_plan(const agcm_grid* g, int per_sm, bool fp64) {
   // where the column kernel's warps are one to a scheduler and the row
   // segments' two, the column kernel's is the shorter (180x90x30: 207 against
   // 221 us a stage)
-  p.column = fp64 && best >= 2 && (long long)((g->I + 31) / 32) * g->J <= 4LL * nsm;
+  p.column = p.column || (fp64 && best >= 2 && (long long)((g->I + 31) / 32) * g->J <= 4LL * nsm);
   return p;
 }
 
