@@ -605,8 +605,11 @@ __device__ __forceinline__ P* opaque(P* p) {
 // rows whose strides are small, and this kernel the nrows rows in `rows`.
 // The level sums of the 2-D factors' adjoints are written per chunk to
 // part[3][nchunks][nrows][I] and added in chunk order by k_adj_fold.  Chunks of
-// one level, as long as the grid's z holds them: for few rows, the more chunks
-// the shorter the launch (256x128x30: 282 against 297 us a reverse step with 4).
+// one level where the blocks are few: the more the shorter the launch
+// (256x128x30: 282 against 297 us a reverse step with 4); up to four levels
+// where that leaves four blocks an SM, since the fold reads a value a chunk and
+// a block's set-up is that of many levels (strides of 75 in every row, FP32: the
+// gather of a reverse step at 720x360x30 2696 -> 2282 us, 256x128x30 327 -> 265).
 // Offsets in row j (stride M = Mu_j):  a0 = i - (M-1)/2, b0 = i + (M+1)/2 =
 // a0 + M (the pair whose face flux is F^u(i) for a Phi point, one of the two
 // for a U point), a1 = i - (M+1)/2, b1 = i + (M-1)/2 = a1 + M (the other U
@@ -889,7 +892,7 @@ enum AdjRowArr {
   kAdjPub
 };
 constexpr int kAdjRaw = 28;
-template <class T>
+template <class T, int B>
 struct AdjRing {
   static constexpr int R = sizeof(T) == 4 ? 4 : 2;
 };
@@ -902,9 +905,9 @@ __host__ __device__ inline int adj_row_halo(int M, int Mv, int Mvm) {
   if (hm > h) h = hm;
   return (h + 3) & ~3;
 }
-template <class T>
+template <class T, int B = kRowB>
 constexpr size_t adj_row_smem(int K) {
-  return sizeof(T) * ((size_t)kRowB * (AdjRing<T>::R * kAdjRaw + 2 * kAdjPub) + K + 64);
+  return sizeof(T) * ((size_t)B * (AdjRing<T, B>::R * kAdjRaw + 2 * kAdjPub) + K + 64);
 }
 
 template <class T>
@@ -917,10 +920,10 @@ struct AdjRowArgs {
   int vec;                   // 1: every row is 16-byte aligned
 };
 
-template <class T, bool M1>
+template <class T, bool M1, int NTP = kRowB>
 __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs, const AdjRowArgs<T>& a,
                                         const AdjM<T>& m, const AdjOut<T>& o, const int4 item, unsigned char* smem) {
-  constexpr int R = AdjRing<T>::R, NTP = kRowB;
+  constexpr int R = AdjRing<T, NTP>::R;
   const int I = g.I, J = g.J, K = g.K;
   const int j = item.x & 0xffffff, c0 = item.y, own = item.z, H = item.w;
   const bool hasS = M1 || j < J - 1, hasN = M1 || j > 0;
@@ -1270,6 +1273,23 @@ __global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_R
     adj_row<T, true>(g, cs, a, m, o, item, smem);
   else
     adj_row<T, false>(g, cs, a, m, o, item, smem);
+}
+
+// The same in CTAs of 192 threads, two an SM (12 warps, as above): FP32 rows of
+// halo 33 to 48, of which a CTA of kRowB threads would own under half, where
+// they make one and a half CTAs an SM.  Reverse step's gather with strides of 35
+// (45) in every row, 720x360x30: 1008 (1165) us, 2685 in k_adj_gather; in a
+// tenth of the rows 659 (681) against 787; with fewer the one wave's latency
+// counts (256x128x30, a third of the rows: 230 against 198).  256 threads and
+// 128 registers: 1166 (1263), 84 B of spills.
+constexpr int kAdjWide = 192;
+template <class T>
+__global__ void __launch_bounds__(kAdjWide, 2)
+    k_adj_rows_wide(const __grid_constant__ Geom<T> g, const __grid_constant__ ColState<T> cs,
+                    const __grid_constant__ AdjRowArgs<T> a, const __grid_constant__ AdjM<T> m,
+                    const __grid_constant__ AdjOut<T> o) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  adj_row<T, false, kAdjWide>(g, cs, a, m, o, a.items[blockIdx.x], smem);
 }
 
 // pi-bar = direct psi part + m-bar, with m^u_i = (m_i + m_{i+1})/2 and

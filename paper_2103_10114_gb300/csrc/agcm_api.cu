@@ -276,6 +276,8 @@ struct agcm_state {
   // adj_threads; and the rows left to k_adj_gather
   int4* adj_items = nullptr;
   int n_adj_items = 0, n_adj_any = 0, adj_threads = 32;
+  int4* adj_wide = nullptr;  // row-segment items of k_adj_rows_wide
+  int n_adj_wide = 0;
   int4* col_items = nullptr;  // row-segment items of k_adj_col, CTAs of col_threads
   int n_col_items = 0, col_threads = 32;
   int* adj_rows = nullptr;
@@ -415,6 +417,15 @@ inline int row_lists(const agcm_grid* g, const RowPlan& plan, std::vector<int4>*
   return threads;
 }
 
+inline int sm_count() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+      n > 0)
+    return n;
+  cudaGetLastError();
+  return 152;
+}
+
 // Pairs, as long as they make two CTAs an SM (720x360x30 FP32: 87 us a stage
 // against 114 with single rows, 512x256x26: 50 against 64, 405x203x26: 49
 // against 52); with fewer, single rows (256x128x30: 23.5 against 28.4 us; FP64
@@ -438,12 +449,7 @@ inline RowPlan row_plan(const agcm_grid* g, int per_sm, bool fp64) {
   int wide = 0;
   for (int j = 0; j < g->J; ++j) wide += agcm::row_on_columns(j, g->J, g->Mu.data(), g->Mv.data());
   p.column = 5LL * wide >= 2LL * g->J;
-  int dev = 0, nsm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      nsm < 1) {
-    cudaGetLastError();
-    nsm = p.nsm;
-  }
+  const int nsm = sm_count();
   p.nsm = nsm;
   const size_t slots = (size_t)per_sm * nsm;
   std::vector<int4> items;
@@ -1450,8 +1456,9 @@ int ensure_adj(agcm_state* s) {
   // holds its table of the levels (up to some 39,000 in FP32, 17,000 in FP64)
   const agcm_grid* g = s->grid;
   const bool staged = (s->prec == AGCM_FP64 ? agcm::adj_row_smem<double>(g->K) : agcm::adj_row_smem<float>(g->K)) <= kMaxShared;
-  std::vector<int4> items, ones;
-  std::vector<int> rows;
+  std::vector<int4> items, ones, wide;
+  std::vector<int> rows, rest;  // rest: without the rows of `wide`
+  const bool widths = s->prec == AGCM_FP32 && agcm::adj_row_smem<float, agcm::kAdjWide>(g->K) <= kMaxShared;
   for (int j = 0; j < g->J; ++j) {
     const int M = g->Mu[j], Mv = j < g->J - 1 ? g->Mv[j] : 0, Mvm = j > 0 ? g->Mv[j - 1] : 0;
     const int H = agcm::adj_row_halo(M, Mv, Mvm);
@@ -1459,6 +1466,11 @@ int ensure_adj(agcm_state* s) {
     agcm::row_segments(g->I, H, agcm::kRowB, &n, &S);
     if (n == 0 || !staged) {
       rows.push_back(j);
+      agcm::row_segments(g->I, H, agcm::kAdjWide, &n, &S, agcm::kAdjWide);
+      if (n == 0 || !widths)
+        rest.push_back(j);
+      else
+        for (int q = 0; q < g->I; q += S) wide.push_back(make_int4(j, q, std::min(S, g->I - q), H));
       continue;
     }
     const bool one = M == 1 && Mv == 1 && Mvm == 1;
@@ -1468,6 +1480,11 @@ int ensure_adj(agcm_state* s) {
       s->adj_threads = std::max(s->adj_threads, (own + 2 * H + 31) & ~31);
     }
   }
+  const int nsm = sm_count();
+  if (2 * wide.size() < 3 * (size_t)nsm)
+    wide.clear();
+  else
+    rows.swap(rest);
   s->n_adj_any = (int)items.size();
   items.insert(items.end(), ones.begin(), ones.end());
   auto put_ints = [&](const auto& v) {
@@ -1478,6 +1495,8 @@ int ensure_adj(agcm_state* s) {
   };
   s->adj_items = put_ints(items);
   s->n_adj_items = (int)items.size();
+  s->adj_wide = put_ints(wide);
+  s->n_adj_wide = (int)wide.size();
   std::vector<int4> citems;  // the rows that read their pair from global memory first
   for (int wide = 1; wide >= 0; --wide)
     for (int j = 0; j < g->J; ++j) {
@@ -1496,7 +1515,11 @@ int ensure_adj(agcm_state* s) {
   s->adj_rows = put_ints(rows);
   s->n_adj_rows = (int)rows.size();
   if (!rows.empty()) {
-    s->adj_lev = (g->K + kMaxGridZ - 1) / kMaxGridZ;
+    // chunks of one level to four, four blocks an SM at least (k_adj_gather's comment)
+    const size_t blocks = (size_t)((g->I + agcm::kAdjTileX - 1) / agcm::kAdjTileX) *
+                          ((rows.size() + agcm::kAdjTileY - 1) / agcm::kAdjTileY) * g->K;
+    const size_t lev = std::min<size_t>(4, std::max<size_t>(1, blocks / (4 * (size_t)nsm)));
+    s->adj_lev = (int)std::max<size_t>(lev, (size_t)(g->K + kMaxGridZ - 1) / kMaxGridZ);
     s->adj_chunks = (g->K + s->adj_lev - 1) / s->adj_lev;
     s->adj_part = get(3 * (size_t)s->adj_chunks * rows.size() * g->I * e);
   }
@@ -1575,15 +1598,32 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
                           sum ? (const T*)sum_in[2] : nullptr, sum ? (const T*)sum_in[3] : nullptr, (T)scale,
                           accumulate};
   s->prof.begin(KID_ADJ_GATHER, st);
-  // the rows of the L1 form run on the state's second stream beside the
-  // row-segment kernel (they write other rows)
-  const bool fork = s->n_adj_items > 0 && s->n_adj_rows > 0 && s->aux[0];
+  // the rows of the other two forms run on the state's second stream beside
+  // the row-segment kernel (they write other rows)
+  const int nother = s->n_adj_rows + s->n_adj_wide;
+  const bool fork = s->n_adj_items > 0 && nother > 0 && s->aux[0];
   if (fork) {
     CUDA_TRY(cudaEventRecord(s->ev_fork, st));
     CUDA_TRY(cudaStreamWaitEvent(s->aux[0], s->ev_fork, 0));
   }
+  cudaStream_t q = fork ? s->aux[0] : st;
+  const T* const r[3] = {sum ? o.rU : (accumulate ? o.oU : nullptr), sum ? o.rV : (accumulate ? o.oV : nullptr),
+                         sum ? o.rPhi : (accumulate ? o.oPhi : nullptr)};
+  bool vec = G.I % 4 == 0;
+  for (const void* p : {(const void*)x[0], (const void*)x[1], (const void*)x[2], (const void*)y[0], (const void*)y[1],
+                        (const void*)y[2], (const void*)r[0], (const void*)r[1], (const void*)r[2]})
+    vec = vec && ((uintptr_t)p & 15) == 0;
+  agcm::AdjRowArgs<T> ra{(const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)y[0], (const T*)y[1],
+                         (const T*)y[2], c.W, c.psi, c.Db, c.aPhi, c.arP, r[0], r[1], r[2], s->adj_wide, vec ? 1 : 0};
+  if constexpr (sizeof(T) == 4) {
+    if (s->n_adj_wide > 0) {
+      const size_t smem = agcm::adj_row_smem<T, agcm::kAdjWide>(G.K);
+      CUDA_TRY(allow_shared(agcm::k_adj_rows_wide<T>, smem));
+      CUDA_TRY(launch(agcm::k_adj_rows_wide<T>, dim3((unsigned)s->n_adj_wide), agcm::kAdjWide, smem, q, false, G, cs, ra, m,
+                      o));
+    }
+  }
   if (s->n_adj_rows > 0) {
-    cudaStream_t q = fork ? s->aux[0] : st;
     const dim3 agrid((unsigned)((G.I + agcm::kAdjTileX - 1) / agcm::kAdjTileX),
                      (unsigned)((s->n_adj_rows + agcm::kAdjTileY - 1) / agcm::kAdjTileY), (unsigned)s->adj_chunks);
     agcm::k_adj_gather<T><<<agrid, agcm::kAdjTileX * agcm::kAdjTileY, 0, q>>>(
@@ -1596,15 +1636,7 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
   if (s->n_adj_items > 0) {
     const size_t smem = agcm::adj_row_smem<T>(G.K);
     CUDA_TRY(allow_shared(agcm::k_adj_rows<T>, smem));
-    const T* const r[3] = {sum ? o.rU : (accumulate ? o.oU : nullptr), sum ? o.rV : (accumulate ? o.oV : nullptr),
-                           sum ? o.rPhi : (accumulate ? o.oPhi : nullptr)};
-    bool vec = G.I % 4 == 0;
-    for (const void* p : {(const void*)x[0], (const void*)x[1], (const void*)x[2], (const void*)y[0], (const void*)y[1],
-                          (const void*)y[2], (const void*)r[0], (const void*)r[1], (const void*)r[2]})
-      vec = vec && ((uintptr_t)p & 15) == 0;
-    const agcm::AdjRowArgs<T> ra{(const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)y[0], (const T*)y[1],
-                                 (const T*)y[2], c.W, c.psi, c.Db, c.aPhi, c.arP, r[0], r[1], r[2], s->adj_items,
-                                 vec ? 1 : 0};
+    ra.items = s->adj_items;
     CUDA_TRY(launch(agcm::k_adj_rows<T>, dim3((unsigned)s->n_adj_items), s->adj_threads, smem, st, true, G, cs, ra, m, o,
                     s->n_adj_any));
   }
