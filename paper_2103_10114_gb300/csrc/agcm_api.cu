@@ -276,6 +276,7 @@ struct agcm_state {
   // adj_threads; and the rows left to k_adj_gather
   int4* adj_items = nullptr;
   int n_adj_items = 0, n_adj_any = 0, adj_threads = 32;
+  bool adj_early = true;  // the gather is a dependent launch of the column pass
   int4* adj_wide = nullptr;  // row-segment items of k_adj_rows_wide
   int n_adj_wide = 0;
   int4* col_items = nullptr;  // row-segment items of k_adj_col, CTAs of col_threads
@@ -1512,6 +1513,14 @@ int ensure_adj(agcm_state* s) {
     }
   s->col_items = put_ints(citems);
   s->n_col_items = (int)citems.size();
+  // Blocks of the gather that start while the column pass still holds its SMs
+  // are put where there is room, several to an SM, and stay there: where one to
+  // an SM would do, they wait for the pass instead (a reverse step of 128x64x16
+  // FP64 973 -> 646 us, 131x60x13 820 -> 561, 128x64x64 FP32 355 -> 266, 128x64x16
+  // 119 -> 108).  With more of them, or where both launches fit side by side, the
+  // early start is worth more (256x128x30 FP32 247 against 264 us, 200x100x10 FP64
+  // 794 against 811, 100x48x30 FP32 141 against 147).
+  s->adj_early = s->n_adj_items > nsm || s->n_adj_items + s->n_col_items <= nsm;
   s->adj_rows = put_ints(rows);
   s->n_adj_rows = (int)rows.size();
   if (!rows.empty()) {
@@ -1637,7 +1646,7 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
     const size_t smem = agcm::adj_row_smem<T>(G.K);
     CUDA_TRY(allow_shared(agcm::k_adj_rows<T>, smem));
     ra.items = s->adj_items;
-    CUDA_TRY(launch(agcm::k_adj_rows<T>, dim3((unsigned)s->n_adj_items), s->adj_threads, smem, st, true, G, cs, ra, m, o,
+    CUDA_TRY(launch(agcm::k_adj_rows<T>, dim3((unsigned)s->n_adj_items), s->adj_threads, smem, st, s->adj_early, G, cs, ra, m, o,
                     s->n_adj_any));
   }
   if (fork) {
