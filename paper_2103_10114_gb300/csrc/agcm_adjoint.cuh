@@ -76,10 +76,11 @@ struct AdjCol {
 // The sums run in the state's precision: FP64 issues at 1/64 of the FP32 rate
 // on this GPU, and per level and column they would be the bulk of the pass.
 //   k_adj_col    a row segment per block, rows staged in shared memory, one
-//                walk down and one up the levels, each level's D and adjoint
-//                of W kept in shared memory between them;
-//   k_adj_col_w  more levels than shared memory holds: 32 columns and kColG
-//                groups of levels per block, stencil read through L1.
+//                walk down and one up the levels, each level's D (and adjoint
+//                of W) kept in shared memory between them;
+//   k_adj_col_w  so many levels that shared memory holds few such blocks or
+//                none: 32 columns and kColG groups of levels per block, stencil
+//                read through L1.
 constexpr int kColG = 2;
 
 // Level tables: ds, Hkk, hk, hk_rds, r2ds, 1 - sh, rho.
@@ -259,8 +260,8 @@ __device__ __forceinline__ void col_suffix(const ColCtx<T>& c, const AdjCol<T>& 
 // V and ybar_V (V rows j-1, j), Phi and ybar_Phi arrive level by level in a
 // ring of shared-memory slots, two 16-byte copies a thread, on the way down;
 // that walk forms D, the gathered adjoints of psi and W, the prefix sums and
-// with them the adjoint of Phi, and keeps D and the adjoint of W; the walk up
-// forms W, psi and Dbar from the suffix sums, reading Phi and ybar_Phi once
+// with them the adjoint of Phi, and keeps D and the adjoint of W (kKeep 1: that
+// in Dbar's place); the walk up forms W, psi and Dbar from the suffix sums, reading Phi and ybar_Phi once
 // more (from L2).  Rows whose divergence pair lies outside the halo (kind 1)
 // read the pair from global memory a level ahead.
 // Bound by load latency (16 warps an SM, 95 registers) in FP32 and by the FP64
@@ -272,19 +273,20 @@ __device__ __forceinline__ void col_suffix(const ColCtx<T>& c, const AdjCol<T>& 
 // chain of FP64 issue); 128 x 64 x 120 FP32 71 -> 42, FP64 368 -> 313.  Ring of two slots 107, three 90 (five blocks 82, but
 // 256 x 128 and 405 x 203 4 to 7 % slower); groups of six levels 83.  FP64
 // keeps the adjoint of W in Dbar's place instead of shared memory: 80 KB a
-// block would hold two blocks (1209).
+// block would hold two blocks (1209); so does FP32 where three blocks an SM
+// would not hold both.
 constexpr int kColRaw = 8;  // U, yU, V j-1, V j, yV j-1, yV j, Phi, yPhi
 constexpr int kColPad = 64;  // before the ring: a halo column's pair reaches at most H <= 32 to the west of it
 constexpr int kColB = 8;  // levels of a partial sum
 template <class T>
 struct ColRing {
   static constexpr int R = sizeof(T) == 4 ? 4 : 2;      // slots
-  static constexpr int kKeep = sizeof(T) == 4 ? 2 : 1;  // arrays kept over the levels
   static constexpr int kCtas = sizeof(T) == 4 ? 4 : 3;  // blocks per SM
 };
+// keep: the arrays kept over the levels in shared memory, D alone or D and the adjoint of W
 template <class T>
-constexpr size_t adj_col_smem(int K) {
-  return sizeof(T) * (kColPad + (size_t)kRowB * (ColRing<T>::R * kColRaw + ColRing<T>::kKeep * K) + (size_t)kLN * K);
+constexpr size_t adj_col_smem(int K, int keep) {
+  return sizeof(T) * (kColPad + (size_t)kRowB * (ColRing<T>::R * kColRaw + keep * K) + (size_t)kLN * K);
 }
 // Halo of row j's column pass: the divergence pair and the column to the west.
 __host__ __device__ inline int adj_col_halo(int M) { return ((M + 1) / 2 + 3) & ~3; }
@@ -295,13 +297,13 @@ struct AdjColArgs {
   const int4* items;                // kind << 24 | row j, first own column, own columns, halo
   int vec;                          // 1: every row is 16-byte aligned
 };
-template <class T>
+template <class T, int kKeep>
 __global__ void __launch_bounds__(kRowB, ColRing<T>::kCtas)
     k_adj_col(const __grid_constant__ Geom<T> g, const __grid_constant__ ColState<T> cs,
               const __grid_constant__ AdjColArgs<T> a, const __grid_constant__ AdjCol<T> o) {
   extern __shared__ __align__(128) unsigned char smem[];
   pdl_launch();
-  constexpr int R = ColRing<T>::R, NTP = kRowB, kKeep = ColRing<T>::kKeep;
+  constexpr int R = ColRing<T>::R, NTP = kRowB;
   const int I = g.I, J = g.J, K = g.K;
   const int4 item = a.items[blockIdx.x];
   const bool wide = item.x >> 24;

@@ -276,6 +276,7 @@ struct agcm_state {
   // adj_threads; and the rows left to k_adj_gather
   int4* adj_items = nullptr;
   int n_adj_items = 0, n_adj_any = 0, adj_threads = 32;
+  int adj_nsm = 152;      // SMs of the device
   bool adj_early = true;  // the gather is a dependent launch of the column pass
   int4* adj_wide = nullptr;  // row-segment items of k_adj_rows_wide
   int n_adj_wide = 0;
@@ -1481,7 +1482,7 @@ int ensure_adj(agcm_state* s) {
       s->adj_threads = std::max(s->adj_threads, (own + 2 * H + 31) & ~31);
     }
   }
-  const int nsm = sm_count();
+  const int nsm = s->adj_nsm = sm_count();
   if (2 * wide.size() < 3 * (size_t)nsm)
     wide.clear();
   else
@@ -1583,16 +1584,34 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
   const agcm::AdjCol<T> c{(T*)s->W, (T*)s->psi, (T*)s->adj3[0], (T*)s->adj3[1], (T*)s->adj2[0], (T*)s->adj2[1]};
   s->prof.begin(KID_ADJ_COL, st);
   const dim3 cgrid((unsigned)((G.I + 31) / 32), (unsigned)G.J);
-  const size_t csmem = agcm::adj_col_smem<T>(G.K);
-  // up to some 200 levels.  The other form at 128 x 64 x 120: FP32 71 us against
-  // 42, FP64 368 against 313; at 256 x 128 x 100 94 against 107, 1091 against 792.
-  if (csmem <= kMaxShared) {
-    CUDA_TRY(allow_shared(agcm::k_adj_col<T>, csmem));
+  // Both arrays kept in shared memory while three blocks an SM hold them (57
+  // levels; 256x128x45 FP32 79.5 against 83.6 us a step's three passes with one,
+  // 720x360x30 250 against 263, but 256x128x64 160 against 110, 720x360x100 1678
+  // against 945).
+  const int keep = sizeof(T) == 4 && 3 * agcm::adj_col_smem<T>(G.K, 2) <= kMaxShared ? 2 : 1;
+  const size_t csmem = agcm::adj_col_smem<T>(G.K, keep);
+  // The other form where staging leaves FP32 one block of an SM (184 levels and
+  // more; 256x128x160 395 staged against 451 us, 220 levels 730 against 603),
+  // unless the blocks are one to an SM anyway (128x64x160 171 against 291), and
+  // where a block does not hold D at all (397 levels in FP32, 199 in FP64, which
+  // is the faster staged up to there: 256x128x160 3791 against 5239).
+  if (csmem <= kMaxShared && (sizeof(T) == 8 || 2 * csmem <= kMaxShared || s->n_col_items <= s->adj_nsm)) {
     bool vec = G.I % 4 == 0;
     for (int f = 0; f < 3; ++f) vec = vec && ((uintptr_t)x[f] & 15) == 0 && ((uintptr_t)y[f] & 15) == 0;
     const agcm::AdjColArgs<T> ca{(const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)x[3], (const T*)y[0],
                                  (const T*)y[1], (const T*)y[2], (const T*)y[3], s->col_items, vec ? 1 : 0};
-    CUDA_TRY(launch(agcm::k_adj_col<T>, dim3((unsigned)s->n_col_items), s->col_threads, csmem, st, true, G, cs, ca, c));
+    auto col = [&](auto kern) -> int {
+      CUDA_TRY(allow_shared(kern, csmem));
+      CUDA_TRY(launch(kern, dim3((unsigned)s->n_col_items), s->col_threads, csmem, st, true, G, cs, ca, c));
+      return AGCM_OK;
+    };
+    int rc = AGCM_OK;
+    if constexpr (sizeof(T) == 4) {
+      rc = keep == 2 ? col(agcm::k_adj_col<T, 2>) : col(agcm::k_adj_col<T, 1>);
+    } else {
+      rc = col(agcm::k_adj_col<T, 1>);
+    }
+    if (rc) return rc;
   } else {
     agcm::k_adj_col_w<T><<<cgrid, dim3(32, agcm::kColG), 0, st>>>(
         G, (const T*)x[0], (const T*)x[1], (const T*)x[2], (const T*)x[3], cs, (const T*)y[0], (const T*)y[1],
