@@ -1751,6 +1751,11 @@ void* g_static_ptr[kStaticMaxDevices] = {};
 // per device: the grid id and precision whose tables the array holds (0: none)
 uint64_t g_static_uid[kStaticMaxDevices] = {};
 int g_static_prec[kStaticMaxDevices] = {};
+// the row-segment items that lie in the array with them
+struct StaticItems {
+  int off[3], cnt[3], cls[agcm::kRowCls + 1], nitems, rowT, column;
+};
+StaticItems g_static_items[kStaticMaxDevices] = {};
 
 // Typed device tables from the raw FP64 ones (same formulas as the state path).
 template <class T>
@@ -1833,7 +1838,7 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
 // tables: upload the grid's tables and build the typed ones (false when the
 // array already holds this grid's tables in this precision).
 template <class T>
-int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, const void* V, const void* Phi,
+int tendency_static(const agcm_grid* g, char* base, StaticItems& it, bool tables, const void* U, const void* V, const void* Phi,
                     const void* pi, void* tU, void* tV, void* tPhi, void* tpi, cudaStream_t st) {
   const int I = g->I, J = g->J, K = g->K;
   const size_t rS = kRowB / 8, lS = kLevB / 8, cS = kColB / 8;  // strides in elements of 8 bytes
@@ -1850,11 +1855,6 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   T* rowtab = (T*)(base + kOffRowT + 12 * kRowB);
   double* rAz = (double*)(base + kOffRowT + (12 + agcm::kRowTabN) * kRowB);
   agcm::Geom<T> G{};
-  const RowPlan plan = row_plan(g, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64, sizeof(T) == 8);
-  std::vector<int4> items;  // host only
-  G.rowT = row_lists(g, plan, &items, G.off, G.cnt, G.cls);
-  G.nitems = (int)items.size();
-  G.column = plan.column;
   if (tables) {
   const std::vector<double>* rows[6] = {&g->s, &g->c, &g->cot, &g->A, &g->sv, &g->Av};
   for (int q = 0; q < 6; ++q)
@@ -1869,8 +1869,13 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   if (!g->Mv.empty())
     CUDA_TRY(cudaMemcpyAsync(Mv, g->Mv.data(), g->Mv.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   {
-    if (!items.empty())
-      CUDA_TRY(cudaMemcpyAsync(base + kOffRowL, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
+    const RowPlan plan = row_plan(g, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64, sizeof(T) == 8);
+    std::vector<int4> v;
+    it.rowT = row_lists(g, plan, &v, it.off, it.cnt, it.cls);
+    it.nitems = (int)v.size();
+    it.column = plan.column;
+    if (!v.empty())
+      CUDA_TRY(cudaMemcpyAsync(base + kOffRowL, v.data(), v.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
   }
   k_static_geom<T><<<nblocks(std::max<size_t>((size_t)I * J, (size_t)K), 256), 256, 0, st>>>(
       I, J, K, raw, rawlev, pitraw, Mu, Mv, rowT, rowtab, rAz, levT, (float4*)(base + kOffDs3), colT, rS, lS, cS, g->beta2);
@@ -1901,6 +1906,12 @@ int tendency_static(const agcm_grid* g, char* base, bool tables, const void* U, 
   G.ds3 = (const float4*)(base + kOffDs3);
   G.lev = levT + 7 * lS;
   G.items = (const int4*)(base + kOffRowL);
+  std::copy(it.off, it.off + 3, G.off);
+  std::copy(it.cnt, it.cnt + 3, G.cnt);
+  std::copy(it.cls, it.cls + agcm::kRowCls + 1, G.cls);
+  G.nitems = it.nitems;
+  G.rowT = it.rowT;
+  G.column = it.column;
   double* ubar = (double*)(base + kOffBar);
   double* vbar = (double*)(base + kOffBar + kColB);
   agcm::k_vsum<T><<<dim3(nblocks((size_t)I * J, 256), 2), 256, 0, st>>>(G, (const T*)U, (const T*)V, ubar, vbar);
@@ -1945,8 +1956,8 @@ extern "C" int agcm_tendency_static(const agcm_grid_t* g, int precision, const v
   g_static_uid[dev] = 0;  // stays 0 if this call fails part-way
   cudaStream_t st = as_stream(stream);
   const int rc = precision == AGCM_FP64
-                     ? tendency_static<double>(g, (char*)base, tables, U, V, Phi, pi, tU, tV, tPhi, tpi, st)
-                     : tendency_static<float>(g, (char*)base, tables, U, V, Phi, pi, tU, tV, tPhi, tpi, st);
+                     ? tendency_static<double>(g, (char*)base, g_static_items[dev], tables, U, V, Phi, pi, tU, tV, tPhi, tpi, st)
+                     : tendency_static<float>(g, (char*)base, g_static_items[dev], tables, U, V, Phi, pi, tU, tV, tPhi, tpi, st);
   if (rc == AGCM_OK) {
     g_static_uid[dev] = g->uid;
     g_static_prec[dev] = precision;
