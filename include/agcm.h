@@ -265,7 +265,9 @@ int agcm_profile_enable(agcm_state_t* state, int enable);
  * (process-wide; results agree to rounding, both match the oracle).
  *   0 (default): the row-segment kernel (whole latitude-row segments staged in
  *     shared memory) on grids of at least 4096 columns, else the column kernel
- *     (one thread per column, stencil read through L1);
+ *     (one thread per column, stencil read through L1), which also keeps grids
+ *     of which two rows in five or more have leap strides above 31, and FP64
+ *     grids that give it one warp a scheduler and the other two;
  *   1: always the column kernel;
  *   2: the row-segment kernel on any grid size.
  * Rows whose leap stride exceeds 31 (next to the poles on fine grids) always

@@ -918,7 +918,7 @@ struct AdjRowArgs {
   const T *yU, *yV, *yPhi;   // ybar
   const T *W, *psi, *Db, *aPhi, *arPcol;
   const T *rU, *rV, *rPhi;   // the array added to: stage sum or the output itself; null: none
-  const int4* items;         // kind << 24 | row j, first own column, own columns, halo; kind 1: all strides 1
+  const int4* items;         // row j, first own column, own columns, halo
   int vec;                   // 1: every row is 16-byte aligned
 };
 

@@ -602,7 +602,7 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
          o_cn = putT(cn.empty() ? std::vector<double>{0} : cn),
          o_cs = putT(cs.empty() ? std::vector<double>{0} : cs);
   size_t o_ds = putT(g->ds), o_r2ds = putT(r2ds), o_hk = putT(hkb), o_Hkk = putT(Hkkb),
-         o_hkr = putT(hk_rds), o_oms = putT(oms), o_rho = putT(rho), o_dsd = putD(g->ds), o_shd = putD(g->sh), o_Ad = putD(g->A),
+         o_hkr = putT(hk_rds), o_oms = putT(oms), o_rho = putT(rho), o_dsd = putD(g->ds), o_Ad = putD(g->A),
          o_Avd = putD(g->Av.empty() ? std::vector<double>{0} : g->Av);
   std::vector<float4> ds3(K);
   for (int k = 0; k < K; ++k) ds3[k] = split3(g->ds[k]);
@@ -652,7 +652,6 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   G.nfU = nfU;
   G.nfV = nfV;
   G.dsd = (const double*)(base + o_dsd);
-  G.shd = (const double*)(base + o_shd);
   G.Ad = (const double*)(base + o_Ad);
   G.Avd = (const double*)(base + o_Avd);
   G.rt0pit = (const T*)(base + o_rt0);
@@ -661,7 +660,6 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
   G.nl = g->beta2 != 0.0 && g->th.delta != 0.0;
   leap1_band(g, &G.l1lo, &G.l1hi);
   G.rady = (T)(1.0 / (kA * g->dth));
-  G.adl = (T)(kA * g->dlam);
   G.ds3 = (const float4*)(base + o_ds3);
   G.lev = (const T*)(base + o_lev);
   G.rowtab = (const T*)(base + o_rtab);
@@ -1894,13 +1892,11 @@ int tendency_static(const agcm_grid* g, char* base, StaticItems& it, bool tables
   G.nl = g->beta2 != 0.0 && g->th.delta != 0.0;
   leap1_band(g, &G.l1lo, &G.l1hi);  // no second stream here: the two launches run in order
   G.dsd = rawlev + 1 * lS;
-  G.shd = rawlev + 0 * lS;
   G.Ad = raw + 3 * rS;
   G.Avd = raw + 5 * rS;
   G.pit = colT;
   G.rt0pit = colT + cS;
   G.rady = (T)(1.0 / (kA * g->dth));
-  G.adl = (T)(kA * g->dlam);
   G.rowtab = rowtab;
   G.rAz = rAz;
   G.ds3 = (const float4*)(base + kOffDs3);

@@ -55,7 +55,6 @@ struct Geom {
   int nfU, nfV;
   const double* dsd;  // dsigma_k in FP64 (column integral of the divergence)
   const float4* ds3;  // dsigma_k as the sum of three FP32 parts x + y + z (K)
-  const double* shd;  // half levels sigma_hat_h in FP64 (K+1)
   const double* Ad;   // A_j in FP64 (J)     (diagnostics)
   const double* Avd;  // Av_j in FP64 (J-1)  (diagnostics)
   // columns (J*I)
@@ -64,7 +63,6 @@ struct Geom {
   int nl;           // 1: the delta kappa Phi/P term is on (beta2 != 0)
   int l1lo, l1hi;   // rows [l1lo, l1hi): interior rows whose strides Mu_j, Mv_j, Mu_{j+1} are all 1
   T rady;           // 1 / (a dth)
-  T adl;            // a dlam
   // work items of the row-segment stage kernel (agcm_row.cuh), longest first:
   // chunks of the rows left to the column body, pairs of rows of equal strides,
   // single rows; kind q's items are items[off[q]] .. items[off[q] + cnt[q]],
