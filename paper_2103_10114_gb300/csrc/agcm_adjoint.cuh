@@ -922,7 +922,8 @@ struct AdjRowArgs {
   int vec;                   // 1: every row is 16-byte aligned
 };
 
-template <class T, bool M1, int NTP = kRowB>
+// VEC: as in row_segment.
+template <class T, bool M1, int VEC = -1, int NTP = kRowB>
 __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs, const AdjRowArgs<T>& a,
                                         const AdjM<T>& m, const AdjOut<T>& o, const int4 item, unsigned char* smem) {
   constexpr int R = AdjRing<T, NTP>::R;
@@ -952,10 +953,11 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
   // quarter of the threads each: a thread four columns of seven rows, next to
   // each other, or tr apart where rows are not aligned.  Rows outside the grid
   // are zeros.
-  const int tr = NTW >> 2, cr = t / tr, cc = (a.vec ? 4 : 1) * (t - cr * tr);
+  const bool al = VEC < 0 ? a.vec != 0 : VEC != 0;
+  const int tr = NTW >> 2, cr = t / tr, cc = (al ? 4 : 1) * (t - cr * tr);
   int c4 = cstart + cc;
   while (c4 >= I) c4 -= I;
-  const unsigned turns = own_columns(cc, a.vec ? 1 : tr, H, own) | (a.vec ? 0u : row_turns(c4, tr, I));
+  const unsigned turns = own_columns(cc, al ? 1 : tr, H, own) | (al ? 0u : row_turns(c4, tr, I));
   const int jr = cr < 3 ? j + cr - 1 : j;
   const bool in = cc < NT, ok3 = in && jr >= 0 && jr < J, okv = in && jr >= 0 && jr < J - 1;
   const bool oks = in && hasS;
@@ -1000,7 +1002,7 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
     }
   };
   auto issue_level = [&](int k, int s) __attribute__((always_inline)) {
-    if (a.vec)
+    if (al)
       issue_form(std::true_type{}, k, s);
     else
       issue_form(std::false_type{}, k, s);
@@ -1263,7 +1265,7 @@ __device__ __forceinline__ void adj_row(const Geom<T>& g, const ColState<T>& cs,
   }
 }
 
-template <class T>
+template <class T, int VEC = -1>
 __global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64)
     k_adj_rows(const __grid_constant__ Geom<T> g, const __grid_constant__ ColState<T> cs,
                const __grid_constant__ AdjRowArgs<T> a, const __grid_constant__ AdjM<T> m,
@@ -1272,9 +1274,9 @@ __global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_R
   pdl_launch();
   const int4 item = a.items[blockIdx.x];
   if ((int)blockIdx.x >= nany)
-    adj_row<T, true>(g, cs, a, m, o, item, smem);
+    adj_row<T, true, VEC>(g, cs, a, m, o, item, smem);
   else
-    adj_row<T, false>(g, cs, a, m, o, item, smem);
+    adj_row<T, false, VEC>(g, cs, a, m, o, item, smem);
 }
 
 // The same in CTAs of 192 threads, two an SM (12 warps, as above): FP32 rows of
@@ -1291,7 +1293,7 @@ __global__ void __launch_bounds__(kAdjWide, 2)
                     const __grid_constant__ AdjRowArgs<T> a, const __grid_constant__ AdjM<T> m,
                     const __grid_constant__ AdjOut<T> o) {
   extern __shared__ __align__(128) unsigned char smem[];
-  adj_row<T, false, kAdjWide>(g, cs, a, m, o, a.items[blockIdx.x], smem);
+  adj_row<T, false, -1, kAdjWide>(g, cs, a, m, o, a.items[blockIdx.x], smem);
 }
 
 // pi-bar = direct psi part + m-bar, with m^u_i = (m_i + m_{i+1})/2 and

@@ -576,9 +576,8 @@ int upload_geom(const agcm_grid* g, void** blob_out, agcm::Geom<T>* geom_out) {
     L[agcm::kLevRho] = rho[k];
   }
   for (int j = 0; j < J; ++j) {
-    const agcm::RowTab t = agcm::row_tab(j, J, kA * g->dlam, kA * g->dth, g->A.data(), g->sv.data(), g->Av.data(),
-                                         g->Mu.data(), [&](int r) { return 2.0 * kOmega * g->c[r]; },
-                                         [&](int r) { return g->cot[r] / kA; });
+    const agcm::RowTab t = agcm::row_tab(j, J, kA * g->dlam, kA * g->dth, 2.0 * kOmega, 1.0 / kA, g->A.data(), g->sv.data(),
+                                         g->Av.data(), g->c.data(), g->cot.data(), g->Mu.data());
     std::copy(t.v, t.v + agcm::kRowTabN, rowtab.begin() + (size_t)j * agcm::kRowTabN);
     const double z = kA * g->dth / g->Mu[j];
     rAz[2 * j] = z / g->A[j];
@@ -802,7 +801,14 @@ int launch_fused(const agcm::Geom<T>& G, const void* const xs[4], const double* 
       agcm::RowArgs<T> ra{(const T*)xs[0], (const T*)xs[1], (const T*)xs[2], (const T*)xs[3], ub, vb,
                           (const T*)xb[0], (const T*)xb[1], (const T*)xb[2], (const T*)xb[3], (T*)out[0],
                           (T*)out[1], (T*)out[2], (T*)out[3], ubo, vbo, ubb, vbb, (T)cdt, vec ? 1 : 0, gap(xs[2], xs[0]), gap(xs[1], xs[0]), MODE == 2 ? gap(xb[1], xb[0]) : 0, 0};
-      auto kern = agcm::k_row_stage<T, MODE, TERMS, decltype(nl)::value>;
+      constexpr bool NL = decltype(nl)::value;
+      auto pick = [&] {
+        if constexpr (sizeof(T) == 4 && TERMS == 3 && MODE != 0)  // a step's stages: a body for either way to copy
+          return vec ? agcm::k_row_stage<T, MODE, TERMS, NL, 1> : agcm::k_row_stage<T, MODE, TERMS, NL, 0>;
+        else
+          return agcm::k_row_stage<T, MODE, TERMS, NL>;
+      };
+      const auto kern = pick();
       CUDA_TRY(allow_shared(kern, smem));
       auto go = [&](int off, int n, cudaStream_t q, bool dependent) -> int {
         agcm::RowArgs<T> rc = ra;
@@ -1661,9 +1667,16 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
   }
   if (s->n_adj_items > 0) {
     const size_t smem = agcm::adj_row_smem<T>(G.K);
-    CUDA_TRY(allow_shared(agcm::k_adj_rows<T>, smem));
+    auto pick = [&] {
+      if constexpr (sizeof(T) == 4)
+        return vec ? agcm::k_adj_rows<T, 1> : agcm::k_adj_rows<T, 0>;
+      else
+        return agcm::k_adj_rows<T>;
+    };
+    const auto kern = pick();
+    CUDA_TRY(allow_shared(kern, smem));
     ra.items = s->adj_items;
-    CUDA_TRY(launch(agcm::k_adj_rows<T>, dim3((unsigned)s->n_adj_items), s->adj_threads, smem, st, s->adj_early, G, cs, ra, m, o,
+    CUDA_TRY(launch(kern, dim3((unsigned)s->n_adj_items), s->adj_threads, smem, st, s->adj_early, G, cs, ra, m, o,
                     s->n_adj_any));
   }
   if (fork) {
@@ -1792,8 +1805,7 @@ __global__ void k_static_geom(int I, int J, int K, const double* raw, const doub
         rowT[10 * rowStride + j] = (T)(0.25 * A[j] / Av[j]);
         rowT[11 * rowStride + j] = (T)(0.25 * A[j + 1] / Av[j]);
       }
-      const agcm::RowTab t = agcm::row_tab(j, J, kA * dlam, kA * dth, A, sv, Av, Mu,
-                                           [&](int r) { return 2.0 * kOmega * c[r]; }, [&](int r) { return cot[r] / kA; });
+      const agcm::RowTab t = agcm::row_tab(j, J, kA * dlam, kA * dth, 2.0 * kOmega, 1.0 / kA, A, sv, Av, c, cot, Mu);
       for (int q = 0; q < agcm::kRowTabN; ++q) rowtab[(size_t)j * agcm::kRowTabN + q] = (T)t.v[q];
       const double z = kA * dth / Mu[j];
       rAz[2 * j] = z / A[j];

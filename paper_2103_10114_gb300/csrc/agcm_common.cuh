@@ -87,15 +87,16 @@ enum { kRtPh, kRtV, kRtYv, kRtYn, kRtAf, kRtAc, kRtRvn, kRtRvs, kRtOwn, kRtYs = 
 struct RowTab {
   double v[kRowTabN];
 };
-// Row j's values; A, sv, Av and f0(j), c(j) = cot(theta_j) / a in FP64; V rows 0 .. J-2.
-template <class F0, class Cot>
-__host__ __device__ inline RowTab row_tab(int j, int J, double adlam, double adth, const double* A, const double* sv,
-                                          const double* Av, const int* Mu, F0 f0, Cot c) {
+// Row j's values from FP64 tables: A and Av, sv = sin(theta^v), c = cos(theta), cot
+// = cot(theta); adlam, adth = a dlam, a dth; om2 = 2 Omega; ra = 1 / a.
+__host__ __device__ inline RowTab row_tab(int j, int J, double adlam, double adth, double om2, double ra, const double* A,
+                                          const double* sv, const double* Av, const double* c, const double* cot,
+                                          const int* Mu) {
   RowTab t{};
   const double z = adth / Mu[j];
   t.v[kRtPh] = 0.5 * z / A[j];
-  t.v[kRtAf] = A[j] * f0(j) / z;
-  t.v[kRtAc] = A[j] * c(j) / z;
+  t.v[kRtAf] = A[j] * (om2 * c[j]) / z;
+  t.v[kRtAc] = A[j] * (cot[j] * ra) / z;
   if (j > 0) t.v[kRtYn] = adlam * sv[j - 1] / z;
   if (j < J - 1) {
     t.v[kRtV] = 0.5 * z / Av[j];
@@ -103,8 +104,8 @@ __host__ __device__ inline RowTab row_tab(int j, int J, double adlam, double adt
     t.v[kRtRvn] = Av[j] / A[j];
     t.v[kRtRvs] = Av[j] / A[j + 1];
     t.v[kRtZs] = (double)Mu[j] / Mu[j + 1];
-    t.v[kRtAfs] = A[j + 1] * f0(j + 1) / z;
-    t.v[kRtAcs] = A[j + 1] * c(j + 1) / z;
+    t.v[kRtAfs] = A[j + 1] * (om2 * c[j + 1]) / z;
+    t.v[kRtAcs] = A[j + 1] * (cot[j + 1] * ra) / z;
   }
   if (j < J - 2) t.v[kRtYs] = adlam * sv[j + 1] / z;
   return t;
