@@ -100,12 +100,12 @@ void dev_free(void* p) {
 
 // A table from host memory into fresh device memory, there when this returns.
 // cudaMemcpy from pageable memory may return while the last of it is on its
-// way, and nothing orders a launch on a non-blocking stream behind it; and
-// memory from a caching allocator may still be written by what its last owner
-// queued on a stream of its own.
+// way, and nothing orders a launch on a non-blocking stream behind it.  Memory
+// from a caching allocator may still be written by what its last owner queued
+// on a stream of its own: where that can be, the caller waits first (not for the
+// device in a call that may run while another thread captures a graph).
 bool upload(void* d, const void* h, size_t bytes) {
-  return cudaDeviceSynchronize() == cudaSuccess && cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice) == cudaSuccess &&
-         cudaStreamSynchronize(nullptr) == cudaSuccess;
+  return cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice) == cudaSuccess && cudaStreamSynchronize(nullptr) == cudaSuccess;
 }
 
 // Lets `kern` be launched with that much dynamic shared memory on the current device.
@@ -1188,6 +1188,7 @@ int agcm_state_create(const agcm_grid_t* g, int precision, int nmembers, agcm_st
   *out = nullptr;
   if (precision != AGCM_FP64 && precision != AGCM_FP32) return fail(AGCM_EINVAL, "precision must be AGCM_FP64 or AGCM_FP32");
   if (nmembers != 1) return fail(AGCM_EINVAL, "nmembers must be 1; ensembles use agcm_ensemble_*");
+  if (cudaDeviceSynchronize() != cudaSuccess) cudaGetLastError();  // the memory's last owners are done with it (upload)
   int rc = ensure_geom(g, AGCM_FP64);
   if (!rc && precision == AGCM_FP32) rc = ensure_geom(g, AGCM_FP32);
   if (rc) return rc;
@@ -1221,7 +1222,6 @@ int agcm_state_create(const agcm_grid_t* g, int precision, int nmembers, agcm_st
     delete s;
     return fail(AGCM_ENOMEM, "device allocation for a %zu x %zu x %zu state failed", I, J, K);
   }
-  cudaDeviceSynchronize();  // as in upload
   for (int c = 0; c < 3; ++c)
     for (int f = 0; f < 4; ++f) {
       size_t n = f == 1 ? std::max<size_t>(s->nv, 1) : (f == 3 ? s->n2 : s->n3);
@@ -1441,8 +1441,13 @@ const char* agcm_kernel_name(int id) { return (id >= 0 && id < KID_COUNT) ? kKer
 // ------------------------------------------------------------------ adjoint
 namespace {
 
-int ensure_adj(agcm_state* s) {
+int ensure_adj(agcm_state* s, cudaStream_t st) {
   if (s->adj_ready) return AGCM_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+    cudaStreamSynchronize(st);  // as in upload
+  else
+    cudaGetLastError();
   const size_t e = s->esz, n3 = s->n3 * e, nv = std::max<size_t>(s->nv, 1) * e, n2 = s->n2 * e;
   const size_t nw = (size_t)(s->grid->K + 1) * s->grid->J * s->grid->I * e;
   bool ok = true;
@@ -1697,7 +1702,7 @@ int vjp(agcm_state* s, int stage, void* const x[4], const void* const y[4], void
 template <class T>
 int adjoint_step(agcm_state* s, const void* const lam_in[4], void* const lam_out[4], double dt, cudaStream_t st) {
   int rc;
-  if ((rc = ensure_adj(s))) return rc;
+  if ((rc = ensure_adj(s, st))) return rc;
   if ((rc = ensure_bar<T>(s, st))) return rc;
   if ((rc = fused_stage<T, 1>(s, 0, s->x[1], 1, 0.5 * dt, st))) return rc;
   if ((rc = fused_stage<T, 2>(s, 1, s->x[2], 2, 0.5 * dt, st))) return rc;

@@ -68,3 +68,46 @@ def test_first_persistent_step_on_a_side_stream(cuda_ok):
         for s in states:
             s.close()
     assert all(torch.equal(a[f], b[f]) for a, b in zip(*outs) for f in agcm.FIELDS)
+
+
+@pytest.mark.gpu
+def test_first_adjoint_beside_a_capture(cuda_ok):
+    """The workspace of a first reverse step is made while another thread
+    captures a graph on a stream of its own: neither disturbs the other."""
+    import threading
+
+    import torch
+
+    agcm.build()
+    I, J, K = 96, 48, 4
+    st = inputs.random_state(I, J, K, seed=1)
+    lam = inputs.random_direction(I, J, K, seed=2)
+    a, b, c = (agcm.State(agcm.Grid(I, J, K, phis=st["phis"]), agcm.AGCM_FP32) for _ in range(3))
+    side = torch.cuda.Stream()
+    lam = {f: torch.as_tensor(lam[f], dtype=torch.float32, device="cuda") for f in agcm.FIELDS}
+    for s in (a, b, c):
+        s.load(st)
+    a.step(1, 1.0)
+    out = b.empty()
+    torch.cuda.synchronize()
+    errors = []
+
+    def other():
+        try:
+            args = [(agcm._vp * 4)(*[t[f].data_ptr() for f in agcm.FIELDS]) for t in (lam, out)]
+            agcm.check(agcm.lib().agcm_step_adjoint(b.handle, *args, 1.0, agcm._stream_ptr(side)))
+            side.synchronize()
+        except Exception as e:  # reported by the test's own thread
+            errors.append(e)
+
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="thread_local"):
+        a.step(1, 1.0)
+        t = threading.Thread(target=other)
+        t.start()
+        t.join()
+    assert not errors, errors
+    g.replay()
+    want = c.step_adjoint(lam, 1.0)
+    torch.cuda.synchronize()
+    assert all(torch.equal(out[f], want[f]) for f in agcm.FIELDS)
