@@ -261,20 +261,20 @@ __device__ __forceinline__ void col_suffix(const ColCtx<T>& c, const AdjCol<T>& 
 // ring of shared-memory slots, two 16-byte copies a thread, on the way down;
 // that walk forms D, the gathered adjoints of psi and W, the prefix sums and
 // with them the adjoint of Phi, and keeps D and the adjoint of W (kKeep 1: that
-// in Dbar's place); the walk up forms W, psi and Dbar from the suffix sums, reading Phi and ybar_Phi once
-// more (from L2).  Rows whose divergence pair lies outside the halo (kind 1)
-// read the pair from global memory a level ahead.
-// Bound by load latency (16 warps an SM, 95 registers) in FP32 and by the FP64
+// in Dbar's place); the walk up forms W, psi and Dbar from the suffix sums,
+// reading Phi and ybar_Phi once more (from L2).  Rows whose divergence pair lies
+// outside the halo (kind 1) read the pair from global memory a level ahead.
+// Bound by load latency (16 warps an SM, 106 registers) in FP32 and by the FP64
 // pipe in FP64.  Per launch of the reverse pass, before (32 columns and four
 // groups of eight levels per block, stencil through L1) and now: 720 x 360 x 30
 // FP32 108 -> 82 us (7.8 M points, 40 B a point at the copy rate 46 us), FP64
 // 1503 -> 1108; 256 x 128 x 30 FP64 201 -> 193, FP32 20 either way; 128 x 64 x
 // 16 FP32 13.5 -> 11.1, FP64 39 -> 48 (one warp a scheduler: its levels are one
-// chain of FP64 issue); 128 x 64 x 120 FP32 71 -> 42, FP64 368 -> 313.  Ring of two slots 107, three 90 (five blocks 82, but
-// 256 x 128 and 405 x 203 4 to 7 % slower); groups of six levels 83.  FP64
-// keeps the adjoint of W in Dbar's place instead of shared memory: 80 KB a
-// block would hold two blocks (1209); so does FP32 where three blocks an SM
-// would not hold both.
+// chain of FP64 issue); 128 x 64 x 120 FP32 71 -> 42, FP64 368 -> 313.  Ring of
+// two slots 107, three 90 (five blocks 82, but 256 x 128 and 405 x 203 4 to 7 %
+// slower); groups of six levels 83.  FP64 keeps the adjoint of W in Dbar's place
+// instead of shared memory: 80 KB a block would hold two blocks (1209); so does
+// FP32 where three blocks an SM would not hold both.
 constexpr int kColRaw = 8;  // U, yU, V j-1, V j, yV j-1, yV j, Phi, yPhi
 constexpr int kColPad = 64;  // before the ring: a halo column's pair reaches at most H <= 32 to the west of it
 constexpr int kColB = 8;  // levels of a partial sum
@@ -882,9 +882,9 @@ __global__ void __launch_bounds__(256) k_adj_fold(Geom<T> g, const int* __restri
 // 240.  M1: all strides of the row are 1, which makes half of the partner
 // reads the own or an already read value.
 //
-// Bound by shared-memory reads (their pipe is busy 62 % of the cycles) and the
-// latency left at 12 warps an SM: 187 us a launch at 720x360x30 FP32 (ncu,
-// cold caches), 377 thread instructions a point, against 250 us and 810 for
+// Bound by shared-memory reads (their pipe is busy half of the cycles) and the
+// latency left at 12 warps an SM: 181 us a launch at 720x360x30 FP32 (ncu,
+// cold caches), 396 instructions a point, against 250 us and 810 for
 // 256-thread CTAs that loaded their rows into registers a level ahead; 200 at
 // two ring slots, 215 with four CTAs an SM at 128 registers.  FP64: 3.0 ms.
 enum AdjRowArr {

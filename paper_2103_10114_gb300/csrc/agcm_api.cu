@@ -1997,6 +1997,7 @@ struct agcm_ensemble {
   std::vector<int4> host_items;  // the row items of every member, member << 8 in w
   void* d_items = nullptr;
   int nitems_rows = 0;
+  bool aligned = false;          // every row of every member is 16-byte aligned
   size_t rows_smem = 0;          // dynamic shared memory of that launch
   std::vector<double> last_dt;
   Profiler prof;
@@ -2009,6 +2010,7 @@ void fill_desc(agcm_ensemble* e) {
   e->host_desc.assign(e->members.size() * sizeof(agcm::EnsMember<T>), 0);
   auto* d = reinterpret_cast<agcm::EnsMember<T>*>(e->host_desc.data());
   int begin = 0;
+  e->aligned = true;
   for (size_t m = 0; m < e->members.size(); ++m) {
     agcm_state* s = e->members[m];
     d[m].g = geom_of<T>(s);
@@ -2021,6 +2023,7 @@ void fill_desc(agcm_ensemble* e) {
     for (int c = 0; c < 3; ++c)
       for (int f = 0; f < 3; ++f)
         if ((uintptr_t)s->x[c][f] & 15) d[m].vec = 0;
+    e->aligned = e->aligned && d[m].vec;
     d[m].nbx = (s->grid->I + 31) / 32;
     d[m].item_begin = begin;
     d[m].dt = (T)0;
@@ -2071,7 +2074,13 @@ int ensemble_step(agcm_ensemble* e, int nsteps, const double* dt, cudaStream_t s
   CUDA_TRY(cudaDeviceGetAttribute(&clock_khz, cudaDevAttrClockRate, dev));
   const int threads = 32 * e->warps_per_block;
   if (e->warps_per_block == 8) {  // the row-segment persistent launch
-    auto kr = agcm::k_ensemble_rows<T>;
+    auto pick = [&] {  // a body for members whose rows are all aligned (row_segment's VEC), one for any
+      if constexpr (sizeof(T) == 4)
+        return e->aligned ? agcm::k_ensemble_rows<T, 1> : agcm::k_ensemble_rows<T>;
+      else
+        return agcm::k_ensemble_rows<T>;
+    };
+    const auto kr = pick();
     if (e->rows_smem > kMaxShared) return fail(AGCM_EINVAL, "ensemble member with too many levels for the row launch");
     CUDA_TRY(allow_shared(kr, e->rows_smem));
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kr, agcm::kRowB, e->rows_smem));

@@ -87,7 +87,7 @@ __device__ __forceinline__ RowSums<float> diag_row(const float* __restrict__ x, 
 }
 
 // A warp takes rows in a fixed order (fields U, Phi, V, then pi), so the sums
-// do not depend on the order in which warps run.  199 us at 1440x720x30 FP32.
+// do not depend on the order in which warps run.  197 us at 1440x720x30 FP32.
 template <class T>
 __global__ void __launch_bounds__(kDiagThreads) k_diag(Geom<double> g, const T* __restrict__ U,
                                                        const T* __restrict__ V, const T* __restrict__ Phi,

@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(32, sizeof(T) == 4 ? AGCM_ENS_MINB : 8)
 // row items with the member << 8 in w.  Every stage uses x_n as its base (stage 1 reads it as
 // input and base), the three stages of a step as in agcm_step; a bounded grid
 // barrier separates them.
-template <class T>
+template <class T, int VEC = -1>
 __global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_ROW_MINB64)
     k_ensemble_rows(const EnsMember<T>* __restrict__ mem, const int4* __restrict__ items, int nitems, int nsteps,
                     EnsSync* sy, unsigned expected_blocks, long long limit) {
@@ -194,9 +194,9 @@ __global__ void __launch_bounds__(kRowB, sizeof(T) == 4 ? AGCM_ROW_MINB : AGCM_R
         }
         const int kind = item_kind(w);
         if (kind == kRowPair) {
-          row_segment<T, 2, 3, false, 2, true, false>(e.g, ra, w, smem);
+          row_segment<T, 2, 3, false, 2, true, false, VEC>(e.g, ra, w, smem);
         } else if (kind == kRowAny) {
-          row_segment<T, 2, 3, false, 1, false, false>(e.g, ra, w, smem);
+          row_segment<T, 2, 3, false, 1, false, false, VEC>(e.g, ra, w, smem);
         } else {
           polar_columns<T, 2, 3, false>(e.g, ra, w, smem);
         }
