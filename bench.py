@@ -43,7 +43,7 @@ BYTES_PER_POINT_STEP = {4: 96, 8: 192}  # 24 words: stages read/write 6 + 9 + 9 
 NCU_TRAFFIC = {
     # kernel bracket name: (sha1 of the stage-kernel sources at capture time,
     # DRAM bytes per stage summed over the stage's launches)
-    "k_fused_stage": ("c1c333369dcd630f2d9209d55613c2a8eb1a78bd", 1051927000),
+    "k_fused_stage": ("3644bc1f69afbb779e21909ab8ace1349b5ba0d6", 1051477000),
 }
 
 # Instruction counters of the dominant kernel (ncu per-opcode counts, this
@@ -52,14 +52,14 @@ NCU_TRAFFIC = {
 # point and stage (fadd + fmul + 2 ffma), thread instructions per point, warp
 # instructions issued per point.
 NCU_OPS = {
-    "k_fused_stage": ("c1c333369dcd630f2d9209d55613c2a8eb1a78bd", 130.4, 204.9, 6.444),
+    "k_fused_stage": ("3644bc1f69afbb779e21909ab8ace1349b5ba0d6", 132.5, 204.5, 6.408),
 }
 
 
 # DRAM traffic of one FP32 adjoint step at 720x360x30 (all its launches: the
 # forward recompute of the two stage states and three adjoint products), from
 # an ncu capture, valid while the kernel sources are the captured ones.
-NCU_ADJ = ("0d16c78c5b45f51e362fdecf29f62457a668cc9b", 2842200064)
+NCU_ADJ = ("5d8a58b9639d6e3a7ed971de0487b170e7b9ce8a", 2839441664)
 
 
 def kernel_source_hash(names=("agcm_row.cuh", "agcm_fused.cuh", "agcm_common.cuh")):
